@@ -43,19 +43,19 @@ struct BlockDev {
   int cav;               // cavity this block belongs to
   int tiles_x, tiles_y, tiles_z;
   int tile_begin;        // first partial slot (k_step tile) of this block
-  // z chunking of the step kernels: chunks 0 .. tiles_zc-1 of KC planes cover
+  // z chunking of the step kernels: chunks 0 .. tiles_zc-1 of kc planes cover
   // planes 1 .. zsplit, the other tiles_z - tiles_zc chunks split planes
-  // zsplit+1 .. nz into fine chunks (kFineKC planes in the FP64 form,
-  // kFineKC32 in the FP32 form, whose KC = zsplit / tiles_zc is set at run
-  // time).  Scheduling index c runs over every block's
-  // coarse tiles first (coarse_begin + local) and the fine ones last
-  // (ncoarse + fine_begin + local): the persistent FP64 grid's counter and
-  // the FP32 grids' block order both end on short tiles.  Partial slots stay
-  // block-major (tile_begin + local tile index), so a cavity's are contiguous.
+  // zsplit+1 .. nz into chunks of kf planes.  Scheduling index c runs over
+  // every block's coarse tiles first (coarse_begin + local) and the fine ones
+  // last (ncoarse + fine_begin + local): the persistent FP64 grid's counter
+  // and the FP32 grids' block order both end on short tiles.  Partial slots
+  // stay block-major (tile_begin + local tile index), so a cavity's are
+  // contiguous.
   int tiles_zc, zsplit, coarse_begin, fine_begin;
+  int kc, kf;
   void *base[2];         // buffer sets (field f at base + f * fstride)
 };
-constexpr int kFineKC = 2, kFineKC32 = 8;
+constexpr int kFineKC32 = 8;  // kf of the FP32 form
 
 struct CavConst {
   double h[3], ih[3], ih2[3], ihh[3];
@@ -252,24 +252,58 @@ __device__ __forceinline__ double warp_max(double v) {
 }
 
 // ---------------------------------------------------------------------------
-// Square root of a positive, normal, finite FP64 value by Newton's method on
-// s^2 - q = 0 with a fixed slope: the seed y ~ 1/sqrt(q) comes from the PTX
-// instruction rsqrt.approx.ftz.f64 (measured relative error below 1e-6),
-// s_0 = q y, then twice s <- s + (q - s^2) y / 2.  The relative error of s
-// after a step is about 1.5 e^2 (e the seed's), so the second step lands below
-// the FP64 rounding: the result is within one unit in the last place of the
-// correctly rounded root (cavity_check_sqrt measures this against CUDA's sqrt).
-// It takes about 30% less FP64-pipe time than the library sqrt on GB300.
-// Arguments below the normal range or infinite give NaN (the seed is infinite
-// or zero): the rates only take it of V_d^2 + 4 beta^2 >= 4 kappa u_ref^2,
-// which the parameter check keeps normal.
+// Square root of a positive, normal, finite FP64 value with one operation on
+// the FP64 pipe.  GB300 issues an FP64 warp instruction every 16 cycles an SM
+// (two lanes a clock), FP32 and integer ones up to four a cycle, and the FP64
+// step leaves 90% of the issue slots unused, so everything but the exact
+// residual runs beside it.  With q = 4^k m, m in [1, 4):
+//   y ~ 1/sqrt(m) (rsqrt.approx.ftz.f32), s_0 = sh + sl by one Newton step on
+//   the FP32 pair of m's leading 46 bits: relative error below 2^-43;
+//   r = m - s_0^2, exact to its last bit in FP64 (one fused multiply-add);
+//   s = s_0 + r y / 2, the correction (below 2^9 units in the last place)
+//   formed in FP32 and added to s_0's significand as an integer.
+// The result is within one unit in the last place of the correctly rounded
+// root (cavity_check_sqrt measures this against CUDA's sqrt; the clamps keep
+// s_0 in [1, 2], where a unit of its last place is 2^-52).  Six FP64
+// operations (an FP64 reciprocal-square-root seed and two Newton steps) gave
+// the same accuracy.  Arguments that are NaN or infinite give a finite value:
+// the rates reach NaN or infinity through beta^2 and the weights.
 __device__ __forceinline__ double sqrt_newton(double q) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(q));
-  const double hy = 0.5 * y;
-  double s = q * y;
-  s = fma(fma(-s, s, q), hy, s);
-  return fma(fma(-s, s, q), hy, s);
+  const int hi = __double2hiint(q);
+  const unsigned lo = (unsigned)__double2loint(q);
+  const int odd = ~(hi >> 20) & 1;  // the unbiased exponent is odd
+  const int mhi = (hi & 0xfffff) | ((1023 + odd) << 20);
+  const double m = __hiloint2double(mhi, (int)lo);
+  const float qh = __int_as_float((int)(__funnelshift_l(lo, (unsigned)hi, 3) & 0x7fffffu) | ((127 + odd) << 23));
+  // the significand's next 23 bits, as an integer in FP32
+  const float ql = __fsub_rn(__uint_as_float(0x4b000000u | ((lo & 0x1fffffffu) >> 6)), 8388608.f);
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(qh));
+  const float hy = 0.5f * y;
+  const float sh = fminf(fmaxf(__fmul_rn(qh, y), 1.f), 1.99999988f);
+  const float res = __fmaf_rn(ql, __int_as_float((127 - 46 + odd) << 23), __fmaf_rn(-sh, sh, qh));
+  const int n = __float2int_rn(__fmul_rn(__fmul_rn(res, hy), 0x1p46f));
+  long long s0 = ((long long)__float_as_int(sh) << 29) + (896ll << 52) + ((long long)n << 6);
+  s0 = max(min(s0, 0x4000000000000000ll), 0x3ff0000000000000ll);
+  const double s0d = __longlong_as_double(s0);
+  const double r = fma(-s0d, s0d, m);
+  const int rhi = __double2hiint(r);
+  // |r| in [2^-104, 2^-20] or 0 (which the maximum maps to 2^-126): FP32 bits, truncated
+  const unsigned ra = max((unsigned)rhi & 0x7fffffffu, 897u << 20) - (896u << 20);
+  const float rf = __uint_as_float(__funnelshift_l((unsigned)__double2loint(r), ra, 3) | ((unsigned)rhi & 0x80000000u));
+  const int n2 = __float2int_rn(__fmul_rn(rf, __fmul_rn(hy, 0x1p52f)));
+  return __longlong_as_double(s0 + n2 + ((long long)((hi - mhi) >> 1) << 32));
+}
+
+// 4 x for a positive normal x (the exponent raised by two; infinite or NaN
+// past FP64's range), and the larger of two non-negative values (their bit
+// patterns order like the values, a NaN above all): integer operations
+// instead of FP64-pipe slots.
+__device__ __forceinline__ double times4(double x) {
+  return __hiloint2double(min(__double2hiint(x) + (2 << 20), 0x7ff00000), __double2loint(x));
+}
+__device__ __forceinline__ double max_nonneg(double a, double b) {
+  return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
 }
 
 // ---------------------------------------------------------------------------
@@ -290,8 +324,8 @@ struct NodeF64 {
 
 __device__ __forceinline__ void rates_f64(const CavConst &C, const NodeF64 &n, double r[5]) {
   const double u0 = n.u[0], v0 = n.v[0], w0 = n.w[0];
-  const double b2 = fmax(fma(u0, u0, fma(v0, v0, w0 * w0)), C.b2min);
-  const double f4 = 4.0 * b2;
+  const double b2 = max_nonneg(fma(u0, u0, fma(v0, v0, w0 * w0)), C.b2min);
+  const double f4 = times4(b2);
   const double ex = (fabs(u0) + sqrt_newton(fma(u0, u0, f4))) * C.dsc[0];
   const double ey = (fabs(v0) + sqrt_newton(fma(v0, v0, f4))) * C.dsc[1];
   const double ez = (fabs(w0) + sqrt_newton(fma(w0, w0, f4))) * C.dsc[2];
@@ -326,8 +360,8 @@ __device__ __forceinline__ void rates_f64(const CavConst &C, const NodeF64 &n, d
 // roots within one unit in the last place (sqrt_newton), so dt is the
 // correctly rounded formula's to a few ulp
 __device__ __forceinline__ double spectral_f64(const CavConst &C, double u, double v, double w) {
-  const double b2 = fmax(u * u + v * v + w * w, C.b2min);
-  const double f4 = 4.0 * b2;
+  const double b2 = max_nonneg(u * u + v * v + w * w, C.b2min);
+  const double f4 = times4(b2);
   const double sx = fabs(u) + sqrt_newton(u * u + f4);
   const double sy = fabs(v) + sqrt_newton(v * v + f4);
   const double sz = fabs(w) + sqrt_newton(w * w + f4);
@@ -416,9 +450,18 @@ __device__ __forceinline__ int float_key(float f) {
 __device__ __forceinline__ float key_float(int k) { return __int_as_float(k >= 0 ? k : k ^ 0x7fffffff); }
 
 // ---------------------------------------------------------------------------
-// k_step, FP64: one thread per (i, j) column of a TX x TY tile, sweeping a
-// chunk of KC planes in k.  The z-neighbours live in register queues
-// (5 deep for p, 3 deep for u, v, w, T); x/y neighbours come through L1.
+// k_step, FP64: a tile is NT consecutive nodes of a block's (x, y) plane, x
+// fastest (node e = (i - 1) + nx (j - 1)), over a chunk of planes; one thread
+// per (i, j) column sweeps the chunk in k.  The z-neighbours live in register
+// queues (5 deep for p, 3 deep for u, v, w, T); x/y neighbours come through L1.
+//
+// Why these tiles: the FP64 pipe (two lanes a clock per SM) takes a warp
+// instruction's 16 cycles whether its lanes hold a node or not, and one warp a
+// scheduler already keeps it 70% busy.  So what counts is that every lane of
+// every warp holds a node -- consecutive nodes do, whatever nx is, where a
+// 32-wide tile leaves 24% of the lanes of a 97-wide and 38% of a 40-wide block
+// idle -- and that the SMs get equal numbers of planes (the chunk depth:
+// assign_tiles in cavity_capi.cu).
 
 struct StepArgs {
   const BlockDev *blocks;
@@ -460,13 +503,11 @@ __device__ __forceinline__ int find_block(const BlockDev *blocks, int nblocks, i
 }
 
 // The tile of scheduling index c: its block, x/y tile, plane range and
-// partial slot (coarse chunks of KC planes, fine chunks of KF planes, as
-// described at BlockDev).
+// partial slot (coarse and fine chunks as described at BlockDev).
 struct TileRef {
   int b, tx, ty, k0, k1, slot;
 };
 
-template <int KC, int KF>
 __device__ __forceinline__ TileRef tile_ref(const BlockDev *blocks, int nblocks, int ncoarse, int c) {
   const bool coarse = c < ncoarse;
   const int u = coarse ? c : c - ncoarse;
@@ -485,16 +526,11 @@ __device__ __forceinline__ TileRef tile_ref(const BlockDev *blocks, int nblocks,
   T.tx = l % B.tiles_x;
   T.ty = (l / B.tiles_x) % B.tiles_y;
   const int zl = l / (B.tiles_x * B.tiles_y);
-  T.k0 = coarse ? zl * KC + 1 : B.zsplit + zl * KF + 1;
-  T.k1 = coarse ? min(T.k0 + KC - 1, B.zsplit) : min(T.k0 + KF - 1, B.nz);
+  T.k0 = coarse ? zl * B.kc + 1 : B.zsplit + zl * B.kf + 1;
+  T.k1 = coarse ? min(T.k0 + B.kc - 1, B.zsplit) : min(T.k0 + B.kf - 1, B.nz);
   const int tz = coarse ? zl : B.tiles_zc + zl;
   T.slot = B.tile_begin + T.tx + B.tiles_x * (T.ty + B.tiles_y * tz);
   return T;
-}
-
-template <int KC>
-__device__ __forceinline__ TileRef f64_tile(const StepArgs &a, int c) {
-  return tile_ref<KC, kFineKC>(a.blocks, a.nblocks, a.ncoarse, c);
 }
 
 // wfloor: a warp-uniform FP32 value of D = S - S0 at or below the one of an
@@ -507,10 +543,9 @@ __device__ __forceinline__ TileRef f64_tile(const StepArgs &a, int c) {
 // hence dt -- is exactly the FP64 one.  Carried across the warp's tiles of
 // one cavity (`fcav`: the cavity it belongs to; a tile of another cavity,
 // in a batch, starts again from -inf).
-template <int TX, int TY, int KC>
+template <int NT>
 __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float &wfloor, int &fcav) {
-  constexpr int NT = TX * TY;
-  const TileRef tile = f64_tile<KC>(a, cta);
+  const TileRef tile = tile_ref(a.blocks, a.nblocks, a.ncoarse, cta);
   const BlockDev &B = a.blocks[tile.b];
   const CavConst &C = a.cc[B.cav];
   if (B.cav != fcav) {
@@ -525,11 +560,11 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
     if (u != 0u) wfloor = fmaxf(wfloor, key_float((int)(u ^ 0x80000000u)));
   }
   float published = wfloor;
-  const int i = tile.tx * TX + threadIdx.x + 1;
-  const int j = tile.ty * TY + threadIdx.y + 1;
+  const int tid = threadIdx.x, e = tile.tx * NT + tid;
+  const int j = e / B.nx + 1, i = e - (j - 1) * B.nx + 1;
   const int k0 = tile.k0;
   const int k1 = tile.k1;
-  const bool active = (i <= B.nx) && (j <= B.ny);
+  const bool active = j <= B.ny;
   const double dt = a.cs[B.cav].dt;
   const double cshift = a.cs[B.cav].c;
 
@@ -600,46 +635,63 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
       uq0 = uq1; uq1 = uq2; vq0 = vq1; vq1 = vq2; wq0 = wq1; wq1 = wq2; Tq0 = Tq1; Tq1 = Tq2;
     }
   }
-  // deterministic CTA reduction of the six partials
-  __shared__ double red[NT / 32][6];
-  const int tid = threadIdx.y * TX + threadIdx.x;
+  // CTA reduction of the six partials, in a fixed order and with few FP64
+  // warp instructions (25 warp adds for the five sums of 128 threads, where a
+  // shuffle tree in every warp takes 100): field f by the 16 threads 16 f ..
+  // 16 f + 15, each NT / 16 values, then a butterfly; the maximum (of positive
+  // values) on the bit patterns.
+  __shared__ double red[5][NT];
+  __shared__ unsigned long long redm[NT / 32];
   const int lane = tid & 31, wid = tid >> 5;
-  s0 = warp_sum(s0); s1 = warp_sum(s1); s2 = warp_sum(s2); s3 = warp_sum(s3); s4 = warp_sum(s4);
-  smax = warp_max(smax);
-  if (lane == 0) {
-    red[wid][0] = s0; red[wid][1] = s1; red[wid][2] = s2; red[wid][3] = s3; red[wid][4] = s4; red[wid][5] = smax;
+  red[0][tid] = s0; red[1][tid] = s1; red[2][tid] = s2; red[3][tid] = s3; red[4][tid] = s4;
+  {
+    const unsigned mh = (unsigned)__double2hiint(smax), ml = (unsigned)__double2loint(smax);
+    const unsigned wh = __reduce_max_sync(0xffffffffu, mh);
+    const unsigned wl = __reduce_max_sync(0xffffffffu, mh == wh ? ml : 0u);
+    if (lane == 0) redm[wid] = ((unsigned long long)wh << 32) | wl;
   }
   __syncthreads();
-  if (tid < 6) {
-    double acc = red[0][tid];
-    for (int q = 1; q < NT / 32; ++q) acc = (tid == 5) ? fmax(acc, red[q][tid]) : acc + red[q][tid];
-    a.partials[(long long)tile.slot * kPartStride + tid] = acc;
+  if (wid < 3) {
+    const int f = tid >> 4, s = tid & 15;
+    double v = 0.0;
+    if (f < 5) {
+      const double *p = &red[f][s];
+#pragma unroll
+      for (int q = 0; q < NT / 16; ++q) v = q == 0 ? p[0] : v + p[16 * q];
+    }
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (f == 5) {
+      unsigned long long m = redm[0];
+      for (int q = 1; q < NT / 32; ++q) m = redm[q] > m ? redm[q] : m;
+      v = __longlong_as_double((long long)m);
+    }
+    if (s == 0) a.partials[(long long)tile.slot * kPartStride + f] = v;
   }
 }
 
 // Persistent form: as many CTAs as fit on the GPU at once take tiles in
 // order from a counter, so the last round is short (one CTA per tile left a
 // partial wave of up to a third of the step on 152 SMs); the counter hands
-// out every block's 8-plane tiles before the 2-plane tail tiles.  Partials
-// stay indexed by tile slot: the reductions do not depend on which CTA took
-// a tile.
-template <int TX, int TY, int KC>
-__global__ void __launch_bounds__(TX *TY) k_step_f64(StepArgs a) {
+// out every block's coarse tiles before the fine tail tiles, and the next
+// tile is fetched while the current one is computed.  Partials stay indexed by
+// tile slot: the reductions do not depend on which CTA took a tile.
+template <int NT>
+__global__ void __launch_bounds__(NT) k_step_f64(StepArgs a) {
   float wfloor = -INFINITY;
   int fcav = -1;
   if (!a.tile_counter) {
-    step_tile_f64<TX, TY, KC>(a, blockIdx.x, wfloor, fcav);
+    step_tile_f64<NT>(a, blockIdx.x, wfloor, fcav);
     return;
   }
-  __shared__ int s_tile;
-  const int tid = threadIdx.y * TX + threadIdx.x;
-  for (;;) {
-    if (tid == 0) s_tile = (int)atomicAdd(a.tile_counter, 1u);
+  // the first tile of each CTA is its own index; the counter starts at the grid's size
+  __shared__ int s_tile[2];
+  int tile = blockIdx.x;
+  for (int n = 0; tile < a.ntiles; n ^= 1) {
+    if (threadIdx.x == 0) s_tile[n] = (int)(gridDim.x + atomicAdd(a.tile_counter, 1u));
+    step_tile_f64<NT>(a, tile, wfloor, fcav);
     __syncthreads();
-    const int tile = s_tile;
-    if (tile >= a.ntiles) break;
-    step_tile_f64<TX, TY, KC>(a, tile, wfloor, fcav);
-    __syncthreads();
+    tile = s_tile[n];
   }
 }
 

@@ -215,37 +215,6 @@ __device__ __forceinline__ void wall_temperature(float h1, float l1, float h2, f
   pair_add(h1, l1, vmul(d, 1.f / 3.f), hw, lw);
 }
 
-// Tile of FP32 scheduling index c: coarse chunks of every block first, then
-// the fine 8-plane chunks of each block's last planes (they shorten the
-// grid's last wave), x tiles fastest, then y, then z.  The coarse chunk depth
-// is zsplit / tiles_zc (a run-time parameter of the tiling).  The partial slot
-// stays block-major (tile_begin + tx + tiles_x (ty + tiles_y tz)).
-__device__ __forceinline__ TileRef f32_tile_ref(const BlockDev *blocks, int nblocks, int ncoarse, int c) {
-  const bool coarse = c < ncoarse;
-  const int u = coarse ? c : c - ncoarse;
-  // the last block whose first tile of this class is at or before u (blocks
-  // without tiles of the class share their successor's start and are passed)
-  int lo = 0, hi = nblocks - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    const int begin = coarse ? blocks[mid].coarse_begin : blocks[mid].fine_begin;
-    if (begin <= u) lo = mid; else hi = mid - 1;
-  }
-  const BlockDev &B = blocks[lo];
-  const int l = u - (coarse ? B.coarse_begin : B.fine_begin);
-  const int kc = B.zsplit / B.tiles_zc;
-  TileRef T;
-  T.b = lo;
-  T.tx = l % B.tiles_x;
-  T.ty = (l / B.tiles_x) % B.tiles_y;
-  const int zl = l / (B.tiles_x * B.tiles_y);
-  T.k0 = coarse ? zl * kc + 1 : B.zsplit + zl * kFineKC32 + 1;
-  T.k1 = coarse ? min(T.k0 + kc - 1, B.zsplit) : min(T.k0 + kFineKC32 - 1, B.nz);
-  const int tz = coarse ? zl : B.tiles_zc + zl;
-  T.slot = B.tile_begin + T.tx + B.tiles_x * (T.ty + B.tiles_y * tz);
-  return T;
-}
-
 // Tile of one CTA, its partial slot and the walls that fall inside its
 // boxes.  Pressure box: nodes i0-4 .. i0+35, j0-2 .. j0+TY+1; other box:
 // nodes i0-4 .. i0+35, j0-1 .. j0+TY; both over planes k0-2 .. k1+2 (plane
@@ -258,7 +227,7 @@ struct F32Tile {
 template <int TY>
 __device__ __forceinline__ F32Tile f32_tile(const StepF32Args &a, int cta) {
   F32Tile T;
-  const TileRef R = f32_tile_ref(a.blocks, a.nblocks, a.ncoarse, cta);
+  const TileRef R = tile_ref(a.blocks, a.nblocks, a.ncoarse, cta);
   T.b = R.b;
   T.slot = R.slot;
   const BlockDev &B = a.blocks[T.b];
@@ -868,7 +837,7 @@ __global__ void __launch_bounds__(kF32TX / 2 * TY, 512 / (kF32TX / 2 * TY)) k_st
 template <class S, int TX, int TY>
 __global__ void __launch_bounds__(TX *TY) k_spectral(StepArgs a) {
   constexpr int NT = TX * TY;
-  const TileRef R = f32_tile_ref(a.blocks, a.nblocks, a.ncoarse, blockIdx.x);
+  const TileRef R = tile_ref(a.blocks, a.nblocks, a.ncoarse, blockIdx.x);
   const BlockDev &B = a.blocks[R.b];
   const CavConst &C = a.cc[B.cav];
   const int i = R.tx * TX + threadIdx.x + 1, j = R.ty * TY + threadIdx.y + 1;

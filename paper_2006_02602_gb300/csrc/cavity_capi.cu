@@ -29,10 +29,10 @@ using namespace bdc;
 
 namespace {
 
-// k_step tile of the FP64 form: 32 x 4 threads (166 registers each: three
-// CTAs, 12 warps, per SM hide the FP64 pipe's latency better than one CTA of
-// 32 x 8), 8-plane chunks
-constexpr int kTX = 32, kTY = 4, kKC = 8;
+// k_step tile of the FP64 form: 32 * ty consecutive nodes of a plane (ty = 4:
+// 128 threads; three CTAs, 12 warps, per SM hide the FP64 pipe's latency
+// better than one of 256); the chunk depths: assign_tiles
+constexpr int kTX = 32, kTY = 4;
 
 int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
@@ -120,7 +120,7 @@ struct cavity {
   size_t esize = 8;               // bytes per stored element
   int na = 5;                     // stored arrays per buffer set
   int np = 1;                     // pressure arrays
-  int tx = kTX, ty = kTY, kc = kKC;
+  int tx = kTX, ty = kTY, kc = 8;
   int f32_r = 0;                  // ring depth of the FP32 step kernel
   int f32_p = 1;                  // nodes per thread along x of the FP32 step kernel
   int local_dt = 0;               // CAVITY_DT_LOCAL: each node at its own stable step
@@ -155,6 +155,7 @@ struct cavity {
   long long log_cap = 0;
   unsigned int *d_counter = nullptr;  // [ncav] k_bc CTAs done per cavity, the FP64 step's tile counter,
                                       // [ncav] the FP64 step's dt-filter floors
+  int nsm = 0;                        // SMs of the device
   int persist_ctas = 0;               // CTAs of the persistent FP64 step kernel that fit on the GPU
   void *d_fields = nullptr, *d_xbuf = nullptr;
   size_t field_bytes = 0;
@@ -231,26 +232,48 @@ int check_desc(const cavity_desc &d) {
 // layout: blocks of every cavity, wall / cut face lists, centre nodes
 
 // Step-kernel tiles and their partial slots, block by block (a cavity's
-// slots are contiguous).  The planes below the last KC-plane boundary go in
-// KC-plane chunks, the rest in fine chunks scheduled after every block's
-// coarse tiles: kFineKC planes in the FP64 form; kFineKC32 planes in the
-// FP32 form, and only in blocks deeper than one chunk (a shallower block is
-// one chunk: the ring's fill is paid per tile).
+// slots are contiguous): kc-plane chunks below the last chunk boundary, the
+// planes above it in fine chunks scheduled after every block's coarse tiles.
+//
+// FP64: what counts is the number of tile planes (128 nodes x 1 plane) an SM
+// gets.  A tile plane takes its SM's FP64 pipe about 3.3 us whatever else the
+// SM runs; a tile's own cost (queue loads, tile look-up, reduction) is about a
+// third of one.  So large cavities take 8-plane tiles with 2-plane ones in the
+// end, small ones 4-plane and 1-plane tiles, and the fine tiles hold 8 planes
+// an SM (all of a cavity of up to 38^3), enough to level what the coarse ones
+// leave.  Measured per step, chunks of 8 and 8-plane tails before: 32^3
+// 59.4 -> 20.6 us, 64^3 137 -> 66.5, 128^3 410 (8 planes, fine tiles in the
+// last 8 of 128 only) -> 384; the other side of the line: 4 planes at 256^3
+// 2835 against 2798 us, 8 planes at 64^3 80 against 66.5.
+//
+// FP32: kFineKC32-plane tail chunks, only in blocks deeper than one chunk (a
+// shallower block is one chunk: the ring's fill is paid per tile).
 void assign_tiles(cavity *h) {
+  long long planes = 0;
+  if (!h->f32) {
+    for (const BlockDev &B : h->hb) planes += (long long)ceil_div((long long)B.nx * B.ny, h->tx * h->ty) * B.nz;
+    h->kc = planes >= 64LL * h->nsm ? 8 : 4;
+  }
   int tile = 0, coarse = 0, fine = 0;
   for (int c = 0; c < h->ncav; ++c) h->hcc[c].tile_begin = -1;
   for (BlockDev &B : h->hb) {
-    B.tiles_x = ceil_div(B.nx, h->tx);
-    B.tiles_y = ceil_div(B.ny, h->ty);
-    const int kf = h->f32 ? kFineKC32 : kFineKC;
-    if (h->f32 && B.nz <= h->kc) {
-      B.tiles_zc = 1;
-      B.zsplit = B.nz;
-    } else {
+    B.kc = h->kc;
+    if (h->f32) {
+      B.tiles_x = ceil_div(B.nx, h->tx);
+      B.tiles_y = ceil_div(B.ny, h->ty);
+      B.kf = kFineKC32;
       B.tiles_zc = (B.nz - 1) / h->kc;
+      if (B.nz <= h->kc) B.tiles_zc = 1;
+      B.zsplit = std::min(B.nz, B.tiles_zc * h->kc);
+    } else {
+      B.tiles_x = ceil_div((long long)B.nx * B.ny, h->tx * h->ty);
+      B.tiles_y = 1;
+      B.kf = h->kc == 8 ? 2 : 1;
+      const int nfine = ceil_div(8LL * h->nsm * B.nz, planes);
+      B.tiles_zc = std::max(0, B.nz - nfine) / h->kc;
       B.zsplit = B.tiles_zc * h->kc;
     }
-    B.tiles_z = B.tiles_zc + ceil_div(B.nz - B.zsplit, kf);
+    B.tiles_z = B.tiles_zc + ceil_div(B.nz - B.zsplit, B.kf);
     B.tile_begin = tile;
     B.coarse_begin = coarse;
     B.fine_begin = fine;
@@ -492,13 +515,12 @@ int alloc_device(cavity *h) {
   CK(cudaMalloc(&h->d_counter, sizeof(unsigned int) * (2 * h->ncav + 1)));
   CK(cudaMemsetAsync(h->d_counter, 0, sizeof(unsigned int) * (2 * h->ncav + 1), h->stream));
   {
-    int nsm = 0, per_sm = 0;
-    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->dev));
+    int per_sm = 0;
     if (h->ty == 4)
-      CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_f64<kTX, 4, kKC>, kTX * 4, 0));
+      CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_f64<kTX * 4>, kTX * 4, 0));
     else
-      CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_f64<kTX, 8, kKC>, kTX * 8, 0));
-    h->persist_ctas = std::max(1, nsm * per_sm);
+      CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_f64<kTX * 8>, kTX * 8, 0));
+    h->persist_ctas = std::max(1, h->nsm * per_sm);
   }
   CK(cudaMalloc(&h->d_twall, sizeof(double) * std::max<size_t>(1, h->twall.size())));
   if (h->xbuf_elems > 0) CK(cudaMalloc(&h->d_xbuf, h->esize * (size_t)h->xbuf_elems));
@@ -580,14 +602,14 @@ ExchArgs exch_args(cavity *h, int parity) {
   return a;
 }
 
-// The persistent FP64 step kernel of the handle's tile height (8 or 4 rows;
-// 32 x TY threads, as many CTAs as fit on the GPU at once).
+// The persistent FP64 step kernel of the handle's tile size (32 * ty threads,
+// as many CTAs as fit on the GPU at once).
 void launch_step_f64(cavity *h, const StepArgs &a) {
   const int grid = std::min(h->n_step, h->persist_ctas);
   if (h->ty == 4)
-    k_step_f64<kTX, 4, kKC><<<grid, dim3(kTX, 4), 0, h->stream>>>(a);
+    k_step_f64<kTX * 4><<<grid, kTX * 4, 0, h->stream>>>(a);
   else
-    k_step_f64<kTX, 8, kKC><<<grid, dim3(kTX, 8), 0, h->stream>>>(a);
+    k_step_f64<kTX * 8><<<grid, kTX * 8, 0, h->stream>>>(a);
 }
 
 // `after_finalise`: the launch directly follows, in the same stream capture,
@@ -998,6 +1020,8 @@ int create_common(const cavity_desc *descs, const cavity_params *params, int n, 
       if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess) rc = CAVITY_ERR_CUDA;
       h->own_stream = true;
     }
+    if (rc == CAVITY_OK && cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->dev) != cudaSuccess)
+      rc = CAVITY_ERR_CUDA;
     if (rc == CAVITY_OK) rc = build_layout(h);
     if (rc == CAVITY_OK) rc = alloc_device(h);
     if (rc == CAVITY_OK) rc = upload_consts(h);

@@ -107,8 +107,8 @@ extern "C" CAVITY_API int cavity_step_block_noalloc(const double *q_in, double *
                                                     double *out6, void *stream) {
   if (!q_in || !q_out || !out6 || !p || q_in == q_out) return CAVITY_ERR_INVALID_ARG;
   if (nx < 2 || ny < 2 || nz < 2 || !(dt >= 0.0) || !std::isfinite(pshift)) return CAVITY_ERR_INVALID_ARG;
-  const long long ntiles = (long long)ceil_div(nx, kTX) * ceil_div(ny, kTY) * ceil_div(nz, kKC);
-  if (ntiles > CAVITY_NOALLOC_MAX_TILES) return CAVITY_ERR_INVALID_ARG;  // beyond the fixed scratch
+  const long long limit_tiles = (long long)ceil_div(nx, kTX) * ceil_div(ny, kTY) * ceil_div(nz, kKC);
+  if (limit_tiles > CAVITY_NOALLOC_MAX_TILES) return CAVITY_ERR_INVALID_ARG;  // beyond the fixed scratch
   cavity_params q = *p;
   if (!(q.u_ref >= 0.0)) q.u_ref = std::max(1.0, std::sqrt(q.Ra * q.Pr));
   if (std::isnan(q.t_inf)) q.t_inf = 0.5 * (q.t_hot + q.t_cold);
@@ -135,11 +135,12 @@ extern "C" CAVITY_API int cavity_step_block_noalloc(const double *q_in, double *
   B.plane = (long long)B.pitch * B.rows;
   B.fstride = B.plane * (nz + 4);
   for (int f = 0; f < 6; ++f) { B.wall[f] = 1; B.nbr[f] = -1; }
-  B.tiles_x = ceil_div(nx, kTX);
-  B.tiles_y = ceil_div(ny, kTY);
+  B.tiles_x = ceil_div((long long)nx * ny, kTX * kTY);
+  B.tiles_y = 1;
   B.tiles_z = ceil_div(nz, kKC);
   B.tiles_zc = B.tiles_z;  // one CTA per tile: KC-plane chunks only
   B.zsplit = nz;
+  B.kc = B.kf = kKC;
   B.coarse_begin = 0;
   B.fine_begin = 0;
   B.base[0] = (void *)(q_in - (XO<double>::v - 2));
@@ -158,11 +159,12 @@ extern "C" CAVITY_API int cavity_step_block_noalloc(const double *q_in, double *
   if (cudaGetLastError() != cudaSuccess) return CAVITY_ERR_CUDA;
   StepArgs a{};  // tile_counter null: one CTA per tile
   a.blocks = d_block; a.nblocks = 1; a.cc = d_cc; a.cs = d_cs;
-  a.partials = d_part; a.parity = 0; a.mode = 0; a.ntiles = (int)ntiles;
-  a.ncoarse = (int)ntiles;
-  k_step_f64<kTX, kTY, kKC><<<(int)ntiles, dim3(kTX, kTY), 0, st>>>(a);
+  const int ntiles = B.tiles_x * B.tiles_z;  // at most the limit's count: 256 consecutive nodes fill no fewer tiles
+  a.partials = d_part; a.parity = 0; a.mode = 0; a.ntiles = ntiles;
+  a.ncoarse = ntiles;
+  k_step_f64<kTX * kTY><<<ntiles, kTX * kTY, 0, st>>>(a);
   if (cudaGetLastError() != cudaSuccess) return CAVITY_ERR_CUDA;
-  k_noalloc_reduce<<<1, 256, 0, st>>>(d_part, (int)ntiles, d_cc, out6);
+  k_noalloc_reduce<<<1, 256, 0, st>>>(d_part, ntiles, d_cc, out6);
   if (cudaGetLastError() != cudaSuccess) return CAVITY_ERR_CUDA;
   return CAVITY_OK;
 }
