@@ -413,7 +413,7 @@ CAVITY_API int cavity_step_block_noalloc(const double *q_in, double *q_out, int 
  * clock cycles in [1000, 4e9]; 4e9, about 2 s, is the default) and, with
  * withhold_plane >= 0, leaves the load of that plane of every tile (0 = the
  * first halo plane below the tile's z range) unissued, so that its waits run
- * out; withhold_plane = -1 issues every load.  The step graphs are rebuilt.
+ * out; withhold_plane = -1 issues every load.
  * FP32-mixed handles only (CAVITY_ERR_UNSUPPORTED otherwise); the state of a
  * handle whose wait ran out is not a step of the scheme: destroy it. */
 CAVITY_API int cavity_test_wait_timeout(cavity_t *h, long long wait_cycles, int withhold_plane);

@@ -1,17 +1,20 @@
 // Device-side data structures and kernels of the buoyancy-driven-cavity step
 // (Xue & Roy, arXiv 2006.02602).  Shared by the C-ABI translation unit only.
 //
-// Per step, on the handle's stream (one CUDA graph per buffer parity):
+// Per step, on the handle's stream (CUDA graphs of 1, 4 and 16 steps per
+// buffer parity, each kernel a programmatic dependent of the one before):
 //   k_step      fused residual (Eqs. 1-3) + explicit Euler update of every
-//               interior node of every block, FP64 residual sums and the
-//               spectral-radius max of the new state as per-CTA partials;
-//   k_bc        wall conditions (Section 2) and the hot/cold-wall Nusselt
-//               sums; the last CTA to finish reduces the partials in a
-//               fixed order: residual norms, next dt, centre pressure,
-//               Nusselt numbers, time, step, non-finite flag;
-//   k_pack      cut-face ghost data -> contiguous buffers (Section 4.5,
-//               Listings 1-2, V3): p at depth 2, u, v, w, T at depth 1;
-//   k_unpack    buffers -> the neighbour's ghost layers.
+//               interior node of every block, walls (Section 2) formed where
+//               they are read; FP64 residual sums as per-CTA partials, the
+//               spectral-radius maximum of the new state as an atomic maximum;
+//   k_between   what the next step waits for: dt from that maximum, the centre
+//               shift, and with cut faces the ghost layers of the new state
+//               from the neighbours' layers (Section 4.5, Listings 1-2, V3: p
+//               at depth 2, u, v, w, T at depth 1);
+//   k_finalize  once a graph, for all of its steps: the partials reduced in a
+//               fixed order: residual norms, Nusselt numbers, time, step log,
+//               non-finite flag.
+// On a state refresh: k_bc (walls stored), k_pack / k_unpack.
 //
 // Storage: each block holds two buffer sets (ping-pong); a set is NF
 // consecutive padded arrays, x fastest.  Local node (i, j, k), i in
@@ -19,6 +22,7 @@
 // so that node 1 of every row starts on a 32-byte boundary.
 #pragma once
 
+#include <cfloat>
 #include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -87,6 +91,7 @@ struct CavConst {
   double wscale[2];                  // FP32 step's sums of 3 T_w - 4 T_1 + T_2 -> hot, cold wall fluxes: +-h_x^-1 / (2 dT)
   int bc_begin, bc_end;              // k_bc CTAs of this cavity (all wall faces)
   int bc_xend;                       // the x walls' CTAs (the Nusselt partials) come first: bc_begin .. bc_xend-1
+  int nu_begin, nu_end;              // CTAs of this cavity in the list of its x walls alone
   long long wall_off;                // offset of this cavity's wall temperatures
 };
 
@@ -158,6 +163,12 @@ struct CavState {
   double nu_hot, nu_cold;
   int flags;         // bit 0: non-finite residual or spectral radius
   int pad;
+  // for the step in flight (zero before it): the largest spectral bound of its
+  // new state, and the FP64 step's largest published dt-filter floor
+  // (float_key ^ 0x80000000, 0 = none)
+  double smax;
+  unsigned int sfl, pad2;
+  double dt0;        // dt as the last finalise left it (dt itself moves on within a graph)
 };
 
 struct StepRecord {   // one step's record in the host-memory step log (the C ABI's cavity_step_record)
@@ -322,64 +333,79 @@ struct NodeF64 {
   double u[7], v[7], w[7], T[7];
 };
 
-__device__ __forceinline__ void rates_f64(const CavConst &C, const NodeF64 &n, double r[5]) {
+// The part of the rates that reads the velocities alone (and the centre T):
+// beta^2, the dissipation weights, div V and the momentum rates without the
+// pressure gradient.
+struct VelF64 {
+  double b2, ex, ey, ez, divV, ru, rv, rw;
+};
+
+#define BDC_TRANSPORT(q, xm, xp, ym, yp, zm, zp, centre) \
+  fma(xp, q[2], fma(xm, q[1], fma(yp, q[4], fma(ym, q[3], fma(zp, q[6], fma(zm, q[5], centre))))))
+
+__device__ __forceinline__ void rates_vel_f64(const CavConst &C, const NodeF64 &n, VelF64 &x) {
   const double u0 = n.u[0], v0 = n.v[0], w0 = n.w[0];
   const double b2 = max_nonneg(fma(u0, u0, fma(v0, v0, w0 * w0)), C.b2min);
   const double f4 = times4(b2);
-  const double ex = (fabs(u0) + sqrt_newton(fma(u0, u0, f4))) * C.dsc[0];
-  const double ey = (fabs(v0) + sqrt_newton(fma(v0, v0, f4))) * C.dsc[1];
-  const double ez = (fabs(w0) + sqrt_newton(fma(w0, w0, f4))) * C.dsc[2];
-  const double p0 = n.p[0];
-  const double d4x = fma(6.0, p0, fma(-4.0, n.p[2] + n.p[1], n.p[8] + n.p[7]));
-  const double d4y = fma(6.0, p0, fma(-4.0, n.p[4] + n.p[3], n.p[10] + n.p[9]));
-  const double d4z = fma(6.0, p0, fma(-4.0, n.p[6] + n.p[5], n.p[12] + n.p[11]));
-  const double diss = fma(ex, d4x, fma(ey, d4y, ez * d4z));
-  const double divV = fma(n.u[2] - n.u[1], C.ih2[0], fma(n.v[4] - n.v[3], C.ih2[1], (n.w[6] - n.w[5]) * C.ih2[2]));
-  r[0] = fma(-b2, divV, -diss);
-
+  x.b2 = b2;
+  x.ex = (fabs(u0) + sqrt_newton(fma(u0, u0, f4))) * C.dsc[0];
+  x.ey = (fabs(v0) + sqrt_newton(fma(v0, v0, f4))) * C.dsc[1];
+  x.ez = (fabs(w0) + sqrt_newton(fma(w0, w0, f4))) * C.dsc[2];
+  x.divV = fma(n.u[2] - n.u[1], C.ih2[0], fma(n.v[4] - n.v[3], C.ih2[1], (n.w[6] - n.w[5]) * C.ih2[2]));
   // neighbour weights: m = minus side, p = plus side
   const double nxm = fma(u0, C.ih2[0], C.nuhh[0]), nxp = fma(-u0, C.ih2[0], C.nuhh[0]);
   const double nym = fma(v0, C.ih2[1], C.nuhh[1]), nyp = fma(-v0, C.ih2[1], C.nuhh[1]);
   const double nzm = fma(w0, C.ih2[2], C.nuhh[2]), nzp = fma(-w0, C.ih2[2], C.nuhh[2]);
-#define BDC_TRANSPORT(q, xm, xp, ym, yp, zm, zp, centre) \
-  fma(xp, q[2], fma(xm, q[1], fma(yp, q[4], fma(ym, q[3], fma(zp, q[6], fma(zm, q[5], centre))))))
   // the buoyancy force (Eq. 2) enters the gravity-axis momentum rate with its centre term
   const double buoy = fma(C.gs, n.T[0], -C.gst);
   const double bv = C.gaxis == 1 ? buoy : 0.0, bw = C.gaxis == 2 ? buoy : 0.0;
-  r[1] = fma(-(n.p[2] - n.p[1]), C.ih2[0], BDC_TRANSPORT(n.u, nxm, nxp, nym, nyp, nzm, nzp, -C.nu2s * u0));
-  r[2] = fma(-(n.p[4] - n.p[3]), C.ih2[1], BDC_TRANSPORT(n.v, nxm, nxp, nym, nyp, nzm, nzp, fma(-C.nu2s, v0, bv)));
-  r[3] = fma(-(n.p[6] - n.p[5]), C.ih2[2], BDC_TRANSPORT(n.w, nxm, nxp, nym, nyp, nzm, nzp, fma(-C.nu2s, w0, bw)));
+  x.ru = BDC_TRANSPORT(n.u, nxm, nxp, nym, nyp, nzm, nzp, -C.nu2s * u0);
+  x.rv = BDC_TRANSPORT(n.v, nxm, nxp, nym, nyp, nzm, nzp, fma(-C.nu2s, v0, bv));
+  x.rw = BDC_TRANSPORT(n.w, nxm, nxp, nym, nyp, nzm, nzp, fma(-C.nu2s, w0, bw));
+}
+
+__device__ __forceinline__ void rates_pt_f64(const CavConst &C, const NodeF64 &n, const VelF64 &x, double r[5]) {
+  const double u0 = n.u[0], v0 = n.v[0], w0 = n.w[0], p0 = n.p[0];
+  const double d4x = fma(6.0, p0, fma(-4.0, n.p[2] + n.p[1], n.p[8] + n.p[7]));
+  const double d4y = fma(6.0, p0, fma(-4.0, n.p[4] + n.p[3], n.p[10] + n.p[9]));
+  const double d4z = fma(6.0, p0, fma(-4.0, n.p[6] + n.p[5], n.p[12] + n.p[11]));
+  const double diss = fma(x.ex, d4x, fma(x.ey, d4y, x.ez * d4z));
+  r[0] = fma(-x.b2, x.divV, -diss);
+  r[1] = fma(-(n.p[2] - n.p[1]), C.ih2[0], x.ru);
+  r[2] = fma(-(n.p[4] - n.p[3]), C.ih2[1], x.rv);
+  r[3] = fma(-(n.p[6] - n.p[5]), C.ih2[2], x.rw);
   const double txm = fma(u0, C.ih2[0], C.alhh[0]), txp = fma(-u0, C.ih2[0], C.alhh[0]);
   const double tym = fma(v0, C.ih2[1], C.alhh[1]), typ = fma(-v0, C.ih2[1], C.alhh[1]);
   const double tzm = fma(w0, C.ih2[2], C.alhh[2]), tzp = fma(-w0, C.ih2[2], C.alhh[2]);
   r[4] = BDC_TRANSPORT(n.T, txm, txp, tym, typ, tzm, tzp, -C.al2s * n.T[0]);
-#undef BDC_TRANSPORT
 }
+#undef BDC_TRANSPORT
 
 // spectral-radius bound of one node's state (the dt denominator); square
 // roots within one unit in the last place (sqrt_newton), so dt is the
 // correctly rounded formula's to a few ulp
 __device__ __forceinline__ double spectral_f64(const CavConst &C, double u, double v, double w) {
-  const double b2 = max_nonneg(u * u + v * v + w * w, C.b2min);
+  // (every product-sum an explicit FMA: the same bits in every kernel)
+  const double b2 = max_nonneg(fma(u, u, fma(v, v, w * w)), C.b2min);
   const double f4 = times4(b2);
-  const double sx = fabs(u) + sqrt_newton(u * u + f4);
-  const double sy = fabs(v) + sqrt_newton(v * v + f4);
-  const double sz = fabs(w) + sqrt_newton(w * w + f4);
-  return 0.5 * (sx * C.ih[0] + sy * C.ih[1] + sz * C.ih[2]) + C.diffsr;
+  const double sx = fabs(u) + sqrt_newton(fma(u, u, f4));
+  const double sy = fabs(v) + sqrt_newton(fma(v, v, f4));
+  const double sz = fabs(w) + sqrt_newton(fma(w, w, f4));
+  return fma(0.5, fma(sx, C.ih[0], fma(sy, C.ih[1], sz * C.ih[2])), C.diffsr);
 }
 
-// Rates and explicit update of one node: the new p, u, v, w, T in q (p with
+// Rates (from their velocity part x on) and explicit update of one node: the new p, u, v, w, T in q (p with
 // the pending centre shift taken off), the rates in r.  One function for
 // k_step_f64 and k_shell_f64, so a node gives the same bits in either.
-__device__ __forceinline__ void update_node_f64(const CavConst &C, const NodeF64 &n, double dt, double cshift,
-                                                int local_dt, double q[5], double r[5]) {
-  rates_f64(C, n, r);
+__device__ __forceinline__ void update_node_f64(const CavConst &C, const NodeF64 &n, const VelF64 &x, double dt,
+                                                double cshift, int local_dt, double q[5], double r[5]) {
+  rates_pt_f64(C, n, x, r);
   const double dtn = local_dt ? C.cfl / spectral_f64(C, n.u[0], n.v[0], n.w[0]) : dt;
-  q[0] = (n.p[0] - cshift) + dtn * r[0];
-  q[1] = n.u[0] + dtn * r[1];
-  q[2] = n.v[0] + dtn * r[2];
-  q[3] = n.w[0] + dtn * r[3];
-  q[4] = n.T[0] + dtn * r[4];
+  q[0] = fma(dtn, r[0], n.p[0] - cshift);
+  q[1] = fma(dtn, r[1], n.u[0]);
+  q[2] = fma(dtn, r[2], n.v[0]);
+  q[3] = fma(dtn, r[3], n.w[0]);
+  q[4] = fma(dtn, r[4], n.T[0]);
 }
 
 // FP32 estimate of spectral_f64 (the same formula: relative error below
@@ -467,19 +493,51 @@ struct StepArgs {
   const BlockDev *blocks;
   int nblocks;
   const CavConst *cc;
-  const CavState *cs;
+  CavState *cs;
   double *partials;  // [tile][kPartStride]
   int parity;        // read base[parity], write base[parity ^ 1]
   int mode;          // 0 = step, 1 = spectral radius of the current state only
-  unsigned int *sfloor;        // per cavity: the largest published dt-filter floor of this step
-                               // (float_key ^ 0x80000000, 0 = none; reset by the next k_bc); null: none
-  unsigned int *tile_counter;  // persistent CTAs fetch tiles from it (reset by the next k_bc);
-                               // null: one CTA per tile
+  unsigned int *tile_counter;  // persistent CTAs fetch tiles from it (zero before a step); null: one CTA per tile
   int ntiles;
   int local_dt;                // 1: each node at dt_n = cfl / S_n of its state (pseudo time)
   int skip_shell;              // 1: leave the nodes within two layers of a cut face to k_shell_f64
   int ncoarse;                 // coarse tiles of all blocks (scheduling indices below it)
+  int nnu;                     // the first CTAs: the x walls' Nusselt sums of the state read here
 };
+
+// p of one stored node through L2
+template <class S>
+__device__ __forceinline__ double load_p_l2(const S *base, long long fs, long long o);
+template <>
+__device__ __forceinline__ double load_p_l2<double>(const double *base, long long, long long o) {
+  return __ldcg(base + o);
+}
+template <>
+__device__ __forceinline__ double load_p_l2<float>(const float *base, long long fs, long long o) {
+  return (double)__ldcg(base + o) + (double)__ldcg(base + fs + o);
+}
+
+// The mean of p over the centre nodes (their count is 1, 2, 4 or 8: the scaling
+// is exact), summed in lexicographic (k, j, i) order; absent nodes are zeros.
+__device__ __forceinline__ double centre_mean(int n, const double *v) {
+  double csum = 0.0;
+  for (int m = 0; m < kMaxCentre; ++m) csum += v[m];
+  return csum * (n == 8 ? 0.125 : n == 4 ? 0.25 : n == 2 ? 0.5 : 1.0);
+}
+
+__device__ __forceinline__ void step_max(CavState &st, double smax) {
+  // positive values order like their bit patterns
+  atomicMax((unsigned long long *)&st.smax, (unsigned long long)__double_as_longlong(smax));
+}
+
+// A programmatic dependent: every earlier kernel of the chain has finished
+// and its memory is visible.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The kernel after this one may start when every CTA has said so (or ended): a
+// step's CTAs do at the end of their sweeps, so that the next step's are not
+// placed beside them on whichever SMs have room (an uneven spread: 128^3
+// FP32-mixed 71 us a step against 52).
+__device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // whether local node (i, j, k) of B lies within two layers of one of B's cut
 // faces with index below `faces` (all six: faces = 6)
@@ -533,6 +591,19 @@ __device__ __forceinline__ TileRef tile_ref(const BlockDev *blocks, int nblocks,
   return T;
 }
 
+// x / 3 correctly rounded in three FP64 operations (a rounded reciprocal, then
+// one residual correction through fused multiply-adds: Markstein, IBM J. Res.
+// Dev. 34 (1990)), where a full division is a long dependent FP64 sequence on
+// GB300's narrow FP64 pipe.
+__device__ __forceinline__ double div3(double x) {
+  constexpr double y = 1.0 / 3.0;
+  const double q = x * y;
+  return fma(fma(-q, 3.0, x), y, q);
+}
+
+// the adiabatic wall's T from the two interior nodes next to it
+__device__ __forceinline__ double adiabatic_T(double T1, double T2) { return div3(fma(4.0, T1, -T2)); }
+
 // wfloor: a warp-uniform FP32 value of D = S - S0 at or below the one of an
 // exact spectral value of this step that some lane of the warp -- or, through
 // the cavity's published floor, of any CTA -- has already recorded, lowered
@@ -543,11 +614,21 @@ __device__ __forceinline__ TileRef tile_ref(const BlockDev *blocks, int nblocks,
 // hence dt -- is exactly the FP64 one.  Carried across the warp's tiles of
 // one cavity (`fcav`: the cavity it belongs to; a tile of another cavity,
 // in a batch, starts again from -inf).
-template <int NT>
+//
+// Walls (Section 2) are formed where they are read (FORM), from the two
+// interior layers next to each wall, by the formulas k_bc stores them with: two
+// FP64 operations in the warps that hold a node next to an x wall, a few in the
+// first and last planes.  u = v = w = 0 and the isothermal T never change and
+// stay stored.  Large cavities read stored walls, which k_between writes: the
+// line is at 64 tile planes an SM, where forming them takes 3.5% of the step
+// (128^3: 390 us a step, 381 stored) and storing them 5 us; at 64^3 the step is
+// 62 us with walls formed, 59 without any.
+template <int NT, bool FORM>
 __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float &wfloor, int &fcav) {
   const TileRef tile = tile_ref(a.blocks, a.nblocks, a.ncoarse, cta);
   const BlockDev &B = a.blocks[tile.b];
   const CavConst &C = a.cc[B.cav];
+  CavState &st = a.cs[B.cav];
   if (B.cav != fcav) {
     wfloor = -INFINITY;
     fcav = B.cav;
@@ -555,8 +636,8 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
   // the cavity's floor as published by every CTA so far this step (a value
   // at or below an exact spectral value some warp recorded): warps far from
   // the maximum start near it too
-  if (a.mode == 0 && a.sfloor) {
-    const unsigned u = *(volatile const unsigned *)&a.sfloor[B.cav];
+  if (a.mode == 0) {
+    const unsigned u = *(volatile const unsigned *)&st.sfl;
     if (u != 0u) wfloor = fmaxf(wfloor, key_float((int)(u ^ 0x80000000u)));
   }
   float published = wfloor;
@@ -565,8 +646,8 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
   const int k0 = tile.k0;
   const int k1 = tile.k1;
   const bool active = j <= B.ny;
-  const double dt = a.cs[B.cav].dt;
-  const double cshift = a.cs[B.cav].c;
+  const double dt = st.dt;
+  const double cshift = st.c;
 
   const double *__restrict__ src = (const double *)B.base[a.parity];
   double *__restrict__ dst = (double *)B.base[a.parity ^ 1];
@@ -578,38 +659,97 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
   const double *__restrict__ TT = src + 4 * fs;
   const long long pl = B.plane, pt = B.pitch;
 
+  // the node's place next to the x and y walls: bits 1, 2 the first and second
+  // node from x = 0, 4, 8 from the other x wall, 16 .. 128 the y walls
+  int edge = 0;
+  if (B.wall[0]) edge |= i == 1 ? 1 : i == 2 ? 2 : 0;
+  if (B.wall[1]) edge |= i == B.nx ? 4 : i == B.nx - 1 ? 8 : 0;
+  if (B.wall[2]) edge |= j == 1 ? 16 : j == 2 ? 32 : 0;
+  if (B.wall[3]) edge |= j == B.ny ? 64 : j == B.ny - 1 ? 128 : 0;
+  const int zlow = B.wall[4] ? 2 : 0, zhigh = B.wall[5] ? B.nz - 1 : B.nz + 1;  // planes next to the z walls
   double s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0, smax = 0;
   if (active) {
+    const bool edge_x = FORM && __any_sync(__activemask(), edge & 15);
+    const bool edge_y = FORM && __any_sync(__activemask(), edge & 240);
     long long o = node_index<double>(B, i, j, k0);
     // z queues: p at k-2..k+1, the others at k-1..k
-    double pq0 = __ldg(P + o - 2 * pl), pq1 = __ldg(P + o - pl), pq2 = __ldg(P + o), pq3 = __ldg(P + o + pl);
-    double uq0 = __ldg(U + o - pl), uq1 = __ldg(U + o);
-    double vq0 = __ldg(V + o - pl), vq1 = __ldg(V + o);
-    double wq0 = __ldg(W + o - pl), wq1 = __ldg(W + o);
-    double Tq0 = __ldg(TT + o - pl), Tq1 = __ldg(TT + o);
+    double pq0 = P[o - 2 * pl], pq1 = P[o - pl], pq2 = P[o], pq3 = P[o + pl];
+    double uq0 = U[o - pl], uq1 = U[o];
+    double vq0 = V[o - pl], vq1 = V[o];
+    double wq0 = W[o - pl], wq1 = W[o];
+    double Tq0 = TT[o - pl], Tq1 = TT[o];
     for (int k = k0; k <= k1; ++k, o += pl) {
       NodeF64 n;
-      const double pq4 = __ldg(P + o + 2 * pl);
-      const double uq2 = __ldg(U + o + pl), vq2 = __ldg(V + o + pl), wq2 = __ldg(W + o + pl), Tq2 = __ldg(TT + o + pl);
+      const double pq4 = P[o + 2 * pl];
+      const double uq2 = U[o + pl], vq2 = V[o + pl], wq2 = W[o + pl], Tq2 = TT[o + pl];
       if (a.mode == 0 && a.skip_shell && in_shell(B, i, j, k, 6)) {
         // computed by k_shell_f64 (interior/shell split)
       } else if (a.mode == 0) {
         n.p[0] = pq2; n.p[5] = pq1; n.p[6] = pq3; n.p[11] = pq0; n.p[12] = pq4;
-        n.p[1] = __ldg(P + o - 1); n.p[2] = __ldg(P + o + 1);
-        n.p[7] = __ldg(P + o - 2); n.p[8] = __ldg(P + o + 2);
-        n.p[3] = __ldg(P + o - pt); n.p[4] = __ldg(P + o + pt);
-        n.p[9] = __ldg(P + o - 2 * pt); n.p[10] = __ldg(P + o + 2 * pt);
+        n.p[1] = P[o - 1]; n.p[2] = P[o + 1];
+        n.p[7] = P[o - 2]; n.p[8] = P[o + 2];
+        n.p[3] = P[o - pt]; n.p[4] = P[o + pt];
+        n.p[9] = P[o - 2 * pt]; n.p[10] = P[o + 2 * pt];
 #define BDC_LOAD7(arr, F, q0, q1, q2)                                           \
   arr[0] = q1; arr[5] = q0; arr[6] = q2;                                        \
-  arr[1] = __ldg(F + o - 1); arr[2] = __ldg(F + o + 1);                         \
-  arr[3] = __ldg(F + o - pt); arr[4] = __ldg(F + o + pt);
+  arr[1] = F[o - 1]; arr[2] = F[o + 1];                         \
+  arr[3] = F[o - pt]; arr[4] = F[o + pt];
+        BDC_LOAD7(n.T, TT, Tq0, Tq1, Tq2)
         BDC_LOAD7(n.u, U, uq0, uq1, uq2)
         BDC_LOAD7(n.v, V, vq0, vq1, vq2)
         BDC_LOAD7(n.w, W, wq0, wq1, wq2)
-        BDC_LOAD7(n.T, TT, Tq0, Tq1, Tq2)
 #undef BDC_LOAD7
+        // the velocities' part first: it needs no wall value, and its arrays are
+        // gone when the walls change p and T in place (168 registers; all
+        // loads and the walls first took 218)
+        VelF64 x;
+        rates_vel_f64(C, n, x);
+        // walls: branches a warp skips as a whole (inlined as predicated code,
+        // their FP64 operations cost every warp 15%)
+        if (FORM) {
+          if (edge_x) {
+            if (edge & 3) {  // x = 0: w = 2 p1 - p2, g = 2 w - p1
+              if (edge & 1) n.p[1] = fma(2.0, pq2, -n.p[2]);
+              n.p[7] = fma(2.0, n.p[1], -pq2);
+            }
+            if (edge & 12) {
+              if (edge & 4) n.p[2] = fma(2.0, pq2, -n.p[1]);
+              n.p[8] = fma(2.0, n.p[2], -pq2);
+            }
+          }
+          if (edge_y) {
+            if (edge & 48) {
+              if (edge & 16) {
+                n.p[3] = fma(2.0, pq2, -n.p[4]);
+                n.T[3] = adiabatic_T(Tq1, n.T[4]);
+              }
+              n.p[9] = fma(2.0, n.p[3], -pq2);
+            }
+            if (edge & 192) {
+              if (edge & 64) {
+                n.p[4] = fma(2.0, pq2, -n.p[3]);
+                n.T[4] = adiabatic_T(Tq1, n.T[3]);
+              }
+              n.p[10] = fma(2.0, n.p[4], -pq2);
+            }
+          }
+          if (k <= zlow) {
+            if (k == 1) {
+              n.p[5] = fma(2.0, pq2, -pq3);
+              n.T[5] = adiabatic_T(Tq1, Tq2);
+            }
+            n.p[11] = fma(2.0, n.p[5], -pq2);
+          }
+          if (k >= zhigh) {
+            if (k == zhigh + 1) {
+              n.p[6] = fma(2.0, pq2, -pq1);
+              n.T[6] = adiabatic_T(Tq1, Tq0);
+            }
+            n.p[12] = fma(2.0, n.p[6], -pq2);
+          }
+        }
         double r[5], qn[5];
-        update_node_f64(C, n, dt, cshift, a.local_dt, qn, r);
+        update_node_f64(C, n, x, dt, cshift, a.local_dt, qn, r);
         const double un = qn[1], vn = qn[2], wn = qn[3];
         for (int f = 0; f < 5; ++f) dst[o + f * fs] = qn[f];
         s0 += r[0] * r[0]; s1 += r[1] * r[1]; s2 += r[2] * r[2]; s3 += r[3] * r[3]; s4 += r[4] * r[4];
@@ -623,9 +763,9 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
         // share over the lanes sweeping this tile (all active lanes run the same k range)
         const unsigned am = __activemask();
         wfloor = fmaxf(wfloor, key_float(__reduce_max_sync(am, float_key(best))));
-        if (wfloor > published && a.sfloor) {  // publish a rise for the other warps
+        if (wfloor > published) {  // publish a rise for the other warps
           if ((int)(threadIdx.x & 31) == __ffs(am) - 1)
-            atomicMax(&a.sfloor[B.cav], (unsigned)float_key(wfloor) ^ 0x80000000u);
+            atomicMax(&st.sfl, (unsigned)float_key(wfloor) ^ 0x80000000u);
           published = wfloor;
         }
       } else {
@@ -665,33 +805,9 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
       unsigned long long m = redm[0];
       for (int q = 1; q < NT / 32; ++q) m = redm[q] > m ? redm[q] : m;
       v = __longlong_as_double((long long)m);
+      if (s == 0 && a.mode == 0) step_max(st, v);
     }
     if (s == 0) a.partials[(long long)tile.slot * kPartStride + f] = v;
-  }
-}
-
-// Persistent form: as many CTAs as fit on the GPU at once take tiles in
-// order from a counter, so the last round is short (one CTA per tile left a
-// partial wave of up to a third of the step on 152 SMs); the counter hands
-// out every block's coarse tiles before the fine tail tiles, and the next
-// tile is fetched while the current one is computed.  Partials stay indexed by
-// tile slot: the reductions do not depend on which CTA took a tile.
-template <int NT>
-__global__ void __launch_bounds__(NT) k_step_f64(StepArgs a) {
-  float wfloor = -INFINITY;
-  int fcav = -1;
-  if (!a.tile_counter) {
-    step_tile_f64<NT>(a, blockIdx.x, wfloor, fcav);
-    return;
-  }
-  // the first tile of each CTA is its own index; the counter starts at the grid's size
-  __shared__ int s_tile[2];
-  int tile = blockIdx.x;
-  for (int n = 0; tile < a.ntiles; n ^= 1) {
-    if (threadIdx.x == 0) s_tile[n] = (int)(gridDim.x + atomicAdd(a.tile_counter, 1u));
-    step_tile_f64<NT>(a, tile, wfloor, fcav);
-    __syncthreads();
-    tile = s_tile[n];
   }
 }
 
@@ -755,7 +871,9 @@ static __global__ void __launch_bounds__(kShellThreads) k_shell_f64(ShellArgs a)
       }
       const CavState &st = a.cs[B.cav];
       double r[5], qn[5];
-      update_node_f64(C, nd, st.dt, st.c, a.local_dt, qn, r);
+      VelF64 x;
+      rates_vel_f64(C, nd, x);
+      update_node_f64(C, nd, x, st.dt, st.c, a.local_dt, qn, r);
       for (int f = 0; f < 5; ++f) {
         dst[o + f * fs] = qn[f];
         s[f] = r[f] * r[f];
@@ -783,13 +901,20 @@ static __global__ void __launch_bounds__(kShellThreads) k_shell_f64(ShellArgs a)
 // k_bc (wall conditions + Nusselt partials) and k_finalize (reduction of the
 // partials, state advance).
 
-// k_pack / k_unpack / the finalise's exchange CTAs (below)
+// k_pack / k_unpack / k_exchange (below)
 struct ExchArgs {
   const BlockDev *blocks;
   const CutFace *faces;
   int nfaces;
   double *buf;   // FP64 storage: values; FP32 storage: reinterpreted as float
   int parity;
+};
+
+constexpr int kGraphMax = 16;  // steps of the longest graph
+
+struct StepResult {  // one step's outcome of one cavity, from that step's last finalise CTA
+  double res[5], dt, nu[2];
+  int bad;
 };
 
 struct BcArgs {
@@ -801,17 +926,20 @@ struct BcArgs {
   int ncav;
   const double *step_partials;
   double *bc_partials;        // [k_bc cta][2]
-  unsigned int *counter;      // per cavity: k_finalize slices done
+  unsigned int *counter;      // [nsteps][ncav] CTAs done, then [ncav] steps done (zero between launches)
   const double *t_wall;       // hot walls then cold walls, per cavity at wall_off
-  unsigned int *tile_counter; // the persistent step kernel's tile counter: reset here
-  unsigned int *sfloor;       // the step kernel's per-cavity dt-filter floors: reset here
+  unsigned int *tile_counter; // the FP64 step's tile counter: reset here
   long long shell_begin, shell_end;  // k_shell_f64 partial slots of this step (single cavity; empty if equal)
   int parity;                 // buffer set holding the new state
-  const CutFace *cuts;        // after a step with cut faces: the exchange of the new state, run by
-  int ncuts;                  //   the CTAs after the finalise CTAs (null / 0: none)
-  void *xbuf;
-  int nslices;                // k_finalize CTAs per cavity (1 .. kFinSlices)
-  int wall_ctas;              // after an FP64 step: k_bc's CTAs, run in the finalise launch (0: none)
+  int nslices;                // finalise CTAs per cavity (1 .. kFinSlices)
+  int wall_ctas;              // after an FP64 step: CTAs of the finalise that take the x walls' Nusselt sums
+                              //   (nu_only), or all walls (the overlapped schedule)
+  int nu_only;                // 1: wall_ctas read the new state's T next to the x walls (faces: the x walls
+                              //   alone) and write no walls
+  int nsteps;                 // steps of the graph (1 .. kGraphMax), their partials part_stride, bc_stride apart
+  long long part_stride, bc_stride;
+  double *mid;                // [nsteps][ncav][kFinSlices][8] slice totals
+  StepResult *rec;            // [nsteps][ncav]
   StepRecord *log;            // after a step: the step log (host memory), or null
   long long log_cap;          // its records per cavity
   int mode;                   // 0 after a step, 1 after init / set_fields,
@@ -820,20 +948,15 @@ struct BcArgs {
                               //   sums in the step partials
 };
 
-// x / 3 correctly rounded in three FP64 operations (a rounded reciprocal, then
-// one residual correction through fused multiply-adds: Markstein, IBM J. Res.
-// Dev. 34 (1990)), where a full division is a long dependent FP64 sequence on
-// GB300's narrow FP64 pipe.
-__device__ __forceinline__ double div3(double x) {
-  constexpr double y = 1.0 / 3.0;
-  const double q = x * y;
-  return fma(fma(-q, 3.0, x), y, q);
+// the outward wall heat flux over the temperature difference at an x-wall node
+__device__ __forceinline__ double wall_flux(const CavConst &C, double tw, double T1, double T2) {
+  return (3.0 * tw - 4.0 * T1 + T2) * (0.5 * C.ih[0]) * C.inv_dT;
 }
 
 // Walls of one face node.  u = v = w = 0 and the isothermal T never change
 // between steps: they are written (into both buffer sets) only when `other`
-// is given (state refresh); every step rewrites p's wall and ghost values and
-// the adiabatic T, and reads T next to the x walls for the Nusselt sums.
+// is given (state refresh); p's wall and ghost values and the adiabatic T are
+// written, and T next to the x walls goes into the Nusselt sums.
 template <class S>
 __device__ __forceinline__ void apply_wall(const BlockDev &B, const CavConst &C, S *base, int face,
                                            int c1, int c2, const double *t_wall, double &nu_h,
@@ -871,10 +994,10 @@ __device__ __forceinline__ void apply_wall(const BlockDev &B, const CavConst &C,
       store_T<S>(base, fs, W, tw);
       store_T<S>(other, fs, W, tw);
     }
-    const double flux = (3.0 * tw - 4.0 * T1 + T2) * (0.5 * C.ih[0]) * C.inv_dT;
+    const double flux = wall_flux(C, tw, T1, T2);
     if (high) nu_c += -flux; else nu_h += flux;
   } else {
-    store_T<S>(base, fs, W, div3(4.0 * T1 - T2));
+    store_T<S>(base, fs, W, adiabatic_T(T1, T2));
   }
 }
 
@@ -888,10 +1011,18 @@ __device__ __forceinline__ void apply_wall(const BlockDev &B, const CavConst &C,
 // slice) and every sum is a shallow fixed tree: within a CTA the eight
 // fields are transposed through shared memory and summed by 16 threads each
 // (an 8-term tree, then four butterfly levels), and the last CTA of a cavity
-// combines the slice totals by the same butterfly.  Nusselt sums: the wall
-// kernel's partials (modes 0, 1) or the step partials' slots 6 and 7, sums of
-// 3 T_w - 4 T_1 + T_2 (mode 4, FP32 step).  After a step of a decomposed
-// cavity, CTAs after the finalise CTAs exchange the new state's cut faces.
+// combines the slice totals by the same butterfly.  Nusselt sums: the x-wall
+// CTAs' or the wall kernel's partials (modes 0, 1) or the step partials' slots
+// 6 and 7, sums of 3 T_w - 4 T_1 + T_2 (mode 4, FP32 step).
+//
+// Where it runs: nothing of it is needed to start the next step (dt comes from
+// the atomic maximum, the centre shift from the state itself), so it runs once
+// at the end of a graph, for all of the graph's steps at once, each from its own
+// set of partials; the last step's last CTA then goes through the steps in
+// order (time, step log, flags).  As a kernel between the steps it took 7-9 us
+// of every step (FP32-mixed 256^3), 12 with the FP64 walls and 16-19 with a
+// decomposed cavity's exchange.  (In the first CTAs of the next step's launch
+// instead, its call cost the FP32 step kernel spills and 7% of its time.)
 constexpr int kFinThreads = 128;
 
 __device__ __forceinline__ double fin_comb(int f, double x, double y) { return f == 5 ? fmax(x, y) : x + y; }
@@ -914,19 +1045,20 @@ __device__ __forceinline__ double fin_tree(const double *sv, int f, int s) {
 
 // One slice of a cavity's partials, thread tid's in thread-strided order.
 template <int NT>
-__device__ __forceinline__ void load_slice(const BcArgs &a, long long q0, long long q1, long long b0, long long b1,
-                                           long long s0, long long s1, int tid, double acc[8]) {
+__device__ __forceinline__ void load_slice(const BcArgs &a, const double *step_partials, long long q0, long long q1,
+                                           long long b0, long long b1, long long s0, long long s1, int tid,
+                                           double acc[8]) {
   for (int f = 0; f < 8; ++f) acc[f] = 0.0;  // the spectral radius is positive: 0 is its identity too
   long long q = q0 + tid;
   if (q < q1) {  // the first partial is taken as it is, not added to zero
-    const double2 *pp = reinterpret_cast<const double2 *>(a.step_partials + q * kPartStride);
+    const double2 *pp = reinterpret_cast<const double2 *>(step_partials + q * kPartStride);
     const double2 x0 = pp[0], x1 = pp[1], x2 = pp[2], x3 = pp[3];
     acc[0] = x0.x; acc[1] = x0.y; acc[2] = x1.x; acc[3] = x1.y; acc[4] = x2.x; acc[5] = x2.y;
     if (a.mode == 4) { acc[6] = x3.x; acc[7] = x3.y; }
     q += NT;
   }
   for (; q < q1; q += NT) {
-    const double *pp = a.step_partials + q * kPartStride;
+    const double *pp = step_partials + q * kPartStride;
     for (int f = 0; f < 5; ++f) acc[f] += pp[f];
     acc[5] = fmax(acc[5], pp[5]);
     if (a.mode == 4) {
@@ -935,7 +1067,7 @@ __device__ __forceinline__ void load_slice(const BcArgs &a, long long q0, long l
     }
   }
   for (long long r = s0 + tid; r < s1; r += NT) {  // shell-kernel partials
-    const double *pp = a.step_partials + r * kPartStride;
+    const double *pp = step_partials + r * kPartStride;
     for (int f = 0; f < 5; ++f) acc[f] += pp[f];
     acc[5] = fmax(acc[5], pp[5]);
   }
@@ -955,48 +1087,79 @@ __device__ __forceinline__ double tree_slice(const double acc[8], double *sv, in
   return fin_tree<NT>(sv, tid >> 4, tid & 15);
 }
 
-template <class S, int NT>
-__device__ __forceinline__ void exchange_cta(const ExchArgs &a, int cta);
 template <class S>
 __device__ __forceinline__ int bc_cta(const BcArgs &a, int cta, bool reduce);
 
-// mid: [ncav][kFinSlices][8] slice totals; a.counter: per cavity, zero between launches
+// The x walls' Nusselt partial of one CTA: kBcThreads positions of one face
+// (its first threads; sh: a double per warp).  Returns the face's cavity.
 template <class S>
-__global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, double *mid) {
+__device__ __forceinline__ int nu_cta(const BcArgs &a, int cta, double *sh) {
+  const int tid = threadIdx.x;
+  int fi = 0;
+  for (int base = 0; base < a.nfaces; base += 32) {
+    const int l = base + (tid & 31);
+    const unsigned m = __ballot_sync(0xffffffffu, l < a.nfaces && a.faces[l].cta_begin <= cta);
+    if (m) fi = base + 31 - __clz(m);
+  }
+  const WallFace &F = a.faces[fi];
+  const BlockDev &B = a.blocks[F.block];
+  const CavConst &C = a.cc[F.cav];
+  const int high = F.face & 1, e = (cta - F.cta_begin) * kBcThreads + tid;
+  double flux = 0.0;
+  if (tid < kBcThreads && e < F.n1 * F.n2) {
+    const int j = e % F.n1 + 1, k = e / F.n1 + 1;
+    const S *q = (const S *)B.base[a.parity];
+    const long long N1 = node_index<S>(B, high ? B.nx : 1, j, k), N2 = high ? N1 - 1 : N1 + 1;
+    const double T1 = load_T<S>(q, B.fstride, N1), T2 = load_T<S>(q, B.fstride, N2);
+    const long long widx = (long long)(B.oy + j - 1) + (long long)C.gn[1] * (B.oz + k - 1);
+    flux = wall_flux(C, a.t_wall[C.wall_off + (high ? (long long)C.gn[1] * C.gn[2] : 0) + widx], T1, T2);
+    if (high) flux = -flux;
+  }
+  const double v = warp_sum(flux);
+  if ((tid & 31) == 0) sh[tid >> 5] = v;
+  __syncthreads();
+  if (tid == 0) {
+    double t = 0;
+    for (int q = 0; q < kBcThreads / 32; ++q) t += sh[q];
+    a.bc_partials[2LL * cta] = high ? 0.0 : t;
+    a.bc_partials[2LL * cta + 1] = high ? t : 0.0;
+  }
+  return F.cav;
+}
+
+template <class S>
+__global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a) {
   constexpr int NT = kFinThreads;
   __shared__ double sv[8 * NT];
   __shared__ double shm[kFinSlices * 8];
   __shared__ double shc[8];
-  __shared__ double sht[8];
-  __shared__ double sres[8];  // residual norms, Nusselt numbers, time: the step record's values
-  __shared__ double sdt;
-  __shared__ long long srec;
+  __shared__ double snu[NT / 32];
+  __shared__ double st_t[kGraphMax];
   __shared__ bool am_last;
   static_assert(kFinSlices * 8 <= NT && kFinSlices == 16, "one slice total per thread, 16 threads a field");
-  // the next step kernel (a programmatic dependent) may start its prologue now;
-  // it waits for this grid's completion before it reads the state advanced here
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int nsl = a.nslices, tid = threadIdx.x, f = tid >> 4, s = tid & 15;
-  int cav;
-  if (blockIdx.x >= a.ncav * nsl) {
-    const int c = blockIdx.x - a.ncav * nsl;
-    if (c >= a.wall_ctas) {
-      // the exchange of the new state's cut faces, beside the reductions
-      const ExchArgs x{a.blocks, a.cuts, a.ncuts, (double *)a.xbuf, a.parity};
-      exchange_cta<S, kFinThreads>(x, c - a.wall_ctas);
-      return;
-    }
-    // a wall CTA (FP64 step): its walls and Nusselt partial, then it arrives
-    // at the cavity's counter like a slice (thread 0 wrote the partial)
-    cav = bc_cta<S>(a, c, true);
-    if (tid == 0) __threadfence();
+  static_assert(kBcThreads == NT, "a wall position per thread");
+  chain_wait();
+  const int nsl = a.nslices, tid = threadIdx.x, f = tid >> 4, s = tid & 15, M = a.nsteps;
+  const int nslice = M * a.ncav * nsl;
+  const bool slice = (int)blockIdx.x < nslice;
+  int cav, m = M - 1, g = 0;  // cavity, step of the graph, slice
+  if (slice) {
+    m = blockIdx.x / (a.ncav * nsl);
+    const int r = blockIdx.x - m * a.ncav * nsl;
+    cav = r / nsl;
+    g = r - cav * nsl;
   } else {
-    cav = blockIdx.x / nsl;
+    // a wall CTA (FP64, the last step's state): its Nusselt partial (and
+    // walls), then it arrives like a slice (thread 0 wrote the partial)
+    const int c = blockIdx.x - nslice;
+    BcArgs b = a;
+    b.bc_partials += m * a.bc_stride;
+    cav = a.nu_only ? nu_cta<S>(b, c, snu) : bc_cta<S>(b, c, true);
+    if (tid == 0) __threadfence();
   }
   const CavConst &C = a.cc[cav];
   CavState &st = a.cs[cav];
-  const bool slice = blockIdx.x < a.ncav * nsl;
-  const int g = blockIdx.x - cav * nsl;
+  const bool last_step = m == M - 1;
   double acc[8];
   if (slice) {
     // slice bounds: the step partials' from the host's table; the wall and
@@ -1004,49 +1167,52 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, double *mid)
     // 32-bit arithmetic (counts far below 2^27)
     const unsigned nb = (a.mode == 4 || a.wall_ctas) ? 0u : (unsigned)(C.bc_end - C.bc_begin);
     const unsigned ns = (unsigned)(a.shell_end - a.shell_begin);
-    load_slice<NT>(a, C.slice_q[g], C.slice_q[g + 1], C.bc_begin + nb * g / nsl, C.bc_begin + nb * (g + 1) / nsl,
-                   a.shell_begin + ns * g / nsl, a.shell_begin + ns * (g + 1) / nsl, tid, acc);
+    load_slice<NT>(a, a.step_partials + m * a.part_stride, C.slice_q[g], C.slice_q[g + 1], C.bc_begin + nb * g / nsl,
+                   C.bc_begin + nb * (g + 1) / nsl, a.shell_begin + ns * g / nsl, a.shell_begin + ns * (g + 1) / nsl,
+                   tid, acc);
   }
-  // loads for whichever CTA of the cavity comes last, issued while the
-  // partials are in flight and first used after the reductions: the new
-  // state's centre pressure (at most 8 nodes, written by the step kernel) and
-  // the state it advances (written only by that CTA)
-  double cp = 0.0, st_t = 0.0, st_dt = 0.0;
-  long long st_step = 0;
-  int st_flags = 0;
-  if (a.mode != 1 && tid < C.ncentre) {
+  // loads for whichever CTA of the step comes last, issued while the partials
+  // are in flight: the final state's centre pressure (at most 8 nodes)
+  double cp = 0.0;
+  if (last_step && a.mode != 1 && tid < C.ncentre) {
     const BlockDev &B = a.blocks[C.centre_blk[tid]];
     cp = load_p<S>((const S *)B.base[a.parity], B.fstride, C.centre_off[tid]);
   }
-  if (tid == 0 || tid == 3) { st_step = st.step; st_flags = st.flags; }
-  if (tid == 2) { st_t = st.t; st_dt = st.dt; }
+  double *mid = a.mid + ((long long)m * a.ncav + cav) * kFinSlices * 8;
+  // the step's wall CTAs in this launch
+  const int nwall = !a.wall_ctas ? 0 : a.nu_only ? C.nu_end - C.nu_begin : C.bc_end - C.bc_begin;
+  const int arrivals = nsl + (last_step ? nwall : 0);
   if (slice) {
     const double tf = tree_slice<NT>(acc, sv, tid);
-    if (nsl == 1 && !a.wall_ctas) {
-      // the only CTA of the cavity: its totals go straight to the fold
+    if (arrivals == 1) {
+      // the only CTA of the step: its totals go straight to the fold
       if (s == 0) shm[f] = tf;
     } else if (s == 0) {
-      mid[((long long)cav * kFinSlices + g) * 8 + f] = tf;
+      mid[g * 8 + f] = tf;
       __threadfence();
     }
   }
-  const int nwall = a.wall_ctas ? C.bc_end - C.bc_begin : 0;  // the cavity's wall CTAs in this launch
-  if (nsl + nwall > 1) {
+  if (arrivals > 1) {
+    unsigned int *cnt = a.counter + m * a.ncav + cav;
     __syncthreads();
-    if (tid == 0) am_last = atomicAdd(a.counter + cav, 1u) == (unsigned int)(nsl + nwall) - 1u;
+    if (tid == 0) am_last = atomicAdd(cnt, 1u) == (unsigned int)arrivals - 1u;
     __syncthreads();
     if (!am_last) return;
     __threadfence();
+    if (tid == 0) *cnt = 0u;
     // the slice totals loaded in parallel
-    if (tid < nsl * 8) shm[tid] = mid[(long long)cav * kFinSlices * 8 + tid];
+    if (tid < nsl * 8) shm[tid] = mid[tid];
   }
   if (tid < 8) shc[tid] = cp;
   if (nwall) {
-    // the wall CTAs' Nusselt partials, thread-strided, into fields 6 and 7 of the tree
+    // the wall CTAs' Nusselt partials, thread-strided, into fields 6 and 7 of
+    // the tree (the graph's earlier steps' were left by the next step's launch)
     double h = 0.0, c = 0.0;
-    for (int q = C.bc_begin + tid; q < C.bc_xend; q += NT) {  // the other walls' partials are zeros
-      h += a.bc_partials[2LL * q];
-      c += a.bc_partials[2LL * q + 1];
+    const double *bp = a.bc_partials + m * a.bc_stride;
+    const int q0 = a.nu_only ? C.nu_begin : C.bc_begin, q1 = a.nu_only ? C.nu_end : C.bc_xend;
+    for (int q = q0 + tid; q < q1; q += NT) {  // the other walls' partials are zeros
+      h += bp[2LL * q];
+      c += bp[2LL * q + 1];
     }
     sv[6 * NT + tid] = h;
     sv[7 * NT + tid] = c;
@@ -1058,62 +1224,127 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, double *mid)
   for (int o = 1; o < nsl; o <<= 1) t = fin_comb(f, t, __shfl_xor_sync(0xffffffffu, t, o));
   if (nwall && f >= 6) t += fin_tree<NT>(sv, f, s);
   // one thread of each field group finishes its field (the FP64 chains run
-  // side by side): residual norms, dt, Nusselt numbers; threads 1 and 2 the
-  // centre pressure and the time
+  // side by side): residual norms, dt, Nusselt numbers; thread 1 the centre
+  StepResult &out = a.rec[(long long)m * a.ncav + cav];
+  const bool nonfin = s == 0 && f < 6 && (f == 5 || a.mode != 1) && !isfinite(t);
   if (s == 0) {
-    sht[f] = t;
-    if (f < 5 && a.mode != 1) {
-      const double r = sqrt(t * C.inv_nint);
-      st.res[f] = r;
-      sres[f] = r;
-    }
+    if (f < 5) out.res[f] = sqrt(t * C.inv_nint);
     if (f == 5) {
-      sdt = C.cfl / t;
-      st.dt = sdt;
+      out.dt = C.cfl / t;
+      if (last_step) {  // the next step starts from this state
+        st.smax = 0.0;
+        st.sfl = 0u;
+        if (cav == 0) *a.tile_counter = 0u;
+      }
     }
     if (f >= 6) {
       if (a.mode == 4) t *= C.wscale[f - 6];  // sums of 3 T_w - 4 T_1 + T_2 -> wall fluxes
-      const double nu = t * C.inv_nwall;
-      sres[f - 1] = nu;  // slots 5, 6 of the record's tail
-      if (f == 6) st.nu_hot = nu; else st.nu_cold = nu;
+      out.nu[f - 6] = t * C.inv_nwall;
     }
   }
-  if (tid == 1 && a.mode != 1) {
-    // centre pressure of the new state, lexicographic (k, j, i) order; the
-    // count is 1, 2, 4 or 8 (one or two nodes per axis), so the scaling is exact
-    double csum = 0.0;
-    for (int m = 0; m < C.ncentre; ++m) csum += shc[m];
-    st.c = csum * (C.ncentre == 8 ? 0.125 : C.ncentre == 4 ? 0.25 : C.ncentre == 2 ? 0.5 : 1.0);
+  if (tid == 1 && last_step && a.mode != 1) {  // the pending shift of the final state
+    st.c = centre_mean(C.ncentre, shc);
   }
-  if (tid == 2 && a.mode != 1) {  // the time after this step
-    st_t += st_dt;
-    st.t = st_t;
-    sres[7] = st_t;
+  const int bad = __syncthreads_or(nonfin);
+  if (tid == 0) out.bad = bad;
+  if (M > 1) {
+    // the cavity's last step to get here goes through all of them
+    __threadfence();
+    __syncthreads();
+    unsigned int *cnt = a.counter + M * a.ncav + cav;
+    if (tid == 0) {
+      am_last = atomicAdd(cnt, 1u) == (unsigned int)M - 1u;
+      if (am_last) *cnt = 0u;
+    }
+    __syncthreads();
+    if (!am_last) return;
+    __threadfence();
+  } else {
+    __syncthreads();
   }
-  if (tid == 3 && a.log && a.mode != 1) srec = (st_step % a.log_cap) * a.ncav + cav;  // this step's log record
+  if (a.mode == 1) {  // no step was taken
+    if (tid == 0) {
+      st.dt = st.dt0 = out.dt;
+      st.nu_hot = out.nu[0];
+      st.nu_cold = out.nu[1];
+      if (out.bad) atomicOr(&st.flags, 1);
+    }
+    return;
+  }
+  const StepResult *r = a.rec + cav;  // step q at r[q * ncav]
+  // the time after each step: the dt of a step is the one before it left
+  if (tid < M) sv[tid] = tid == 0 ? st.dt0 : __ldcg(&r[(long long)(tid - 1) * a.ncav].dt);
+  const unsigned badm = __ballot_sync(0xffffffffu, tid < M && __ldcg(&r[(long long)tid * a.ncav].bad));
+  const long long step0 = st.step;
+  const int flags0 = st.flags;
   __syncthreads();
-  if (tid != 0) return;
-  bool bad = !isfinite(sht[5]);
-  if (a.mode != 1) {
-    for (int q = 0; q < 5; ++q) bad = bad || !isfinite(sht[q]);
-    st_step += 1;
-    st.step = st_step;
+  if (tid == 0) {
+    double tt = st.t;
+    for (int q = 0; q < M; ++q) st_t[q] = tt += sv[q];
+    st.t = tt;
+    st.step = step0 + M;
+    if (badm) atomicOr(&st.flags, 1);
   }
-  if (bad) {  // atomic: a timed-out wait of the next step kernel may set bit 1 meanwhile
-    st_flags |= 1;
-    atomicOr(&st.flags, 1);
+  __syncthreads();
+  if (tid < M) {
+    const StepResult &x = r[(long long)tid * a.ncav];
+    double res[5];
+    for (int q = 0; q < 5; ++q) res[q] = __ldcg(&x.res[q]);
+    const double dt = __ldcg(&x.dt), nh = __ldcg(&x.nu[0]), nc = __ldcg(&x.nu[1]);
+    if (tid == M - 1) {
+      for (int q = 0; q < 5; ++q) st.res[q] = res[q];
+      st.dt = st.dt0 = dt;
+      st.nu_hot = nh;
+      st.nu_cold = nc;
+    }
+    if (a.log && M - tid <= a.log_cap) {  // each step's record, written to host memory
+      const long long step = step0 + tid + 1;
+      StepRecord &o = a.log[((step - 1) % a.log_cap) * a.ncav + cav];
+      o.step = step;
+      o.t = st_t[tid];
+      o.dt = dt;
+      for (int q = 0; q < 5; ++q) o.res[q] = res[q];
+      o.nu_hot = nh;
+      o.nu_cold = nc;
+      o.flags = flags0 | ((badm & (2u << tid) - 1u) ? 1 : 0);
+    }
   }
-  if (a.log && a.mode != 1) {  // this step's record, written to host memory
-    StepRecord &r = a.log[srec];
-    r.step = st_step;
-    r.t = sres[7];
-    r.dt = sdt;
-    for (int q = 0; q < 5; ++q) r.res[q] = sres[q];
-    r.nu_hot = sres[5];
-    r.nu_cold = sres[6];
-    r.flags = st_flags;
+}
+
+// ---------------------------------------------------------------------------
+// k_step_f64.  The first a.nnu CTAs take the x walls' Nusselt sums of the state
+// the step reads (d), the result of the step before.
+//
+// Persistent form: as many CTAs as fit on the GPU at once take tiles in
+// order from a counter, so the last round is short (one CTA per tile left a
+// partial wave of up to a third of the step on 152 SMs); the counter hands
+// out every block's coarse tiles before the fine tail tiles, and the next
+// tile is fetched while the current one is computed.  Partials stay indexed by
+// tile slot: the reductions do not depend on which CTA took a tile.
+template <int NT, bool FORM>
+__global__ void __launch_bounds__(NT) k_step_f64(StepArgs a, const __grid_constant__ BcArgs d) {
+  chain_wait();
+  if ((int)blockIdx.x < a.nnu) {
+    __shared__ double snu[NT / 32];
+    nu_cta<double>(d, blockIdx.x, snu);
+    return;
   }
-  a.counter[cav] = 0u;
+  float wfloor = -INFINITY;
+  int fcav = -1;
+  if (!a.tile_counter) {
+    step_tile_f64<NT, FORM>(a, blockIdx.x, wfloor, fcav);
+    return;
+  }
+  // the first tile of each CTA is its own index; the counter goes on from the grid's size
+  __shared__ int s_tile[2];
+  int tile = blockIdx.x - a.nnu;
+  for (int n = 0; tile < a.ntiles; n ^= 1) {
+    if (threadIdx.x == 0) s_tile[n] = (int)(gridDim.x - a.nnu + atomicAdd(a.tile_counter, 1u));
+    step_tile_f64<NT, FORM>(a, tile, wfloor, fcav);
+    __syncthreads();
+    tile = s_tile[n];
+  }
+  chain_trigger();
 }
 
 // k_bc: wall conditions of every wall face node and the Nusselt partials of
@@ -1127,9 +1358,6 @@ __device__ __forceinline__ int bc_cta(const BcArgs &a, int cta, bool reduce) {
   __shared__ double sh[kBcThreads / 32];
   const int tid = threadIdx.x, nwarps = blockDim.x / 32;
   int cav = 0;
-  if (cta == 0 && tid == 0 && a.tile_counter) *a.tile_counter = 0u;  // the step kernel has finished
-  if (cta == 0 && a.sfloor)
-    for (int c = tid; c < a.ncav; c += blockDim.x) a.sfloor[c] = 0u;
   double nu_h = 0.0, nu_c = 0.0;
   bool xwall = false, xhigh = false;
   if (a.nfaces > 0) {
@@ -1260,10 +1488,10 @@ __global__ void __launch_bounds__(256) k_unpack(ExchArgs a) {
 // The step's exchange, one CTA of NT threads per 256 face positions
 // (CutFace::cta_begin counts such CTAs): the ghost values k_pack followed by
 // k_unpack would write, copied straight from the sending block's layers (the
-// face buffer is packed only when asked for, by cavity_get_face_buffer).  Run
-// by the finalise kernel's extra CTAs beside its reductions, so it is written
-// for latency: the face found by a warp-wide search, every value of the
-// thread's positions loaded before the first store.
+// face buffer is packed only when asked for, by cavity_get_face_buffer).  It
+// stands between two steps, so it is written for latency: the face found by a
+// warp-wide search, every value of the thread's positions loaded before the
+// first store.
 template <class S, int NT>
 __device__ __forceinline__ void exchange_cta(const ExchArgs &a, int cta) {
   static_assert(256 % NT == 0, "positions per thread");
@@ -1311,6 +1539,51 @@ __device__ __forceinline__ void exchange_cta(const ExchArgs &a, int cta) {
     }
 #pragma unroll
     for (int v = 0; v < NA - NP; ++v) g[(NP + v) * fd + gv[r]] = x[r][2 * NP + v];
+  }
+}
+
+// Between two steps of a graph: what the next one waits for.  One CTA per cavity
+// takes dt from the maximum and the centre shift from the new state (and clears
+// the step's words); a.faces' CTAs exchange the cut faces; the rest (FP64,
+// large cavities) store the new state's walls.  2 us for an undivided cavity
+// (4-6 with an exchange or walls) where a finalise took 8-19.
+//
+// The one CTA lets the next step's launch start at once (the step before is
+// complete by then: its tile look-ups and first plane loads run beside this),
+// the others when they are done: CTAs of a step placed beside the exchange's
+// are spread unevenly over the SMs (FP32-mixed 128^3 in 2x2x2 blocks 77 us a
+// step, against 64).
+constexpr int kBetweenThreads = 128;
+template <class S>
+__global__ void __launch_bounds__(kBetweenThreads) k_between(ExchArgs a, BcArgs b, int ncut) {
+  chain_wait();
+  if ((int)blockIdx.x >= b.ncav) {
+    const int c = blockIdx.x - b.ncav;
+    if (c < ncut) exchange_cta<S, kBetweenThreads>(a, c);
+    else bc_cta<S>(b, c - ncut, false);
+    return;
+  }
+  chain_trigger();
+  __shared__ double shc[kMaxCentre];
+  const CavConst &C = b.cc[blockIdx.x];
+  CavState &st = b.cs[blockIdx.x];
+  const int tid = threadIdx.x;
+  if (tid < kMaxCentre) {
+    double v = 0.0;
+    if (tid < C.ncentre) {
+      const BlockDev &B = a.blocks[C.centre_blk[tid]];
+      v = load_p_l2<S>((const S *)B.base[a.parity], B.fstride, C.centre_off[tid]);
+    }
+    shc[tid] = v;
+    __syncwarp(0xffu);
+    if (tid == 0) st.c = centre_mean(C.ncentre, shc);
+  }
+  if (tid == 32) {
+    const double t = __ldcg(&st.smax);
+    st.dt = C.cfl / t;
+    st.smax = 0.0;
+    st.sfl = 0u;
+    if (blockIdx.x == 0) *b.tile_counter = 0u;
   }
 }
 

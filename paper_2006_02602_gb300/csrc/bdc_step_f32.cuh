@@ -61,7 +61,7 @@ struct StepF32Args {
   const BlockDev *blocks;
   int nblocks;
   const CavConst *cc;
-  CavState *cs;               // dt and c read; flags bit 1 set on a timed-out wait
+  CavState *cs;               // dt and c read, the maximum taken; flags bit 1 set on a timed-out wait
   const CUtensorMap *maps;    // [block][parity][pressure box, other box], in global memory
   double *partials;           // [slot][kPartStride]: 5 rate sums, spectral max, 2 Nusselt sums
   int parity;
@@ -69,7 +69,7 @@ struct StepF32Args {
   int ncoarse;                // coarse tiles of all blocks (scheduling indices below it)
   long long wait_cycles;      // limit of each bounded mbarrier wait (kWaitCycles)
   int withhold_plane;         // -1; a test of the timeout path sets a plane index whose load is never issued
-  int ghosts_late;            // cut faces: the previous step's finalise launch writes the ghost layers
+  int ghosts_late;            // cut faces: the launch before (k_between) writes the ghost layers
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -447,12 +447,13 @@ __device__ __forceinline__ void f32_spectral_max(const F32K<float> &K, float bou
 // CTA partials: rate sums FP32 per thread and per warp tree, FP64 across
 // warps (fixed order); Nusselt sums FP64 from the column sums on.  Slots:
 // 5 rate sums, spectral max, hot and cold sums of 3 T_w - 4 T_1 + T_2; the
-// per-cavity reduction (k_finalize) reads them in a fixed order.
+// per-cavity reduction (k_finalize) reads them in a fixed order; the maximum
+// also goes to the cavity's state, for the next step's dt.
 // `xwall`: the tile touches an isothermal x wall (uniform over the CTA); only
 // then can a thread hold Nusselt sums, and the FP64 warp sums run.
 template <int NT>
-__device__ __forceinline__ void f32_partials(double *partials, int cta, int tid, float s0, float s1, float s2,
-                                             float s3, float s4, float smax, double nuh, double nuc, bool xwall) {
+__device__ __forceinline__ void f32_partials(double *partials, CavState &st, int cta, int tid, float s0, float s1,
+                                             float s2, float s3, float s4, float smax, double nuh, double nuc, bool xwall) {
   __shared__ double red[NT / 32][8];
   const int lane = tid & 31, wid = tid >> 5;
   const float w0s = warp_sum_f(s0), w1s = warp_sum_f(s1), w2s = warp_sum_f(s2), w3s = warp_sum_f(s3);
@@ -467,6 +468,7 @@ __device__ __forceinline__ void f32_partials(double *partials, int cta, int tid,
     double acc = red[0][tid];
     for (int q = 1; q < NT / 32; ++q) acc = (tid == 5) ? fmax(acc, red[q][tid]) : acc + red[q][tid];
     partials[(long long)cta * kPartStride + tid] = acc;
+    if (tid == 5) step_max(st, acc);
   }
 }
 
@@ -689,8 +691,8 @@ __device__ __forceinline__ void f32q_clear(F32QAcc &acc) {
 
 // The tile's partials (every thread of the CTA calls it: a CTA reduction).
 template <int NT>
-__device__ __forceinline__ void f32q_finish(double *partials, int tile, int tid, const F32Tile &T, const F32QCol &c,
-                                            const F32QAcc &acc) {
+__device__ __forceinline__ void f32q_finish(double *partials, CavState &st, int tile, int tid, const F32Tile &T,
+                                            const F32QCol &c, const F32QAcc &acc) {
   double nuh = 0.0, nuc = 0.0;
   if (c.nus) {
     const double t0 = pair_value(acc.ch.x, acc.cl.x), t1 = c.act1 ? pair_value(acc.ch.y, acc.cl.y) : 0.0;
@@ -700,8 +702,9 @@ __device__ __forceinline__ void f32q_finish(double *partials, int tile, int tid,
     nuh = c.wh0 * t0 + c.wh1 * t1 + (c.hot_next ? wall_t : 0.0);
     nuc = c.wc0 * t0 + c.wc1 * t1 + (c.cold_next ? wall_c : 0.0);
   }
-  f32_partials<NT>(partials, tile, tid, vadd(acc.s0.x, acc.s0.y), vadd(acc.s1.x, acc.s1.y), vadd(acc.s2.x, acc.s2.y),
-                   vadd(acc.s3.x, acc.s3.y), vadd(acc.s4.x, acc.s4.y), acc.smax, nuh, nuc, T.wxl || T.wxh);
+  f32_partials<NT>(partials, st, tile, tid, vadd(acc.s0.x, acc.s0.y), vadd(acc.s1.x, acc.s1.y),
+                   vadd(acc.s2.x, acc.s2.y), vadd(acc.s3.x, acc.s3.y), vadd(acc.s4.x, acc.s4.y), acc.smax, nuh, nuc,
+                   T.wxl || T.wxh);
 }
 
 // The tile's prologue reads once planes 0 .. 3 (z = k0-2 .. k0+1) are resident
@@ -769,9 +772,9 @@ __global__ void __launch_bounds__(kF32TX / 2 * TY, 512 / (kF32TX / 2 * TY)) k_st
   };
   if (tid == 0) {
     if (a.ghosts_late && f32_reads_ghosts<TY>(B, T)) {
-      // the boxes reach a ghost layer, which the previous step's finalise
-      // launch (this launch's programmatic predecessor, if any) writes
-      asm volatile("griddepcontrol.wait;" ::: "memory");
+      // the boxes reach a ghost layer, which the launch between the steps
+      // (this launch's programmatic predecessor, if any) writes
+      chain_wait();
       asm volatile("fence.proxy.async.global;" ::: "memory");
     }
     for (; issued < min(R, T.nplanes); ++issued) issue(issued);
@@ -792,10 +795,10 @@ __global__ void __launch_bounds__(kF32TX / 2 * TY, 512 / (kF32TX / 2 * TY)) k_st
     if (!bad) f32q_prologue_plane<NT, TY>(pl, slot(pl), T, c, tid, acc);
   }
   bad = __syncthreads_or(bad);
-  // a programmatic dependent of the previous step's finalise: only now are its
-  // dt, centre shift and reads of the partials complete (nothing global was
-  // read from the state it writes, nor written, before this point)
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // a programmatic dependent of the launch between the steps: only now are dt
+  // and the centre shift complete (nothing it writes was read, nor anything
+  // written, before this point)
+  chain_wait();
   const F32K<float2> K = f32_consts<float2>(C, a.cs[B.cav]);
   const F32K<float> K1 = f32_consts<float>(C, a.cs[B.cav]);
   if (!bad && tid == 0) {
@@ -829,7 +832,8 @@ __global__ void __launch_bounds__(kF32TX / 2 * TY, 512 / (kF32TX / 2 * TY)) k_st
     }
     __syncthreads();
   }
-  f32q_finish<NT>(a.partials, T.slot, tid, T, c, acc);
+  chain_trigger();
+  f32q_finish<NT>(a.partials, a.cs[B.cav], T.slot, tid, T, c, acc);
 }
 
 // Spectral-radius partials of the current state (no update), with the step

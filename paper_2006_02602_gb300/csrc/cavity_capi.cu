@@ -102,6 +102,11 @@ struct AdjointStore {
   double J = 0.0;
 };
 
+// Steps of one graph: a graph ends with one finalise launch for all of its
+// steps, so a long run is mostly 16-step graphs.
+constexpr int kGraphs = 3;
+constexpr int kGraphSteps[kGraphs] = {1, 4, kGraphMax};
+
 struct cavity {
   int dev = 0;
   bool u_ref_auto = true;  // u_ref follows Ra (default)
@@ -136,25 +141,28 @@ struct cavity {
   int nblocks = 0;
   std::vector<BlockDev> hb;
   std::vector<WallFace> hwall;
+  std::vector<WallFace> hxwall;   // the x walls alone, with their own CTA numbers (Nusselt sums after an FP64 step)
+  int n_nu = 0;                   // their CTAs
   std::vector<CutFace> hcut;
   long long xbuf_elems = 0;
   int n_step = 0, n_bc = 0, n_cut = 0;
   int nslices = kFinSlices;  // k_finalize CTAs per cavity: about 128 step partials a slice
+  int form_walls = 1;  // FP64: walls formed where the step reads them (0: stored between the steps)
   int n_coarse = 0;  // FP64 step tiles of KC planes (scheduled before the fine ones)
   int part_cap = 0;  // step partials allocated (CTAs)
 
   BlockDev *d_blocks = nullptr;
   CavConst *d_cc = nullptr;
   CavState *d_cs = nullptr;
-  WallFace *d_wall = nullptr;
+  WallFace *d_wall = nullptr, *d_xwall = nullptr;
   CutFace *d_cut = nullptr;
   CUtensorMap *d_maps = nullptr;
   double *d_step_part = nullptr, *d_bc_part = nullptr, *d_twall = nullptr, *d_stage = nullptr;
-  double *d_fin = nullptr;  // k_finalize slice totals [ncav][kFinSlices][8]
+  double *d_fin = nullptr;  // k_finalize slice totals [kGraphMax][ncav][kFinSlices][8]
+  StepResult *d_rec = nullptr;  // [kGraphMax][ncav]
   StepRecord *d_log = nullptr;  // the step log (device address of caller-owned host memory), or null
   long long log_cap = 0;
-  unsigned int *d_counter = nullptr;  // [ncav] k_bc CTAs done per cavity, the FP64 step's tile counter,
-                                      // [ncav] the FP64 step's dt-filter floors
+  unsigned int *d_counter = nullptr;  // the FP64 step's tile counter, then BcArgs::counter
   int nsm = 0;                        // SMs of the device
   int persist_ctas = 0;               // CTAs of the persistent FP64 step kernel that fit on the GPU
   void *d_fields = nullptr, *d_xbuf = nullptr;
@@ -163,8 +171,8 @@ struct cavity {
 
   int parity = 0;
   long long steps_taken = 0;
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};   // one step from parity 0 / 1
-  cudaGraphExec_t graph2[2] = {nullptr, nullptr};  // two steps from parity 0 / 1 (programmatic edge between them)
+  cudaGraphExec_t graph[kGraphs][2] = {};  // kGraphSteps[q] steps from parity 0 / 1
+  cudaStream_t capture = nullptr;          // the graphs are captured on it
   std::string err;
 };
 
@@ -253,6 +261,7 @@ void assign_tiles(cavity *h) {
   if (!h->f32) {
     for (const BlockDev &B : h->hb) planes += (long long)ceil_div((long long)B.nx * B.ny, h->tx * h->ty) * B.nz;
     h->kc = planes >= 64LL * h->nsm ? 8 : 4;
+    h->form_walls = h->kc == 4;  // (why the line lies there: step_tile_f64)
   }
   int tile = 0, coarse = 0, fine = 0;
   for (int c = 0; c < h->ncav; ++c) h->hcc[c].tile_begin = -1;
@@ -400,6 +409,18 @@ int build_layout(cavity *h) {
     C.bc_end = bc;
     if (w.face / 2 == 0) C.bc_xend = bc;
   }
+  h->hxwall.clear();
+  h->n_nu = 0;
+  for (int c = 0; c < h->ncav; ++c) h->hcc[c].nu_begin = -1;
+  for (WallFace w : h->hwall) {
+    if (w.face / 2 != 0) continue;
+    CavConst &C = h->hcc[w.cav];
+    w.cta_begin = h->n_nu;
+    if (C.nu_begin < 0) C.nu_begin = h->n_nu;
+    h->n_nu += ceil_div((long long)w.n1 * w.n2, kBcThreads);
+    C.nu_end = h->n_nu;
+    h->hxwall.push_back(w);
+  }
   for (CutFace &c : h->hcut) {
     c.cta_begin = cut;
     c.buf_off = xoff;
@@ -474,6 +495,12 @@ cudaError_t f32_set_smem(int p, int ty, int r) {
   return cudaErrorInvalidValue;
 }
 
+// the FP64 step kernel of a tile of 32 * ty nodes
+auto f64_kernel(int ty, bool form_walls) {
+  if (ty == 4) return form_walls ? k_step_f64<kTX * 4, true> : k_step_f64<kTX * 4, false>;
+  return form_walls ? k_step_f64<kTX * 8, true> : k_step_f64<kTX * 8, false>;
+}
+
 int upload_tables(cavity *h) {
   CK(cudaMemcpyAsync(h->d_blocks, h->hb.data(), sizeof(BlockDev) * h->nblocks, cudaMemcpyHostToDevice, h->stream));
   CK(cudaMemcpyAsync(h->d_cc, h->hcc.data(), sizeof(CavConst) * h->ncav, cudaMemcpyHostToDevice, h->stream));
@@ -487,8 +514,9 @@ int ensure_partials(cavity *h) {
   CK(cudaStreamSynchronize(h->stream));
   if (h->d_step_part) cudaFree(h->d_step_part);
   h->d_step_part = nullptr;
-  CK(cudaMalloc(&h->d_step_part, sizeof(double) * kPartStride * std::max(1, need)));
-  h->part_cap = need;
+  // one set per step of a graph: all are reduced at its end
+  CK(cudaMalloc(&h->d_step_part, kGraphMax * sizeof(double) * kPartStride * std::max(1, need)));
+  h->part_cap = std::max(1, need);
   return CAVITY_OK;
 }
 
@@ -507,25 +535,28 @@ int alloc_device(cavity *h) {
   CK(cudaMalloc(&h->d_cs, sizeof(CavState) * h->ncav));
   CK(cudaMemsetAsync(h->d_cs, 0, sizeof(CavState) * h->ncav, h->stream));
   CK(cudaMalloc(&h->d_wall, sizeof(WallFace) * std::max<size_t>(1, h->hwall.size())));
+  CK(cudaMalloc(&h->d_xwall, sizeof(WallFace) * std::max<size_t>(1, h->hxwall.size())));
   CK(cudaMalloc(&h->d_cut, sizeof(CutFace) * std::max<size_t>(1, h->hcut.size())));
   int rc = ensure_partials(h);
   if (rc != CAVITY_OK) return rc;
-  CK(cudaMalloc(&h->d_bc_part, sizeof(double) * 2 * std::max(1, h->n_bc)));
-  CK(cudaMalloc(&h->d_fin, sizeof(double) * 8 * kFinSlices * h->ncav));
-  CK(cudaMalloc(&h->d_counter, sizeof(unsigned int) * (2 * h->ncav + 1)));
-  CK(cudaMemsetAsync(h->d_counter, 0, sizeof(unsigned int) * (2 * h->ncav + 1), h->stream));
+  // the wall kernel's Nusselt partials, or (FP64) the x walls' of every step of a graph
+  CK(cudaMalloc(&h->d_bc_part, sizeof(double) * 2 * std::max(std::max(1, h->n_bc), h->f32 ? 0 : kGraphMax * h->n_nu)));
+  CK(cudaMalloc(&h->d_fin, sizeof(double) * kGraphMax * 8 * kFinSlices * h->ncav));
+  CK(cudaMalloc(&h->d_rec, sizeof(StepResult) * kGraphMax * h->ncav));
+  const size_t counter_bytes = sizeof(unsigned int) * (1 + (size_t)(kGraphMax + 1) * h->ncav);
+  CK(cudaMalloc(&h->d_counter, counter_bytes));
+  CK(cudaMemsetAsync(h->d_counter, 0, counter_bytes, h->stream));
   {
     int per_sm = 0;
-    if (h->ty == 4)
-      CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_f64<kTX * 4>, kTX * 4, 0));
-    else
-      CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_f64<kTX * 8>, kTX * 8, 0));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f64_kernel(h->ty, h->form_walls), kTX * h->ty, 0));
     h->persist_ctas = std::max(1, h->nsm * per_sm);
   }
   CK(cudaMalloc(&h->d_twall, sizeof(double) * std::max<size_t>(1, h->twall.size())));
   if (h->xbuf_elems > 0) CK(cudaMalloc(&h->d_xbuf, h->esize * (size_t)h->xbuf_elems));
   if (!h->hwall.empty())
     CK(cudaMemcpyAsync(h->d_wall, h->hwall.data(), sizeof(WallFace) * h->hwall.size(), cudaMemcpyHostToDevice, h->stream));
+  if (!h->hxwall.empty())
+    CK(cudaMemcpyAsync(h->d_xwall, h->hxwall.data(), sizeof(WallFace) * h->hxwall.size(), cudaMemcpyHostToDevice, h->stream));
   if (!h->hcut.empty())
     CK(cudaMemcpyAsync(h->d_cut, h->hcut.data(), sizeof(CutFace) * h->hcut.size(), cudaMemcpyHostToDevice, h->stream));
   if (h->f32) {
@@ -554,25 +585,29 @@ int upload_consts(cavity *h) {
 // ---------------------------------------------------------------------------
 // kernel launches
 
-StepArgs step_args(cavity *h, int parity, int mode) {
+// partials of step `s` of a graph
+double *step_partials(cavity *h, int s) { return h->d_step_part + (size_t)s * h->part_cap * kPartStride; }
+
+StepArgs step_args(cavity *h, int parity, int mode, int s) {
   StepArgs a;
   a.blocks = h->d_blocks; a.nblocks = h->nblocks; a.cc = h->d_cc; a.cs = h->d_cs;
-  a.partials = h->d_step_part; a.parity = parity; a.mode = mode;
-  a.tile_counter = h->d_counter + h->ncav; a.ntiles = h->n_step; a.local_dt = h->local_dt;
-  a.sfloor = h->d_counter + h->ncav + 1;
+  a.partials = step_partials(h, s); a.parity = parity; a.mode = mode;
+  a.tile_counter = mode == 0 ? h->d_counter : nullptr;
+  a.ntiles = h->n_step; a.local_dt = h->local_dt;
   a.ncoarse = h->n_coarse;
   a.skip_shell = 0;
+  a.nnu = 0;
   return a;
 }
 
-StepF32Args step_f32_args(cavity *h, int parity) {
+StepF32Args step_f32_args(cavity *h, int parity, int s) {
   StepF32Args a;
   a.blocks = h->d_blocks; a.nblocks = h->nblocks; a.cc = h->d_cc; a.cs = h->d_cs;
-  a.maps = h->d_maps; a.partials = h->d_step_part; a.parity = parity; a.local_dt = h->local_dt;
+  a.maps = h->d_maps; a.partials = step_partials(h, s); a.parity = parity; a.local_dt = h->local_dt;
   a.ncoarse = h->n_coarse;
   a.wait_cycles = h->wait_cycles;
   a.withhold_plane = h->withhold_plane;
-  a.ghosts_late = h->n_cut > 0;  // the finalise after each step writes the ghost layers
+  a.ghosts_late = h->n_cut > 0;
   return a;
 }
 
@@ -582,17 +617,39 @@ BcArgs bc_args(cavity *h, int parity, int mode) {
   a.faces = h->d_wall;
   a.nfaces = (int)h->hwall.size();
   a.cc = h->d_cc; a.cs = h->d_cs; a.ncav = h->ncav;
-  a.step_partials = h->d_step_part; a.bc_partials = h->d_bc_part; a.counter = h->d_counter;
-  a.tile_counter = h->d_counter + h->ncav;
-  a.sfloor = h->d_counter + h->ncav + 1;
+  a.step_partials = h->d_step_part; a.bc_partials = h->d_bc_part; a.counter = h->d_counter + 1;
+  a.tile_counter = h->d_counter;
   a.t_wall = h->d_twall; a.parity = parity; a.mode = mode;
   a.shell_begin = a.shell_end = 0;
   a.log = mode == 1 || mode == 3 ? nullptr : h->d_log;  // after a step (modes 0, 4): the step log
   a.log_cap = h->log_cap;
-  a.cuts = nullptr; a.ncuts = 0; a.xbuf = nullptr;
   a.nslices = h->nslices;
   a.wall_ctas = 0;
+  a.nu_only = 0;
+  a.nsteps = 1;
+  a.part_stride = (long long)h->part_cap * kPartStride;
+  a.bc_stride = 2LL * h->n_nu;
+  a.mid = h->d_fin;
+  a.rec = h->d_rec;
   return a;
+}
+
+// The finalise of a graph of `nsteps` steps that leaves its state in buffer set
+// `parity`, and its CTAs.  In the FP64 form the x walls' Nusselt sums have CTAs
+// of their own (the FP32 step kernel leaves them in its partials): those of
+// the final state here, of the others in the next step's launch.
+BcArgs fin_args(cavity *h, int parity, int nsteps, int *ctas) {
+  BcArgs b = bc_args(h, parity, h->f32 ? 4 : 0);
+  b.nsteps = nsteps;
+  *ctas = nsteps * h->ncav * h->nslices;
+  if (!h->f32) {
+    b.faces = h->d_xwall;
+    b.nfaces = (int)h->hxwall.size();
+    b.nu_only = 1;
+    b.wall_ctas = h->n_nu;
+    *ctas += h->n_nu;
+  }
+  return b;
 }
 
 ExchArgs exch_args(cavity *h, int parity) {
@@ -602,52 +659,57 @@ ExchArgs exch_args(cavity *h, int parity) {
   return a;
 }
 
-// The persistent FP64 step kernel of the handle's tile size (32 * ty threads,
-// as many CTAs as fit on the GPU at once).
-void launch_step_f64(cavity *h, const StepArgs &a) {
-  const int grid = std::min(h->n_step, h->persist_ctas);
-  if (h->ty == 4)
-    k_step_f64<kTX * 4><<<grid, kTX * 4, 0, h->stream>>>(a);
-  else
-    k_step_f64<kTX * 8><<<grid, kTX * 8, 0, h->stream>>>(a);
+// A launch, as a programmatic dependent of the launch before it in the same
+// stream capture if `pdl` (a step, a k_between or a finalise: each waits for its
+// predecessor's completion before it touches anything that one writes).
+template <class K, class... A>
+cudaError_t launch_chained(cavity *h, bool pdl, K kernel, int grid, dim3 block, size_t smem, A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = h->stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// `after_finalise`: the launch directly follows, in the same stream capture,
-// the finalise of the previous step (the second step of a two-step graph).
-// The FP32 step kernel is then launched as a programmatic dependent: its
-// prologue (TMA loads of the state, which the previous step kernel completed
-// before that finalise started) overlaps the finalise, and it waits for the
-// finalise before reading dt and the centre shift.  With cut faces that
-// finalise also exchanges the ghost layers, so a tile whose boxes reach a
-// ghost layer waits for it before its first load.  Every other predecessor
-// (an unpack writing ghost layers, a state upload, a copy) gets a plain
-// launch.
-void launch_step_kernel(cavity *h, int parity, bool after_finalise = false) {
-  if (h->f32) {
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(h->n_step);
-    cfg.stream = h->stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = after_finalise ? 1 : 0;
-    const StepF32Args sa = step_f32_args(h, parity);
-#define BDC_LAUNCH(P, TY, R)                                                     \
-  if (h->f32_p == P && h->ty == TY && h->f32_r == R) {                            \
-    cfg.blockDim = dim3(kF32TX / 2, TY);                                          \
-    cfg.dynamicSmemBytes = f32_smem_bytes(TY, R);                                 \
-    cudaLaunchKernelEx(&cfg, f32_kernel<P, TY, R>(), sa);                         \
+// The persistent FP64 step kernel of the handle's tile size (32 * ty threads,
+// as many CTAs as fit on the GPU at once, after the Nusselt sums' ones); without
+// a tile counter one CTA per tile.
+cudaError_t launch_step_f64(cavity *h, const StepArgs &a, const BcArgs &d, bool pdl) {
+  const int grid = a.nnu + (a.tile_counter ? std::min(h->n_step, h->persist_ctas) : h->n_step);
+  return launch_chained(h, pdl, f64_kernel(h->ty, h->form_walls), grid, dim3(kTX * h->ty), 0, a, d);
+}
+
+// The kernel of step `s` of a graph, reading buffer set `parity`.  From the
+// second step on it is a programmatic dependent of the k_between before it; the
+// first gets a plain launch.
+cudaError_t launch_step_kernel(cavity *h, int parity, int s) {
+  if (!h->f32) {
+    StepArgs a = step_args(h, parity, 0, s);
+    int ctas = 0;
+    BcArgs d = fin_args(h, parity, 1, &ctas);
+    if (s > 0) {
+      a.nnu = h->n_nu;
+      d.bc_partials += (s - 1) * d.bc_stride;
+    }
+    return launch_step_f64(h, a, d, s > 0);
   }
-    BDC_F32_VARIANTS(BDC_LAUNCH)
+  const StepF32Args a = step_f32_args(h, parity, s);
+#define BDC_LAUNCH(P, TY, R)                                                                               \
+  if (h->f32_p == P && h->ty == TY && h->f32_r == R)                                                       \
+    return launch_chained(h, s > 0, f32_kernel<P, TY, R>(), h->n_step, dim3(kF32TX / 2, TY), f32_smem_bytes(TY, R), a);
+  BDC_F32_VARIANTS(BDC_LAUNCH)
 #undef BDC_LAUNCH
-  } else {
-    launch_step_f64(h, step_args(h, parity, 0));
-  }
+  return cudaErrorInvalidValue;
 }
 
 void launch_spectral(cavity *h) {
-  const StepArgs sa = step_args(h, h->parity, 1);
+  const StepArgs sa = step_args(h, h->parity, 1, 0);
   if (h->f32) {
 #define BDC_SPEC(P, TY, R)                                                                                       \
   if (h->f32_p == P && h->ty == TY && h->f32_r == R)                                                             \
@@ -655,51 +717,47 @@ void launch_spectral(cavity *h) {
     BDC_F32_VARIANTS(BDC_SPEC)
 #undef BDC_SPEC
   } else {
-    launch_step_f64(h, sa);
+    launch_step_f64(h, sa, BcArgs{}, false);
   }
 }
 
-// mode 0: after a step; mode 1: state refresh; 3: walls only.  The walls
-// kernel (k_bc) writes the walls and the Nusselt partials, k_finalize reduces
-// the partials and advances the state; after an FP64 step the wall CTAs run
-// inside the finalise launch, arriving at each cavity's completion counter
-// with the finalise CTAs, and the last to arrive folds their partials.  The
-// FP32 step kernel applies the walls where it reads them and leaves the
-// Nusselt sums in its own partials, so after its steps only k_finalize
-// runs.  After a step of a decomposed
-// cavity the finalise launch carries one more CTA per 256 cut-face
-// positions, which exchange the new state's cut faces (Section 4.5 pack and
-// unpack in one pass) beside the reductions: one launch after the step
-// instead of a finalise beside a pack and an unpack.
-void launch_bc_kernel(cavity *h, int parity, int mode) {
+// Walls of the state in buffer set `parity` stored (no sums): the steps form
+// them where they read them, so the stored ones are those of the last refresh.
+void launch_walls(cavity *h, int parity) {
+  const BcArgs b = bc_args(h, parity, 3);
+  if (h->f32) k_bc<float><<<h->n_bc, kBcThreads, 0, h->stream>>>(b);
+  else k_bc<double><<<h->n_bc, kBcThreads, 0, h->stream>>>(b);
+}
+
+// A state refresh (no step): walls with the Nusselt partials, then the
+// reductions, dt among them.
+void launch_refresh(cavity *h, int parity) {
+  const BcArgs b = bc_args(h, parity, 1);
   const int nfin = h->ncav * h->nslices;
-  BcArgs b = bc_args(h, parity, h->f32 && mode == 0 ? 4 : mode);
-  int grid = nfin;
-  if (mode == 0 && !h->f32) {  // the FP64 walls and their Nusselt partials in the same launch
-    b.wall_ctas = h->n_bc;
-    grid += h->n_bc;
-  }
-  if (mode == 0 && h->n_cut > 0) {
-    b.cuts = h->d_cut;
-    b.ncuts = (int)h->hcut.size();
-    b.xbuf = h->d_xbuf;
-    grid += h->n_cut;
-  }
   if (h->f32) {
-    if (mode == 0) {
-      k_finalize<float><<<grid, kFinThreads, 0, h->stream>>>(b, h->d_fin);
-      return;
-    }
-    k_bc<float><<<h->n_bc, kBcThreads, 0, h->stream>>>(bc_args(h, parity, mode));
-    if (mode != 3) k_finalize<float><<<nfin, kFinThreads, 0, h->stream>>>(bc_args(h, parity, mode), h->d_fin);
+    k_bc<float><<<h->n_bc, kBcThreads, 0, h->stream>>>(b);
+    k_finalize<float><<<nfin, kFinThreads, 0, h->stream>>>(b);
   } else {
-    if (mode == 0) {
-      k_finalize<double><<<grid, kFinThreads, 0, h->stream>>>(b, h->d_fin);
-      return;
-    }
-    k_bc<double><<<h->n_bc, kBcThreads, 0, h->stream>>>(bc_args(h, parity, mode));
-    if (mode != 3) k_finalize<double><<<nfin, kFinThreads, 0, h->stream>>>(b, h->d_fin);
+    k_bc<double><<<h->n_bc, kBcThreads, 0, h->stream>>>(b);
+    k_finalize<double><<<nfin, kFinThreads, 0, h->stream>>>(b);
   }
+}
+
+cudaError_t launch_finalize(cavity *h, int parity, int nsteps, bool pdl) {
+  int ctas = 0;
+  const BcArgs b = fin_args(h, parity, nsteps, &ctas);
+  if (h->f32) return launch_chained(h, pdl, k_finalize<float>, ctas, dim3(kFinThreads), 0, b);
+  return launch_chained(h, pdl, k_finalize<double>, ctas, dim3(kFinThreads), 0, b);
+}
+
+// What the step after the one that left its state in buffer set `parity` waits
+// for (dt, the centre shift, ghost layers, stored walls).
+cudaError_t launch_between(cavity *h, int parity, bool pdl) {
+  const ExchArgs x = exch_args(h, parity);
+  const BcArgs b = bc_args(h, parity, 3);
+  const int grid = h->ncav + h->n_cut + (h->f32 || h->form_walls ? 0 : h->n_bc);
+  if (h->f32) return launch_chained(h, pdl, k_between<float>, grid, dim3(kBetweenThreads), 0, x, b, h->n_cut);
+  return launch_chained(h, pdl, k_between<double>, grid, dim3(kBetweenThreads), 0, x, b, h->n_cut);
 }
 
 void launch_pack(cavity *h, int parity, cudaStream_t s = nullptr) {
@@ -746,29 +804,34 @@ int launch_step_overlapped(cavity *h, int parity) {
   launch_unpack(h, parity ^ 1, h->side);
   CK(cudaGetLastError());
   CK(cudaEventRecord(h->ev_exch, h->side));
-  StepArgs st = step_args(h, parity, 0);
+  StepArgs st = step_args(h, parity, 0, 0);
   st.skip_shell = 1;
-  launch_step_f64(h, st);
-  CK(cudaGetLastError());
+  CK(launch_step_f64(h, st, BcArgs{}, false));
   CK(cudaStreamWaitEvent(h->stream, h->ev_exch, 0));
   // the finalise with the walls (and their Nusselt partials) in the same launch
   BcArgs ba = bc_args(h, parity ^ 1, 0);
   ba.wall_ctas = h->n_bc;
   ba.shell_begin = h->n_step;
   ba.shell_end = (long long)h->n_step + h->n_shell;
-  k_finalize<double><<<h->ncav * h->nslices + h->n_bc, kFinThreads, 0, h->stream>>>(ba, h->d_fin);
+  k_finalize<double><<<h->ncav * h->nslices + h->n_bc, kFinThreads, 0, h->stream>>>(ba);
   CK(cudaGetLastError());
   return CAVITY_OK;
 }
 
-// one explicit step reading buffer set `parity`, leaving the new state in parity ^ 1
-// (the exchange of a decomposed cavity runs inside the finalise launch)
-int launch_step(cavity *h, int parity, bool after_finalise = false) {
-  if (h->overlap) return launch_step_overlapped(h, parity);
-  launch_step_kernel(h, parity, after_finalise);
-  CK(cudaGetLastError());
-  launch_bc_kernel(h, parity ^ 1, 0);
-  CK(cudaGetLastError());
+// nsteps explicit steps from buffer set `parity` (captured into one graph):
+// the steps one after another, then one finalise launch for all of them.
+int launch_steps(cavity *h, int parity, int nsteps) {
+  for (int s = 0; s < nsteps; ++s, parity ^= 1) {
+    if (h->overlap) {
+      const int rc = launch_step_overlapped(h, parity);
+      if (rc != CAVITY_OK) return rc;
+      continue;
+    }
+    CK(launch_step_kernel(h, parity, s));
+    // (the state a graph leaves has its ghost layers and stored walls, too)
+    if (s < nsteps - 1 || h->n_cut > 0 || (!h->f32 && !h->form_walls)) CK(launch_between(h, parity ^ 1, true));
+    if (s == nsteps - 1) CK(launch_finalize(h, parity ^ 1, nsteps, true));
+  }
   return CAVITY_OK;
 }
 
@@ -776,41 +839,35 @@ int launch_step(cavity *h, int parity, bool after_finalise = false) {
 int refresh_state(cavity *h) {
   launch_spectral(h);
   CK(cudaGetLastError());
-  launch_bc_kernel(h, h->parity, 1);
+  launch_refresh(h, h->parity);
   CK(cudaGetLastError());
   return launch_exchange(h, h->parity);
 }
 
 void drop_graphs(cavity *h) {
-  for (auto &g : h->graph)
-    if (g) { cudaGraphExecDestroy(g); g = nullptr; }
-  for (auto &g : h->graph2)
-    if (g) { cudaGraphExecDestroy(g); g = nullptr; }
+  for (auto &q : h->graph)
+    for (auto &g : q)
+      if (g) { cudaGraphExecDestroy(g); g = nullptr; }
 }
 
-int build_graphs(cavity *h) {
-  drop_graphs(h);
-  if (h->n_cut > 0) CK(ensure_side(h));
+// The graphs of kGraphSteps[q] steps, built when a call first needs them (every
+// setter that changes a launch drops them), captured on a stream of the
+// handle's own.
+int ensure_graph(cavity *h, int q) {
+  if (h->graph[q][1]) return CAVITY_OK;
+  if (h->overlap) CK(ensure_side(h));
+  if (!h->capture) CK(cudaStreamCreateWithFlags(&h->capture, cudaStreamNonBlocking));
   for (int par = 0; par < 2; ++par) {
+    if (h->graph[q][par]) continue;
     cudaGraph_t g = nullptr;
-    CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    const int rc = launch_step(h, par);
-    const cudaError_t e = cudaStreamEndCapture(h->stream, &g);
+    CK(cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal));
+    std::swap(h->stream, h->capture);
+    const int rc = launch_steps(h, par, kGraphSteps[q]);
+    std::swap(h->stream, h->capture);
+    const cudaError_t e = cudaStreamEndCapture(h->capture, &g);
     if (rc != CAVITY_OK) { if (g) cudaGraphDestroy(g); return rc; }
     CK(e);
-    const cudaError_t e2 = cudaGraphInstantiate(&h->graph[par], g, 0);
-    cudaGraphDestroy(g);
-    CK(e2);
-  }
-  for (int par = 0; par < 2; ++par) {
-    cudaGraph_t g = nullptr;
-    CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    int rc = launch_step(h, par);
-    if (rc == CAVITY_OK) rc = launch_step(h, par ^ 1, true);
-    const cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-    if (rc != CAVITY_OK) { if (g) cudaGraphDestroy(g); return rc; }
-    CK(e);
-    const cudaError_t e2 = cudaGraphInstantiate(&h->graph2[par], g, 0);
+    const cudaError_t e2 = cudaGraphInstantiate(&h->graph[q][par], g, 0);
     cudaGraphDestroy(g);
     CK(e2);
   }
@@ -830,7 +887,8 @@ int retile(cavity *h, int p, int ty, int kc, int r) {
   if (rc == CAVITY_OK) rc = encode_maps(h);
   if (rc != CAVITY_OK) return rc;
   CK(f32_set_smem(p, ty, r));
-  return build_graphs(h);
+  drop_graphs(h);
+  return CAVITY_OK;
 }
 
 int init_state(cavity *h) {
@@ -933,7 +991,7 @@ void release(cavity *h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   drop_graphs(h);
   void *ptrs[] = {h->d_fields, h->d_blocks, h->d_cc, h->d_cs, h->d_wall, h->d_cut, h->d_step_part,
-                  h->d_bc_part, h->d_counter, h->d_twall, h->d_xbuf, h->d_stage, h->d_maps, h->d_fin, h->d_shell};
+                  h->d_bc_part, h->d_counter, h->d_twall, h->d_xbuf, h->d_stage, h->d_maps, h->d_fin, h->d_rec, h->d_shell, h->d_xwall};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   AdjointStore &A = h->adj;
@@ -943,6 +1001,7 @@ void release(cavity *h) {
     if (p) cudaFree(p);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   if (h->side) cudaStreamDestroy(h->side);
+  if (h->capture) cudaStreamDestroy(h->capture);
   if (h->ev_shell) cudaEventDestroy(h->ev_shell);
   if (h->ev_exch) cudaEventDestroy(h->ev_exch);
   for (cudaEvent_t e : h->adj_ev) cudaEventDestroy(e);
@@ -1026,7 +1085,6 @@ int create_common(const cavity_desc *descs, const cavity_params *params, int n, 
     if (rc == CAVITY_OK) rc = alloc_device(h);
     if (rc == CAVITY_OK) rc = upload_consts(h);
     if (rc == CAVITY_OK) rc = init_state(h);
-    if (rc == CAVITY_OK) rc = build_graphs(h);
     if (rc == CAVITY_OK && cudaStreamSynchronize(h->stream) != cudaSuccess) rc = CAVITY_ERR_CUDA;
   }
   if (rc != CAVITY_OK) {
@@ -1181,16 +1239,14 @@ int cavity_set_wall_temperature(cavity_t *h, int wall, const double *host, size_
 int cavity_step(cavity_t *h, int nsteps) {
   if (!h || nsteps < 0) return CAVITY_ERR_INVALID_ARG;
   DeviceGuard g(h->dev);
-  int s = 0;
-  for (; s + 2 <= nsteps; s += 2) {  // two steps per graph: the parity comes back
-    CK(cudaGraphLaunch(h->graph2[h->parity], h->stream));
-    h->steps_taken += 2;
-  }
-  if (s < nsteps) {
-    CK(cudaGraphLaunch(h->graph[h->parity], h->stream));
-    h->parity ^= 1;
-    h->steps_taken += 1;
-  }
+  for (int q = kGraphs - 1; q >= 0; --q)
+    for (; nsteps >= kGraphSteps[q]; nsteps -= kGraphSteps[q]) {
+      const int rc = ensure_graph(h, q);
+      if (rc != CAVITY_OK) return rc;
+      CK(cudaGraphLaunch(h->graph[q][h->parity], h->stream));
+      h->parity ^= kGraphSteps[q] & 1;
+      h->steps_taken += kGraphSteps[q];
+    }
   return CAVITY_OK;
 }
 
@@ -1233,7 +1289,8 @@ int cavity_set_step_log(cavity_t *h, cavity_step_record *host, long long capacit
   CK(cudaStreamSynchronize(h->stream));
   h->d_log = dev;
   h->log_cap = host ? capacity : 0;
-  return build_graphs(h);  // the finalise launches in the graphs carry the log
+  drop_graphs(h);  // the finalise launches in the graphs carry the log
+  return CAVITY_OK;
 }
 
 int cavity_step_log_alloc(long long records, cavity_step_record **out) {
@@ -1370,6 +1427,7 @@ int cavity_get_block_array(cavity_t *h, int block, int field, double *host, size
   DeviceGuard g(h->dev);
   int rc = ensure_stage(h, count);
   if (rc != CAVITY_OK) return rc;
+  if (!h->f32) launch_walls(h, h->parity);  // (the FP32-mixed form returns them as last refreshed)
   if (h->f32) k_copy_block<float><<<ceil_div((long long)n, 256), 256, 0, h->stream>>>(h->d_blocks, block, h->parity, field, h->d_stage);
   else k_copy_block<double><<<ceil_div((long long)n, 256), 256, 0, h->stream>>>(h->d_blocks, block, h->parity, field, h->d_stage);
   CK(cudaGetLastError());
@@ -1572,6 +1630,10 @@ int cavity_adjoint_forward(cavity_t *h, int nsteps, int ckpt, double *J) {
     CK(cudaMemcpyAsync(A.seg_mem + (size_t)s * set_bytes, h->hb[0].base[h->parity], set_bytes,
                        cudaMemcpyDeviceToDevice, h->stream));
   CK(cudaMemsetAsync(A.scal, 0, sizeof(double) * kScCount, h->stream));
+  {
+    const int rc = ensure_graph(h, 0);
+    if (rc != CAVITY_OK) return rc;
+  }
   for (int n = 0; n < nsteps; ++n) {
     if (n % ckpt == 0) {
       const int c = n / ckpt;
@@ -1579,7 +1641,7 @@ int cavity_adjoint_forward(cavity_t *h, int nsteps, int ckpt, double *J) {
                          cudaMemcpyDeviceToDevice, h->stream));
       CK(cudaMemcpyAsync(A.ckpt_cs + c, h->d_cs, sizeof(CavState), cudaMemcpyDeviceToDevice, h->stream));
     }
-    CK(cudaGraphLaunch(h->graph[h->parity], h->stream));
+    CK(cudaGraphLaunch(h->graph[0][h->parity], h->stream));
     h->parity ^= 1;
     h->steps_taken += 1;
     k_adj_acc_nusselt<<<1, 1, 0, h->stream>>>(h->d_cs, A.scal);
@@ -1632,7 +1694,8 @@ int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *gr
     CK(cudaEventCreate(&e));
     h->adj_ev.push_back(e);
   }
-  int rc = CAVITY_OK;
+  int rc = ensure_graph(h, 0);
+  if (rc != CAVITY_OK) return rc;
   auto slot = [&](int s) { return (void *)(A.seg_mem + (size_t)s * A.set_bytes); };
   for (int c = A.ncp - 1; c >= 0 && rc == CAVITY_OK; --c) {
     const int s0 = c * A.ckpt, s1 = std::min(s0 + A.ckpt, A.nsteps);
@@ -1648,20 +1711,21 @@ int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *gr
                                              h->f32 ? A.seg_maps + 2 * (s - s0) : nullptr, slot(s - s0),
                                              slot(s - s0 + 1));
         CK(cudaGetLastError());
-        CK(cudaGraphLaunch(h->graph[0], h->stream));
+        CK(cudaGraphLaunch(h->graph[0][0], h->stream));
       }
     }
-    if (h->f32) {
-      // the FP32-mixed step forms p's and T's wall values where it reads
-      // them: write them into every stored state of the segment, one launch
+    {
+      // the step forms p's and T's wall values where it reads them: write
+      // them into every stored state of the segment, one launch
       BcArgs ba = bc_args(h, 0, 3);
       ba.blocks = A.seg_blocks;
       ba.faces = A.seg_faces;
       ba.nfaces = (int)h->hwall.size() * (s1 - s0);
-      ba.tile_counter = nullptr;
-      ba.sfloor = nullptr;
-      k_bc<float><<<h->n_bc * (s1 - s0), kBcThreads, 0, h->stream>>>(ba);
+      if (h->f32) k_bc<float><<<h->n_bc * (s1 - s0), kBcThreads, 0, h->stream>>>(ba);
+      else k_bc<double><<<h->n_bc * (s1 - s0), kBcThreads, 0, h->stream>>>(ba);
       CK(cudaGetLastError());
+    }
+    if (h->f32) {
       // the argmax of every state of the segment's spectral bound, one launch
       k_adj_argmax_seg<float><<<dim3(A.nparts, s1 - s0), 256, 0, h->stream>>>(A.seg_blocks, h->hcc[0], a.g, A.argpart);
       CK(cudaGetLastError());
@@ -1747,9 +1811,10 @@ int cavity_set_overlap(cavity_t *h, int on) {
     CK(cudaMemcpy(h->d_shell, h->hshell.data(), sizeof(ShellFace) * h->hshell.size(), cudaMemcpyHostToDevice));
     CK(ensure_side(h));
   }
+  if (h->overlap) launch_walls(h, h->parity);  // this schedule's shell kernel reads the stored walls
   const int rc = ensure_partials(h);
-  if (rc != CAVITY_OK) return rc;
-  return build_graphs(h);
+  drop_graphs(h);
+  return rc;
 }
 
 int cavity_set_time_stepping(cavity_t *h, int mode) {
@@ -1757,7 +1822,8 @@ int cavity_set_time_stepping(cavity_t *h, int mode) {
   DeviceGuard g(h->dev);
   CK(cudaStreamSynchronize(h->stream));
   h->local_dt = mode == CAVITY_DT_LOCAL;
-  return build_graphs(h);  // the kernels' arguments are part of the captured graphs
+  drop_graphs(h);  // the kernels' arguments are part of the captured graphs
+  return CAVITY_OK;
 }
 
 int cavity_time_kernels(cavity_t *h, int nsteps, double ms[4]) {
@@ -1770,14 +1836,15 @@ int cavity_time_kernels(cavity_t *h, int nsteps, double ms[4]) {
   for (int s = 0; s < nsteps && rc == CAVITY_OK; ++s) {
     const int par = h->parity;
     cudaEventRecord(ev[0], h->stream);
-    launch_step_kernel(h, par);
+    cudaError_t e = launch_step_kernel(h, par, 0);
     cudaEventRecord(ev[1], h->stream);
-    launch_bc_kernel(h, par ^ 1, 0);
+    if (e == cudaSuccess && (h->n_cut > 0 || (!h->f32 && !h->form_walls))) e = launch_between(h, par ^ 1, false);
+    if (e == cudaSuccess) e = launch_finalize(h, par ^ 1, 1, false);
     cudaEventRecord(ev[2], h->stream);
-    // (the exchange runs inside the finalise launch: nothing here)
     cudaEventRecord(ev[3], h->stream);
     cudaEventRecord(ev[4], h->stream);
-    cudaError_t e = cudaEventSynchronize(ev[4]);
+    const cudaError_t es = cudaEventSynchronize(ev[4]);
+    if (e == cudaSuccess) e = es;
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { rc = fail(h, CAVITY_ERR_CUDA, cudaGetErrorString(e)); break; }
     for (int q = 0; q < 4; ++q) {
@@ -1854,7 +1921,8 @@ int cavity_test_wait_timeout(cavity_t *h, long long wait_cycles, int withhold_pl
   CK(cudaStreamSynchronize(h->stream));
   h->wait_cycles = wait_cycles;
   h->withhold_plane = withhold_plane;
-  return build_graphs(h);
+  drop_graphs(h);
+  return CAVITY_OK;
 }
 
 int cavity_measure_fp64_peak(int device, double *tflops) {

@@ -162,7 +162,8 @@ extern "C" CAVITY_API int cavity_step_block_noalloc(const double *q_in, double *
   const int ntiles = B.tiles_x * B.tiles_z;  // at most the limit's count: 256 consecutive nodes fill no fewer tiles
   a.partials = d_part; a.parity = 0; a.mode = 0; a.ntiles = ntiles;
   a.ncoarse = ntiles;
-  k_step_f64<kTX * kTY><<<ntiles, kTX * kTY, 0, st>>>(a);
+  // walls and ghosts read as the caller filled them
+  k_step_f64<kTX * kTY, false><<<ntiles, kTX * kTY, 0, st>>>(a, BcArgs{});
   if (cudaGetLastError() != cudaSuccess) return CAVITY_ERR_CUDA;
   k_noalloc_reduce<<<1, 256, 0, st>>>(d_part, ntiles, d_cc, out6);
   if (cudaGetLastError() != cudaSuccess) return CAVITY_ERR_CUDA;
