@@ -59,7 +59,7 @@ struct BlockDev {
   int kc, kf;
   void *base[2];         // buffer sets (field f at base + f * fstride)
 };
-constexpr int kFineKC32 = 8;  // kf of the FP32 form
+constexpr int kFineKC32 = 8;  // the largest kf of the FP32 form
 
 struct CavConst {
   double h[3], ih[3], ih2[3], ihh[3];

@@ -39,7 +39,7 @@
 namespace bdc {
 
 constexpr int kF32TX = 32;                       // tile width: 16 threads x 2 nodes
-constexpr int kF32TY = 8, kF32KC = 32, kF32R = 4;  // default shape: tile height, z chunk, ring depth
+constexpr int kF32TY = 8, kF32R = 4;             // default shape: tile height, ring depth (chunk depth: by size)
 constexpr int kF32HX = 4;                        // x halo of both boxes left of the tile (2 needed)
 constexpr int kF32BX = kF32TX + 8;               // box width: 40 floats, 160 bytes
 constexpr int kF32NA = 7;                        // p_hi, p_lo, u, v, w, T_hi, T_lo

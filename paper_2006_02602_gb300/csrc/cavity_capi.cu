@@ -126,6 +126,7 @@ struct cavity {
   int na = 5;                     // stored arrays per buffer set
   int np = 1;                     // pressure arrays
   int tx = kTX, ty = kTY, kc = 8;
+  bool f32_auto = true;           // the FP32 step kernel's chunk depth by size (f32_chunk)
   int f32_r = 0;                  // ring depth of the FP32 step kernel
   int f32_p = 1;                  // nodes per thread along x of the FP32 step kernel
   int local_dt = 0;               // CAVITY_DT_LOCAL: each node at its own stable step
@@ -254,10 +255,48 @@ int check_desc(const cavity_desc &d) {
 // last 8 of 128 only) -> 384; the other side of the line: 4 planes at 256^3
 // 2835 against 2798 us, 8 planes at 64^3 80 against 66.5.
 //
-// FP32: kFineKC32-plane tail chunks, only in blocks deeper than one chunk (a
-// shallower block is one chunk: the ring's fill is paid per tile).
+// FP32: tail chunks of at most kFineKC32 planes, only in blocks deeper than one
+// chunk (a shallower block is one chunk: the ring's fill is paid per tile).
+int f32_zsplit(int nz, int kc) { return nz <= kc ? nz : (nz - 1) / kc * kc; }
+int f32_tiles_z(int nz, int kc) {
+  if (nz <= kc) return 1;
+  return (nz - 1) / kc + ceil_div(nz - f32_zsplit(nz, kc), std::min(kFineKC32, kc));
+}
+
+// Chunk depth of the FP32 form where neither the caller's autotuner nor the
+// environment has set one.  A tile sweeps its planes one after another (1 us a
+// plane alone on an SM), so a cavity whose tiles all run at once takes as long
+// as its deepest tile and the tiles beside it: measured on 32^3 .. 128^3 within
+// 1-2 us, a step is 7.4 + kc + (n - 1) (2.2 + 0.24 kc) us with n tiles on the
+// fullest SM, and the depth is the one that makes this least.  Four tiles run at
+// once on an SM; a fifth costs 8 us more (128^3: 41 us at 16 planes and four
+// tiles, 49 at 12 and five) but still beats deeper ones (128^3 in 2x2x2 blocks:
+// 58 us at 16 planes, 60 at 24).  Larger cavities: 24 planes up to 150 tile planes an
+// SM (160^3: 66 us, 69 at 32, 71 at 16), 64 beyond (batch of 64: 230 us, 235 at
+// 32; 256^3: 211 at either).  With 32 planes at all sizes: 32^3 40 us (8.4 now),
+// 64^3 39 (14.5), 96x80x72 38 (19.5), 128^3 52 (41).
+int f32_chunk(const cavity *h) {
+  double best = 1e300;
+  int kc = 0;
+  long long planes = 0;
+  for (const BlockDev &B : h->hb) planes += (long long)ceil_div(B.nx, h->tx) * ceil_div(B.ny, h->ty) * B.nz;
+  for (int k : {1, 2, 4, 6, 8, 12, 16}) {
+    long long tiles = 0;
+    for (const BlockDev &B : h->hb) tiles += (long long)ceil_div(B.nx, h->tx) * ceil_div(B.ny, h->ty) * f32_tiles_z(B.nz, k);
+    const int n = ceil_div(tiles, h->nsm);
+    if (n > 5) continue;
+    const double us = 7.4 + k + (n - 1) * (2.2 + 0.24 * k) + (n > 4 ? 8.0 : 0.0);
+    if (us < best) {
+      best = us;
+      kc = k;
+    }
+  }
+  return kc ? kc : planes <= 150LL * h->nsm ? 24 : 64;
+}
+
 void assign_tiles(cavity *h) {
   long long planes = 0;
+  if (h->f32 && h->f32_auto) h->kc = f32_chunk(h);
   if (!h->f32) {
     for (const BlockDev &B : h->hb) planes += (long long)ceil_div((long long)B.nx * B.ny, h->tx * h->ty) * B.nz;
     h->kc = planes >= 64LL * h->nsm ? 8 : 4;
@@ -270,10 +309,9 @@ void assign_tiles(cavity *h) {
     if (h->f32) {
       B.tiles_x = ceil_div(B.nx, h->tx);
       B.tiles_y = ceil_div(B.ny, h->ty);
-      B.kf = kFineKC32;
-      B.tiles_zc = (B.nz - 1) / h->kc;
-      if (B.nz <= h->kc) B.tiles_zc = 1;
-      B.zsplit = std::min(B.nz, B.tiles_zc * h->kc);
+      B.kf = std::min(kFineKC32, h->kc);
+      B.zsplit = f32_zsplit(B.nz, h->kc);
+      B.tiles_zc = B.nz <= h->kc ? 1 : B.zsplit / h->kc;
     } else {
       B.tiles_x = ceil_div((long long)B.nx * B.ny, h->tx * h->ty);
       B.tiles_y = 1;
@@ -881,6 +919,7 @@ int retile(cavity *h, int p, int ty, int kc, int r) {
   h->ty = ty;
   h->kc = kc;
   h->f32_r = r;
+  h->f32_auto = false;
   assign_tiles(h);
   int rc = ensure_partials(h);
   if (rc == CAVITY_OK) rc = upload_tables(h);
@@ -1055,7 +1094,6 @@ int create_common(const cavity_desc *descs, const cavity_params *params, int n, 
   if (h->f32) {
     h->tx = kF32TX;
     h->ty = kF32TY;
-    h->kc = kF32KC;
     h->f32_r = kF32R;
     h->f32_p = 3;
     // shape override for tuning sweeps: BDC_F32_TILE="TY,KC,R[,P]" (a compiled shape)
@@ -1067,6 +1105,7 @@ int create_common(const cavity_desc *descs, const cavity_params *params, int n, 
         h->kc = kc;
         h->f32_r = r;
         h->f32_p = p;
+        h->f32_auto = false;
       }
     }
   }
