@@ -495,7 +495,7 @@ def measure_adjoint(m, torch, rank, world, local, stream):
             "forward_ms_per_step": 1e3 * fwd / steps, "backward_ms_per_step": 1e3 * bwd / steps,
             "J": J, "dJ_dRa": gra, "grad_wall_norm": float(np.linalg.norm(g)), "clocks": clk.summary(), "status": rc,
             "autotune": tuned,
-            "roofline": {"kernel": "k_adj_gather (reverse of the rates, FP32 gather form)", "bound": "hbm",
+            "roofline": {"kernel": "k_adj_sweep (reverse of a step, FP32)", "bound": "hbm",
                          "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm if hbm else None,
                          "traffic": None, "kernel_ms": gather_ms, "bytes_per_point": ADJ_BYTES_PER_POINT,
                          "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)"},

@@ -301,10 +301,10 @@ CAVITY_API int cavity_adjoint_forward(cavity_t *h, int nsteps, int ckpt, double 
 CAVITY_API int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *grad_ra);
 
 /* Measurement: mean duration in ms, from CUDA events on the handle's stream
- * around every launch, of the dominant kernel of the last
- * cavity_adjoint_backward: the reverse of the rates (k_adj_gather after an
- * FP32-mixed forward, k_adj_rates after an FP64 one), one launch per reverse
- * step.  CAVITY_ERR_INVALID_ARG before the first reverse sweep. */
+ * around the reverse steps of every checkpoint segment, of the dominant kernel
+ * of the last cavity_adjoint_backward: the reverse of a step (k_adj_sweep), one
+ * launch per reverse step.  CAVITY_ERR_INVALID_ARG before the first reverse
+ * sweep. */
 CAVITY_API int cavity_adjoint_kernel_ms(cavity_t *h, double *ms);
 
 /* Interior/shell split with overlap (Section 4.7): when on, each step first

@@ -169,6 +169,7 @@ struct CavState {
   double smax;
   unsigned int sfl, pad2;
   double dt0;        // dt as the last finalise left it (dt itself moves on within a graph)
+  double nu_sum;     // sum of nu_hot over the steps (the adjoint's forward run zeroes it)
 };
 
 struct StepRecord {   // one step's record in the host-memory step log (the C ABI's cavity_step_record)
@@ -940,10 +941,12 @@ struct BcArgs {
   long long part_stride, bc_stride;
   double *mid;                // [nsteps][ncav][kFinSlices][8] slice totals
   StepResult *rec;            // [nsteps][ncav]
+  double *dt_out;             // k_between: the next step's dt goes here, too (null: nowhere)
   StepRecord *log;            // after a step: the step log (host memory), or null
   long long log_cap;          // its records per cavity
   int mode;                   // 0 after a step, 1 after init / set_fields,
-                              // 3 walls only (k_bc), no reductions,
+                              // 3 walls only (k_bc), no reductions, 5 the same with
+                              //   the constant walls in both buffer sets,
                               // 4 after an FP32 step (k_finalize only): Nusselt
                               //   sums in the step partials
 };
@@ -1283,6 +1286,9 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a) {
     for (int q = 0; q < M; ++q) st_t[q] = tt += sv[q];
     st.t = tt;
     st.step = step0 + M;
+    double sum = st.nu_sum;
+    for (int q = 0; q < M; ++q) sum += __ldcg(&r[(long long)q * a.ncav].nu[0]);
+    st.nu_sum = sum;
     if (badm) atomicOr(&st.flags, 1);
   }
   __syncthreads();
@@ -1377,7 +1383,7 @@ __device__ __forceinline__ int bc_cta(const BcArgs &a, int cta, bool reduce) {
       if (e < F.n1 * F.n2) {
         const BlockDev &B = a.blocks[F.block];
         apply_wall<S>(B, a.cc[F.cav], (S *)B.base[a.parity], F.face, e % F.n1 + 1, e / F.n1 + 1, a.t_wall,
-                        nu_h, nu_c, a.mode == 1 ? (S *)B.base[a.parity ^ 1] : nullptr);
+                      nu_h, nu_c, a.mode == 1 || a.mode == 5 ? (S *)B.base[a.parity ^ 1] : nullptr);
       }
     }
   }
@@ -1404,7 +1410,7 @@ __device__ __forceinline__ int bc_cta(const BcArgs &a, int cta, bool reduce) {
 
 template <class S>
 __global__ void __launch_bounds__(kBcThreads) k_bc(BcArgs a) {
-  bc_cta<S>(a, blockIdx.x, a.mode != 3);
+  bc_cta<S>(a, blockIdx.x, a.mode != 3 && a.mode != 5);
 }
 
 // ---------------------------------------------------------------------------
@@ -1580,7 +1586,9 @@ __global__ void __launch_bounds__(kBetweenThreads) k_between(ExchArgs a, BcArgs 
   }
   if (tid == 32) {
     const double t = __ldcg(&st.smax);
-    st.dt = C.cfl / t;
+    const double dt = C.cfl / t;
+    st.dt = dt;
+    if (b.dt_out) *b.dt_out = dt;
     st.smax = 0.0;
     st.sfl = 0u;
     if (blockIdx.x == 0) *b.tile_counter = 0u;

@@ -80,27 +80,30 @@ std::vector<F32Shape> f32_shapes() {
 
 // checkpoints and work arrays of the discrete adjoint (single-block cavity)
 struct AdjointStore {
-  int nsteps = 0, ckpt = 0, ncp = 0, nparts = 0;
+  int nsteps = 0, run_ckpt = 0;  // of the last forward run
+  int ckpt = 0, ncp = 0;         // as allocated
+  int layout = -1;             // the tiling the segment's tables were made for
   size_t set_bytes = 0;        // one buffer set of the block
   char *ckpt_mem = nullptr;    // ncp buffer sets: the state at steps 0, ckpt, 2 ckpt, ...
   CavState *ckpt_cs = nullptr;  // their scalars (device)
   char *seg_mem = nullptr;     // ckpt buffer sets: one recomputed segment
-  BlockDev *seg_blocks = nullptr;   // ckpt block descriptors, slot s's state as buffer set 0 (walls pass)
+  BlockDev *seg_blocks = nullptr;   // ckpt block descriptors: slot s as buffer set 0, slot s + 1 as buffer set 1
   WallFace *seg_faces = nullptr;    // the block's wall faces once per slot (one walls launch per segment)
   CUtensorMap *seg_maps = nullptr;  // FP32 form: the step kernel's two maps of every slot
   char *final_mem = nullptr;   // the state after the forward run
   CavState final_cs{};
   int final_parity = 0;
   long long final_steps = 0;
-  void *X = nullptr, *Yt = nullptr, *Q = nullptr;  // adjoint arrays: FP64 (FP64 forward) or FP32 (FP32-mixed)
+  void *X = nullptr, *Q = nullptr;  // adjoint arrays: FP64 (FP64 forward) or FP32 (FP32-mixed)
   double *thetabar = nullptr, *scal = nullptr, *argpart = nullptr;
-  double *gpart = nullptr;     // per-CTA node sums of the FP32 gather (3 per CTA)
-  double *dts = nullptr;       // dt of every step (device)
-  unsigned int *cnt = nullptr; // finished CTAs of k_adj_pre (zero between launches)
-  BlockDev *block = nullptr;   // descriptor of a segment slot (wall pass of FP32 states)
+  double *gpart = nullptr;     // per-CTA node sums of the sweep (4 per CTA)
+  double *dts = nullptr;       // dt of every step of a segment (device)
+  unsigned int *cnt = nullptr; // finished CTAs of k_adj_sweep (zero between launches)
+  int kc = 0, ctas = 0;        // the sweep's chunk depth and CTAs
   bool have_forward = false;
   double J = 0.0;
 };
+constexpr int kAdjParts = 2 * 152;  // argmax partials of a state
 
 // Steps of one graph: a graph ends with one finalise launch for all of its
 // steps, so a long run is mostly 16-step graphs.
@@ -111,8 +114,9 @@ struct cavity {
   int dev = 0;
   bool u_ref_auto = true;  // u_ref follows Ra (default)
   AdjointStore adj;
-  std::vector<cudaEvent_t> adj_ev;  // two per reverse step: around the rates' reverse kernel
-  double adj_rates_ms = 0.0;        // its mean duration in the last reverse sweep
+  std::vector<cudaEvent_t> adj_ev;  // two per segment: around its reverse steps' launches
+  double adj_rates_ms = 0.0;        // mean duration of one in the last reverse sweep
+  int layout = 0;                   // counts assign_tiles calls
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   int ncav = 1;
@@ -295,6 +299,7 @@ int f32_chunk(const cavity *h) {
 }
 
 void assign_tiles(cavity *h) {
+  h->layout += 1;
   long long planes = 0;
   if (h->f32 && h->f32_auto) h->kc = f32_chunk(h);
   if (!h->f32) {
@@ -667,6 +672,7 @@ BcArgs bc_args(cavity *h, int parity, int mode) {
   a.nsteps = 1;
   a.part_stride = (long long)h->part_cap * kPartStride;
   a.bc_stride = 2LL * h->n_nu;
+  a.dt_out = nullptr;
   a.mid = h->d_fin;
   a.rec = h->d_rec;
   return a;
@@ -723,6 +729,15 @@ cudaError_t launch_step_f64(cavity *h, const StepArgs &a, const BcArgs &d, bool 
   return launch_chained(h, pdl, f64_kernel(h->ty, h->form_walls), grid, dim3(kTX * h->ty), 0, a, d);
 }
 
+cudaError_t launch_step_f32(cavity *h, const StepF32Args &a, bool pdl) {
+#define BDC_LAUNCH(P, TY, R)                                                                                   \
+  if (h->f32_p == P && h->ty == TY && h->f32_r == R)                                                           \
+    return launch_chained(h, pdl, f32_kernel<P, TY, R>(), h->n_step, dim3(kF32TX / 2, TY), f32_smem_bytes(TY, R), a);
+  BDC_F32_VARIANTS(BDC_LAUNCH)
+#undef BDC_LAUNCH
+  return cudaErrorInvalidValue;
+}
+
 // The kernel of step `s` of a graph, reading buffer set `parity`.  From the
 // second step on it is a programmatic dependent of the k_between before it; the
 // first gets a plain launch.
@@ -737,13 +752,7 @@ cudaError_t launch_step_kernel(cavity *h, int parity, int s) {
     }
     return launch_step_f64(h, a, d, s > 0);
   }
-  const StepF32Args a = step_f32_args(h, parity, s);
-#define BDC_LAUNCH(P, TY, R)                                                                               \
-  if (h->f32_p == P && h->ty == TY && h->f32_r == R)                                                       \
-    return launch_chained(h, s > 0, f32_kernel<P, TY, R>(), h->n_step, dim3(kF32TX / 2, TY), f32_smem_bytes(TY, R), a);
-  BDC_F32_VARIANTS(BDC_LAUNCH)
-#undef BDC_LAUNCH
-  return cudaErrorInvalidValue;
+  return launch_step_f32(h, step_f32_args(h, parity, s), s > 0);
 }
 
 void launch_spectral(cavity *h) {
@@ -912,6 +921,18 @@ int ensure_graph(cavity *h, int q) {
   return CAVITY_OK;
 }
 
+int run_steps(cavity *h, int nsteps) {
+  for (int q = kGraphs - 1; q >= 0; --q)
+    for (; nsteps >= kGraphSteps[q]; nsteps -= kGraphSteps[q]) {
+      const int rc = ensure_graph(h, q);
+      if (rc != CAVITY_OK) return rc;
+      CK(cudaGraphLaunch(h->graph[q][h->parity], h->stream));
+      h->parity ^= kGraphSteps[q] & 1;
+      h->steps_taken += kGraphSteps[q];
+    }
+  return CAVITY_OK;
+}
+
 // change the FP32 step kernel's tile shape: work lists, maps, graphs
 int retile(cavity *h, int p, int ty, int kc, int r) {
   CK(cudaStreamSynchronize(h->stream));
@@ -1025,6 +1046,115 @@ int get_fields_cav(cavity *h, int cav, int mask, double *host, size_t count) {
   return CAVITY_OK;
 }
 
+// The reverse sweep's chunk depth and CTAs: 32 x kAdjTY columns; the depth that
+// makes (waves + 0.25) x (depth + 2.5) least, waves the mean of the exact and the
+// rounded-up number, at least 1.5 in all: a chunk sweeps four planes of z terms
+// beside its own (2.5 planes' work), and the last CTAs run half alone.  128^3 FP32, us a launch: 161 at 4 planes, 146 at 8, 144 at 11,
+// 145 at 16, 154 at 19, 160 at 32 (one wave of 256 CTAs on 304 places).
+int adj_tiling(cavity *h, int *kc, int *ctas) {
+  const cavity_desc &d = h->descs[0];
+  int per_sm = 1;
+  if (h->f32) {
+    constexpr int smem = (int)adj_smem_bytes<float, kAdjTY>();
+    CK(cudaFuncSetAttribute(k_adj_sweep<float, kAdjTY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_sweep<float, kAdjTY>, 32 * kAdjTY, smem));
+  } else {
+    constexpr int smem = (int)adj_smem_bytes<double, kAdjTY>();
+    CK(cudaFuncSetAttribute(k_adj_sweep<double, kAdjTY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_sweep<double, kAdjTY>, 32 * kAdjTY, smem));
+  }
+  const long long xy = (long long)ceil_div(d.nx, 32) * ceil_div(d.ny, kAdjTY);
+  const int slots = h->nsm * std::max(per_sm, 1);
+  double best = 1e300;
+  for (int k = 1; k <= d.nz; ++k) {
+    const long long tiles = xy * ceil_div(d.nz, k);
+    const double cost = std::max(1.5, 0.5 * ((double)tiles / slots + ceil_div(tiles, slots)) + 0.25) * (k + 2.5);
+    if (cost < best) {
+      best = cost;
+      *kc = k;
+      *ctas = (int)tiles;
+    }
+  }
+  return CAVITY_OK;
+}
+
+// Per segment slot: its block descriptor (slot s read, slot s + 1 written), its
+// wall faces (one walls launch covers the segment) and, in the FP32 form, its
+// tensor maps; made again when the tiling has changed.  The constant walls
+// (u = v = w = 0, the isothermal T) go into every slot.
+int adj_tables(cavity *h) {
+  AdjointStore &A = h->adj;
+  const int ckpt = A.ckpt;
+  if (A.layout != h->layout) {
+    std::vector<BlockDev> sb(ckpt, h->hb[0]);
+    std::vector<WallFace> sf;
+    for (int s = 0; s < ckpt; ++s) {
+      sb[s].base[0] = A.seg_mem + (size_t)s * A.set_bytes;
+      sb[s].base[1] = A.seg_mem + (size_t)std::min(s + 1, ckpt - 1) * A.set_bytes;
+      for (WallFace f : h->hwall) {
+        f.block = s;
+        f.cta_begin += s * h->n_bc;
+        sf.push_back(f);
+      }
+    }
+    CK(cudaMemcpyAsync(A.seg_blocks, sb.data(), sizeof(BlockDev) * sb.size(), cudaMemcpyHostToDevice, h->stream));
+    CK(cudaMemcpyAsync(A.seg_faces, sf.data(), sizeof(WallFace) * sf.size(), cudaMemcpyHostToDevice, h->stream));
+    std::vector<CUtensorMap> sm;
+    if (h->f32) {
+      sm.resize(2 * (size_t)ckpt);
+      for (int s = 0; s < ckpt; ++s) {
+        const int rc = encode_block_maps(h, h->hb[0], A.seg_mem + (size_t)s * A.set_bytes, &sm[2 * s]);
+        if (rc != CAVITY_OK) return rc;
+      }
+      CK(cudaMemcpyAsync(A.seg_maps, sm.data(), sizeof(CUtensorMap) * sm.size(), cudaMemcpyHostToDevice, h->stream));
+    }
+    CK(cudaStreamSynchronize(h->stream));  // the host vectors end here
+    A.layout = h->layout;
+  }
+  BcArgs ba = bc_args(h, 0, 5);
+  ba.blocks = A.seg_blocks;
+  ba.faces = A.seg_faces;
+  ba.nfaces = (int)h->hwall.size() * ckpt;
+  if (h->f32) k_bc<float><<<h->n_bc * ckpt, kBcThreads, 0, h->stream>>>(ba);
+  else k_bc<double><<<h->n_bc * ckpt, kBcThreads, 0, h->stream>>>(ba);
+  CK(cudaGetLastError());
+  return CAVITY_OK;
+}
+
+// A recomputed step: slot s to slot s + 1 (nothing is finalised)
+cudaError_t launch_recompute(cavity *h, int s, bool pdl) {
+  const AdjointStore &A = h->adj;
+  if (!h->f32) {
+    StepArgs a = step_args(h, 0, 0, 0);
+    a.blocks = A.seg_blocks + s;
+    return launch_step_f64(h, a, BcArgs{}, pdl);
+  }
+  StepF32Args a = step_f32_args(h, 0, 0);
+  a.blocks = A.seg_blocks + s;
+  a.maps = A.seg_maps + 2 * s;
+  return launch_step_f32(h, a, pdl);
+}
+
+// dt, the centre shift (and stored walls) of slot s for the recomputed step after it
+cudaError_t launch_recompute_between(cavity *h, int s) {
+  const AdjointStore &A = h->adj;
+  ExchArgs x = exch_args(h, 0);
+  BcArgs b = bc_args(h, 0, 3);
+  x.blocks = b.blocks = A.seg_blocks + s;
+  b.dt_out = A.dts + s;
+  const int grid = 1 + (h->f32 || h->form_walls ? 0 : h->n_bc);
+  if (h->f32) return launch_chained(h, true, k_between<float>, grid, dim3(kBetweenThreads), 0, x, b, 0);
+  return launch_chained(h, true, k_between<double>, grid, dim3(kBetweenThreads), 0, x, b, 0);
+}
+
+void free_adjoint(AdjointStore &A) {
+  void *aptrs[] = {A.ckpt_mem, A.ckpt_cs, A.seg_mem, A.final_mem, A.X, A.Q, A.thetabar, A.scal,
+                   A.argpart, A.gpart, A.dts, A.seg_blocks, A.seg_faces, A.seg_maps, A.cnt};
+  for (void *p : aptrs)
+    if (p) cudaFree(p);
+  A = AdjointStore{};
+}
+
 void release(cavity *h) {
   DeviceGuard g(h->dev);
   if (h->stream) cudaStreamSynchronize(h->stream);
@@ -1034,10 +1164,7 @@ void release(cavity *h) {
   for (void *p : ptrs)
     if (p) cudaFree(p);
   AdjointStore &A = h->adj;
-  void *aptrs[] = {A.ckpt_mem, A.ckpt_cs, A.seg_mem, A.final_mem, A.X, A.Yt, A.Q, A.thetabar, A.scal,
-                   A.argpart, A.gpart, A.dts, A.block, A.seg_blocks, A.seg_faces, A.seg_maps, A.cnt};
-  for (void *p : aptrs)
-    if (p) cudaFree(p);
+  free_adjoint(A);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   if (h->side) cudaStreamDestroy(h->side);
   if (h->capture) cudaStreamDestroy(h->capture);
@@ -1138,38 +1265,6 @@ int create_common(const cavity_desc *descs, const cavity_params *params, int n, 
 }  // namespace
 
 // ===========================================================================
-// the reverse of one step: state storage S, adjoint arrays and arithmetic Ad
-template <class S, class Ad>
-void launch_adjoint_step(cavity *h, const AdjArgs &a, int nparts, long long nint, long long nfold, cudaEvent_t eb,
-                         cudaEvent_t ea) {
-  if constexpr (std::is_same<Ad, float>::value) {
-    // FP32 sweep: the objective, the p-adjoint sum and the centre-shift
-    // transpose in place on X in one launch, then the gather reads X as Yt
-    // (no atomics, no full prepare pass); the argmax of this state came with
-    // its segment's (a.argpart), and the dt kernel reduces the gather's
-    // partials itself
-    k_adj_pre<Ad><<<nparts, 256, 0, h->stream>>>(a, h->adj.cnt);
-    AdjArgs g = a;
-    g.Yt = a.X;
-    cudaEventRecord(eb, h->stream);
-    k_adj_gather<<<ceil_div(a.g.fs, 256), 256, 0, h->stream>>>(g);
-    cudaEventRecord(ea, h->stream);
-    AdjArgs d = a;
-    d.gpart2 = nullptr;
-    k_adj_dt<S, Ad><<<1, kAdjDtThreads, 0, h->stream>>>(d, nparts);
-  } else {
-    k_adj_objective<Ad><<<ceil_div((long long)a.g.ny * a.g.nz, 256), 256, 0, h->stream>>>(a);
-    k_adj_sum_p<Ad><<<nparts, 256, 0, h->stream>>>(a);
-    k_adj_prepare<Ad, true><<<dim3((unsigned)ceil_div(a.g.fs, 256), 5), 256, 0, h->stream>>>(a);
-    cudaEventRecord(eb, h->stream);
-    k_adj_rates<S, Ad><<<ceil_div(nint, 256), 256, 0, h->stream>>>(a);
-    cudaEventRecord(ea, h->stream);
-    k_adj_argmax<S><<<nparts, 256, 0, h->stream>>>(a);
-    k_adj_dt<S, Ad><<<1, kAdjDtThreads, 0, h->stream>>>(a, nparts);
-  }
-  k_adj_fold<Ad><<<ceil_div(nfold, 256), 256, 0, h->stream>>>(a);
-}
-
 // cavity_check_sqrt: relative difference of sqrt_newton from CUDA's sqrt
 __global__ void k_check_sqrt(const double *x, long long n, double *rel) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1183,25 +1278,6 @@ __global__ void k_check_div3(const double *x, long long n, unsigned char *diff) 
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   diff[i] = div3(x[i]) != x[i] / 3.0;
-}
-
-// Recomputation of a checkpointed segment without copies: points block 0 of
-// the step graph's descriptor table at two buffer sets -- base[0] (read) = b0,
-// base[1] (written) = b1 -- and, in the FP32 form, replaces the parity-0
-// tensor maps with b0's (src[0], src[1]), so the captured one-step graph of
-// parity 0 steps the state in slot s straight into slot s + 1.  One warp.
-__global__ void k_adj_point(BlockDev *blk, CUtensorMap *maps, const CUtensorMap *src, void *b0, void *b1) {
-  if (threadIdx.x == 0) {
-    blk->base[0] = b0;
-    blk->base[1] = b1;
-  }
-  if (maps) {
-    static_assert(sizeof(CUtensorMap) == 128, "two 128-byte maps, 8 bytes per lane");
-    reinterpret_cast<unsigned long long *>(maps)[threadIdx.x] =
-        reinterpret_cast<const unsigned long long *>(src)[threadIdx.x];
-    // the maps are read through the tensor-map proxy by the next kernel
-    asm volatile("fence.proxy.tensormap::generic.release.gpu;" ::: "memory");
-  }
 }
 
 // FP64 FMA throughput of the GPU: every thread runs kDfmaChains independent
@@ -1278,15 +1354,7 @@ int cavity_set_wall_temperature(cavity_t *h, int wall, const double *host, size_
 int cavity_step(cavity_t *h, int nsteps) {
   if (!h || nsteps < 0) return CAVITY_ERR_INVALID_ARG;
   DeviceGuard g(h->dev);
-  for (int q = kGraphs - 1; q >= 0; --q)
-    for (; nsteps >= kGraphSteps[q]; nsteps -= kGraphSteps[q]) {
-      const int rc = ensure_graph(h, q);
-      if (rc != CAVITY_OK) return rc;
-      CK(cudaGraphLaunch(h->graph[q][h->parity], h->stream));
-      h->parity ^= kGraphSteps[q] & 1;
-      h->steps_taken += kGraphSteps[q];
-    }
-  return CAVITY_OK;
+  return run_steps(h, nsteps);
 }
 
 int cavity_batch_state(cavity_t *h, int cav, double out[10]) {
@@ -1605,95 +1673,54 @@ int cavity_adjoint_forward(cavity_t *h, int nsteps, int ckpt, double *J) {
   const cavity_desc &d = h->descs[0];
   const size_t set_bytes = (size_t)h->na * (size_t)B.fstride * h->esize;
   const int ncp = (nsteps + ckpt - 1) / ckpt;
-  const long long fs = (long long)(d.nx + 4) * (d.ny + 4) * (d.nz + 4);
-  const int nparts = 2 * 152;
   CK(cudaStreamSynchronize(h->stream));
-  if (A.set_bytes != set_bytes || A.ncp < ncp || A.ckpt < ckpt || A.nsteps < nsteps) {
-    void *aptrs[] = {A.ckpt_mem, A.ckpt_cs, A.seg_mem, A.final_mem, A.X, A.Yt, A.Q, A.thetabar, A.scal,
-                     A.argpart, A.gpart, A.dts, A.block, A.seg_blocks, A.seg_faces, A.seg_maps, A.cnt};
-    for (void *p : aptrs)
-      if (p) cudaFree(p);
-    A = AdjointStore{};
+  if (A.set_bytes != set_bytes || A.ncp < ncp || A.ckpt < ckpt) {
+    free_adjoint(A);
+    const size_t abytes = h->esize * 5 * (size_t)B.fstride;
+    const int rt = adj_tiling(h, &A.kc, &A.ctas);
+    if (rt != CAVITY_OK) return rt;
     CK(cudaMalloc(&A.ckpt_mem, set_bytes * ncp));
     CK(cudaMalloc(&A.ckpt_cs, sizeof(CavState) * ncp));
     CK(cudaMalloc(&A.seg_mem, set_bytes * ckpt));
+    // (a slot's velocity walls stay zero, and nothing a step reads is unset)
+    CK(cudaMemsetAsync(A.seg_mem, 0, set_bytes * ckpt, h->stream));
     CK(cudaMalloc(&A.final_mem, set_bytes));
-    const size_t abytes = (h->f32 ? sizeof(float) : sizeof(double)) * 5 * fs;
     CK(cudaMalloc(&A.X, abytes));
-    CK(cudaMalloc(&A.Yt, abytes));
     CK(cudaMalloc(&A.Q, abytes));
     CK(cudaMalloc(&A.thetabar, sizeof(double) * d.ny * d.nz));
     CK(cudaMalloc(&A.scal, sizeof(double) * kScCount));
-    CK(cudaMalloc(&A.argpart, sizeof(double) * 2 * nparts * ckpt));  // one set per segment slot
+    CK(cudaMalloc(&A.argpart, sizeof(double) * 2 * kAdjParts * ckpt));  // one set per segment slot
     CK(cudaMalloc(&A.cnt, sizeof(unsigned int)));
-    CK(cudaMemset(A.cnt, 0, sizeof(unsigned int)));
-    CK(cudaMalloc(&A.gpart, sizeof(double) * 3 * (ceil_div(fs, 256) + nparts)));
-    CK(cudaMalloc(&A.dts, sizeof(double) * nsteps));
-    CK(cudaMalloc(&A.block, sizeof(BlockDev)));
-    A.set_bytes = set_bytes;
-    // per segment slot: its block descriptor, its wall faces (one walls
-    // launch covers the segment) and, in the FP32 form, its tensor maps
-    std::vector<BlockDev> sb(ckpt, h->hb[0]);
-    std::vector<WallFace> sf;
-    for (int s = 0; s < ckpt; ++s) {
-      sb[s].base[0] = A.seg_mem + (size_t)s * set_bytes;
-      for (WallFace f : h->hwall) {
-        f.block = s;
-        f.cta_begin += s * h->n_bc;
-        sf.push_back(f);
-      }
-    }
+    CK(cudaMemsetAsync(A.cnt, 0, sizeof(unsigned int), h->stream));
+    CK(cudaMalloc(&A.gpart, sizeof(double) * 4 * A.ctas));
+    CK(cudaMalloc(&A.dts, sizeof(double) * (ckpt + 1)));
     CK(cudaMalloc(&A.seg_blocks, sizeof(BlockDev) * ckpt));
-    CK(cudaMalloc(&A.seg_faces, sizeof(WallFace) * sf.size()));
-    CK(cudaMemcpy(A.seg_blocks, sb.data(), sizeof(BlockDev) * ckpt, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(A.seg_faces, sf.data(), sizeof(WallFace) * sf.size(), cudaMemcpyHostToDevice));
-    if (h->f32) {
-      std::vector<CUtensorMap> sm(2 * (size_t)ckpt);
-      for (int s = 0; s < ckpt; ++s) {
-        const int rc = encode_block_maps(h, h->hb[0], A.seg_mem + (size_t)s * set_bytes, &sm[2 * s]);
-        if (rc != CAVITY_OK) return rc;
-      }
-      CK(cudaMalloc(&A.seg_maps, sizeof(CUtensorMap) * sm.size()));
-      CK(cudaMemcpy(A.seg_maps, sm.data(), sizeof(CUtensorMap) * sm.size(), cudaMemcpyHostToDevice));
-    }
+    CK(cudaMalloc(&A.seg_faces, sizeof(WallFace) * h->hwall.size() * ckpt));
+    if (h->f32) CK(cudaMalloc(&A.seg_maps, sizeof(CUtensorMap) * 2 * (size_t)ckpt));
+    A.set_bytes = set_bytes;
+    A.ckpt = ckpt;
+    A.ncp = ncp;
   }
+  A.have_forward = false;
+  int rc = adj_tables(h);
+  if (rc != CAVITY_OK) return rc;
   A.nsteps = nsteps;
-  A.ckpt = ckpt;
-  A.ncp = ncp;
-  A.nparts = nparts;
-  // every segment slot starts as a copy of the initial state: the step
-  // writes interior nodes and the walls that change (p, adiabatic T), so the
-  // constant wall values (u = v = w = 0, the isothermal T) a recomputed state
-  // is read with must already be in its slot
-  for (int s = 0; s < ckpt; ++s)
-    CK(cudaMemcpyAsync(A.seg_mem + (size_t)s * set_bytes, h->hb[0].base[h->parity], set_bytes,
+  A.run_ckpt = ckpt;
+  CK(cudaMemsetAsync(&h->d_cs[0].nu_sum, 0, sizeof(double), h->stream));
+  for (int n = 0; n < nsteps; n += ckpt) {
+    const int c = n / ckpt;
+    CK(cudaMemcpyAsync(A.ckpt_mem + (size_t)c * set_bytes, h->hb[0].base[h->parity], set_bytes,
                        cudaMemcpyDeviceToDevice, h->stream));
-  CK(cudaMemsetAsync(A.scal, 0, sizeof(double) * kScCount, h->stream));
-  {
-    const int rc = ensure_graph(h, 0);
+    CK(cudaMemcpyAsync(A.ckpt_cs + c, h->d_cs, sizeof(CavState), cudaMemcpyDeviceToDevice, h->stream));
+    rc = run_steps(h, std::min(ckpt, nsteps - n));
     if (rc != CAVITY_OK) return rc;
-  }
-  for (int n = 0; n < nsteps; ++n) {
-    if (n % ckpt == 0) {
-      const int c = n / ckpt;
-      CK(cudaMemcpyAsync(A.ckpt_mem + (size_t)c * set_bytes, h->hb[0].base[h->parity], set_bytes,
-                         cudaMemcpyDeviceToDevice, h->stream));
-      CK(cudaMemcpyAsync(A.ckpt_cs + c, h->d_cs, sizeof(CavState), cudaMemcpyDeviceToDevice, h->stream));
-    }
-    CK(cudaGraphLaunch(h->graph[0][h->parity], h->stream));
-    h->parity ^= 1;
-    h->steps_taken += 1;
-    k_adj_acc_nusselt<<<1, 1, 0, h->stream>>>(h->d_cs, A.scal);
-    CK(cudaGetLastError());
   }
   CK(cudaMemcpyAsync(A.final_mem, h->hb[0].base[h->parity], set_bytes, cudaMemcpyDeviceToDevice, h->stream));
   CK(cudaMemcpyAsync(&A.final_cs, h->d_cs, sizeof(CavState), cudaMemcpyDeviceToHost, h->stream));
-  double acc = 0.0;
-  CK(cudaMemcpyAsync(&acc, A.scal + kScJ, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   A.final_parity = h->parity;
   A.final_steps = h->steps_taken;
-  A.J = acc / nsteps;
+  A.J = A.final_cs.nu_sum / nsteps;
   A.have_forward = true;
   if (J) *J = A.J;
   return state_status(A.final_cs);
@@ -1706,96 +1733,83 @@ int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *gr
   const cavity_desc &d = h->descs[0];
   if (grad_wall && n != (size_t)d.ny * d.nz) return fail(h, CAVITY_ERR_INVALID_ARG, "grad_wall count must be ny*nz");
   DeviceGuard g(h->dev);
-  const BlockDev B0 = h->hb[0];
   const cavity_params &p = h->prms[0];
+  int rc = adj_tables(h);
+  if (rc != CAVITY_OK) return rc;
   AdjArgs a{};
+  a.B = h->hb[0];
   a.C = h->hcc[0];
-  a.g = AdjGeom{d.nx, d.ny, d.nz, (long long)d.nx + 4, (long long)d.ny + 4,
-                (long long)(d.nx + 4) * (d.ny + 4) * (d.nz + 4)};
-  a.Yt = A.Yt;
   a.scal = A.scal;
   a.thetabar = A.thetabar;
-  a.argpart = A.argpart;
+  a.nparts = kAdjParts;
   a.gpart = A.gpart;
-  a.ngpart = h->f32 ? (int)ceil_div(a.g.fs, 256) : 0;
-  a.gpart2 = A.gpart + 3 * ceil_div(a.g.fs, 256);
+  a.cnt = A.cnt;
+  a.kc = A.kc;
+  a.tiles_x = ceil_div(d.nx, 32);
+  a.tiles_y = ceil_div(d.ny, kAdjTY);
   a.coef = 1.0 / ((double)A.nsteps * d.ny * d.nz * 2.0 * a.C.h[0] * (p.t_hot - p.t_cold));
   a.dfloor = (h->u_ref_auto && p.Ra * p.Pr > 1.0) ? p.kappa * p.Pr : 0.0;
   void *X = A.X, *Q = A.Q;
-  CK(cudaMemsetAsync(X, 0, (h->f32 ? sizeof(float) : sizeof(double)) * 5 * a.g.fs, h->stream));
-  CK(cudaMemsetAsync(A.thetabar, 0, sizeof(double) * d.ny * d.nz, h->stream));
+  const size_t abytes = h->esize * 5 * (size_t)a.B.fstride;
+  CK(cudaMemsetAsync(X, 0, abytes, h->stream));
+  CK(cudaMemsetAsync(Q, 0, abytes, h->stream));
   CK(cudaMemsetAsync(A.scal, 0, sizeof(double) * kScCount, h->stream));
-  const long long nint = (long long)d.nx * d.ny * d.nz;
-  const long long nfold = 2LL * ((long long)d.ny * d.nz + (long long)d.nx * d.nz + (long long)d.nx * d.ny);
-  std::vector<double> dts(A.ckpt);
-  while (h->adj_ev.size() < 2 * (size_t)A.nsteps) {
+  a.Q = X;
+  if (h->f32) k_adj_start<float><<<ceil_div((long long)d.ny * d.nz, 256), 256, 0, h->stream>>>(a);
+  else k_adj_start<double><<<ceil_div((long long)d.ny * d.nz, 256), 256, 0, h->stream>>>(a);
+  CK(cudaGetLastError());
+  const int ck = A.run_ckpt, nseg = (A.nsteps + ck - 1) / ck;
+  while (h->adj_ev.size() < 2 * (size_t)nseg) {
     cudaEvent_t e = nullptr;
     CK(cudaEventCreate(&e));
     h->adj_ev.push_back(e);
   }
-  int rc = ensure_graph(h, 0);
-  if (rc != CAVITY_OK) return rc;
   auto slot = [&](int s) { return (void *)(A.seg_mem + (size_t)s * A.set_bytes); };
-  for (int c = A.ncp - 1; c >= 0 && rc == CAVITY_OK; --c) {
-    const int s0 = c * A.ckpt, s1 = std::min(s0 + A.ckpt, A.nsteps);
+  for (int c = nseg - 1; c >= 0; --c) {
+    const int s0 = c * ck, len = std::min(ck, A.nsteps - s0);
     // recompute the segment from its checkpoint (copied to slot 0), each step
-    // of the parity-0 graph reading slot s - s0 and writing slot s - s0 + 1
+    // reading slot s and writing slot s + 1
     CK(cudaMemcpyAsync(slot(0), A.ckpt_mem + (size_t)c * A.set_bytes, A.set_bytes, cudaMemcpyDeviceToDevice,
                        h->stream));
     CK(cudaMemcpyAsync(h->d_cs, A.ckpt_cs + c, sizeof(CavState), cudaMemcpyDeviceToDevice, h->stream));
-    for (int s = s0; s < s1; ++s) {
-      CK(cudaMemcpyAsync(A.dts + s, &h->d_cs->dt, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
-      if (s < s1 - 1) {
-        k_adj_point<<<1, 32, 0, h->stream>>>(h->d_blocks, h->f32 ? h->d_maps : nullptr,
-                                             h->f32 ? A.seg_maps + 2 * (s - s0) : nullptr, slot(s - s0),
-                                             slot(s - s0 + 1));
-        CK(cudaGetLastError());
-        CK(cudaGraphLaunch(h->graph[0][0], h->stream));
-      }
+    CK(cudaMemcpyAsync(A.dts, &h->d_cs->dt, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
+    for (int s = 0; s + 1 < len; ++s) {
+      CK(launch_recompute(h, s, s > 0));
+      CK(launch_recompute_between(h, s + 1));
     }
-    {
-      // the step forms p's and T's wall values where it reads them: write
-      // them into every stored state of the segment, one launch
-      BcArgs ba = bc_args(h, 0, 3);
-      ba.blocks = A.seg_blocks;
-      ba.faces = A.seg_faces;
-      ba.nfaces = (int)h->hwall.size() * (s1 - s0);
-      if (h->f32) k_bc<float><<<h->n_bc * (s1 - s0), kBcThreads, 0, h->stream>>>(ba);
-      else k_bc<double><<<h->n_bc * (s1 - s0), kBcThreads, 0, h->stream>>>(ba);
-      CK(cudaGetLastError());
-    }
+    // the walls (formed by the step where it reads them) of every stored state
+    BcArgs ba = bc_args(h, 0, 3);
+    ba.blocks = A.seg_blocks;
+    ba.faces = A.seg_faces;
+    ba.nfaces = (int)h->hwall.size() * len;
+    const dim3 parts(kAdjParts, len);
     if (h->f32) {
-      // the argmax of every state of the segment's spectral bound, one launch
-      k_adj_argmax_seg<float><<<dim3(A.nparts, s1 - s0), 256, 0, h->stream>>>(A.seg_blocks, h->hcc[0], a.g, A.argpart);
-      CK(cudaGetLastError());
+      k_bc<float><<<h->n_bc * len, kBcThreads, 0, h->stream>>>(ba);
+      k_adj_argmax_seg<float><<<parts, 256, 0, h->stream>>>(A.seg_blocks, h->hcc[0], A.argpart);
+    } else {
+      k_bc<double><<<h->n_bc * len, kBcThreads, 0, h->stream>>>(ba);
+      k_adj_argmax_seg<double><<<parts, 256, 0, h->stream>>>(A.seg_blocks, h->hcc[0], A.argpart);
     }
-    CK(cudaMemcpyAsync(dts.data(), A.dts + s0, sizeof(double) * (s1 - s0), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
+    CK(cudaGetLastError());
     // reverse sweep over the segment
-    for (int s = s1 - 1; s >= s0; --s) {
-      a.B = B0;
-      a.B.base[0] = slot(s - s0);
-      a.dt = dts[s - s0];
-      a.argpart = h->f32 ? A.argpart + 2 * (size_t)A.nparts * (s - s0) : A.argpart;
+    CK(cudaEventRecord(h->adj_ev[2 * c], h->stream));
+    for (int s = len - 1; s >= 0; --s) {
+      a.B.base[0] = slot(s);
+      a.dt = A.dts + s;
+      a.argpart = A.argpart + 2 * (size_t)kAdjParts * s;
+      a.objective = s0 + s > 0;
       a.X = X;
       a.Q = Q;
-      cudaEvent_t eb = h->adj_ev[2 * s], ea = h->adj_ev[2 * s + 1];
-      if (h->f32) launch_adjoint_step<float, float>(h, a, A.nparts, nint, nfold, eb, ea);
-      else launch_adjoint_step<double, double>(h, a, A.nparts, nint, nfold, eb, ea);
-      if (cudaGetLastError() != cudaSuccess) { rc = fail(h, CAVITY_ERR_CUDA, "adjoint kernel launch failed"); break; }
+      const bool pdl = s < len - 1;
+      if (h->f32)
+        CK(launch_chained(h, pdl, k_adj_sweep<float, kAdjTY>, A.ctas, dim3(32 * kAdjTY), adj_smem_bytes<float, kAdjTY>(), a));
+      else
+        CK(launch_chained(h, pdl, k_adj_sweep<double, kAdjTY>, A.ctas, dim3(32 * kAdjTY), adj_smem_bytes<double, kAdjTY>(), a));
       std::swap(X, Q);
     }
+    CK(cudaEventRecord(h->adj_ev[2 * c + 1], h->stream));
   }
-  // the step graph's table and maps back to the handle's buffers, and the
-  // state after the forward run
-  {
-    const int r2 = upload_tables(h);
-    if (r2 != CAVITY_OK) return r2;
-    if (h->f32) {
-      const int r3 = encode_maps(h);
-      if (r3 != CAVITY_OK) return r3;
-    }
-  }
+  // the state after the forward run
   CK(cudaMemcpyAsync(h->hb[0].base[A.final_parity], A.final_mem, A.set_bytes, cudaMemcpyDeviceToDevice, h->stream));
   CK(cudaMemcpyAsync(h->d_cs, &A.final_cs, sizeof(CavState), cudaMemcpyHostToDevice, h->stream));
   h->parity = A.final_parity;
@@ -1806,16 +1820,14 @@ int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *gr
     CK(cudaMemcpyAsync(grad_wall, A.thetabar, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   if (grad_ra) *grad_ra = ra;
-  if (rc == CAVITY_OK) {
-    double tot = 0.0;
-    for (int s = 0; s < A.nsteps; ++s) {
-      float ms = 0.f;
-      CK(cudaEventElapsedTime(&ms, h->adj_ev[2 * s], h->adj_ev[2 * s + 1]));
-      tot += ms;
-    }
-    h->adj_rates_ms = tot / A.nsteps;
+  double tot = 0.0;
+  for (int c = 0; c < nseg; ++c) {
+    float ms = 0.f;
+    CK(cudaEventElapsedTime(&ms, h->adj_ev[2 * c], h->adj_ev[2 * c + 1]));
+    tot += ms;
   }
-  return rc;
+  h->adj_rates_ms = tot / A.nsteps;
+  return CAVITY_OK;
 }
 
 int cavity_adjoint_kernel_ms(cavity_t *h, double *ms) {
