@@ -1060,6 +1060,7 @@ __device__ __forceinline__ void load_slice(const BcArgs &a, const double *step_p
     if (a.mode == 4) { acc[6] = x3.x; acc[7] = x3.y; }
     q += NT;
   }
+#pragma unroll 4
   for (; q < q1; q += NT) {
     const double *pp = step_partials + q * kPartStride;
     for (int f = 0; f < 5; ++f) acc[f] += pp[f];

@@ -31,7 +31,7 @@ using namespace bdc;
 
 namespace {
 
-constexpr int kTX = 32, kTY = 8, kKC = 16;  // the tile of the FP64 step kernel
+constexpr int kTX = 32, kTY = 8, kKC = 16;  // the tile the size limit is stated in
 constexpr int kDescBytes = 1280;           // BlockDev (256) + CavConst (768) + CavState (256), aligned slots
 constexpr size_t kScratchBytes = kDescBytes + (size_t)CAVITY_NOALLOC_MAX_TILES * kPartStride * sizeof(double);
 constexpr int kMaxDevices = 64;
@@ -62,40 +62,53 @@ cudaError_t scratch_address(int dev, void **out) {
 // Writes the three descriptors into the scratch array.  They arrive as kernel
 // parameters, which the launch copies by value, so the call reads no host
 // memory after it returns and makes no host-to-device copy of its own.
-__global__ void k_noalloc_setup(BlockDev B, CavConst C, CavState S, BlockDev *d_block, CavConst *d_cc,
-                                CavState *d_cs) {
-  if (threadIdx.x == 0) {
-    *d_block = B;
-    *d_cc = C;
-    *d_cs = S;
-  }
+struct Descriptors {
+  BlockDev B;
+  CavConst C;
+  CavState S;
+};
+__global__ void __launch_bounds__(128) k_noalloc_setup(const __grid_constant__ Descriptors d, BlockDev *d_block,
+                                                       CavConst *d_cc, CavState *d_cs) {
+  chain_trigger();  // (the step's launch waits for this one before it reads anything)
+  auto copy = [](void *to, const void *from, int bytes) {
+    for (int n = threadIdx.x; n < bytes / 8; n += 128)
+      static_cast<unsigned long long *>(to)[n] = static_cast<const unsigned long long *>(from)[n];
+  };
+  static_assert(sizeof(BlockDev) % 8 == 0 && sizeof(CavConst) % 8 == 0 && sizeof(CavState) % 8 == 0, "whole words");
+  copy(d_block, &d.B, sizeof(BlockDev));
+  copy(d_cc, &d.C, sizeof(CavConst));
+  copy(d_cs, &d.S, sizeof(CavState));
 }
 
 // RMS of the five rates and the next dt from the per-CTA partials, summed in
-// a fixed order (thread q takes partials q, q + 256, ...; warps in order)
-__global__ void __launch_bounds__(256) k_noalloc_reduce(const double *partials, int ntiles, const CavConst *cc,
-                                                        double *out6) {
-  __shared__ double sh[8][6];
-  const int tid = threadIdx.x;
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  for (int q = tid; q < ntiles; q += 256) {
-    const double *pp = partials + (long long)q * kPartStride;
-    for (int f = 0; f < 5; ++f) acc[f] += pp[f];
-    acc[5] = fmax(acc[5], pp[5]);
-  }
-  for (int f = 0; f < 5; ++f) acc[f] = warp_sum(acc[f]);
-  acc[5] = warp_max(acc[5]);
-  if ((tid & 31) == 0)
-    for (int f = 0; f < 6; ++f) sh[tid >> 5][f] = acc[f];
-  __syncthreads();
-  if (tid == 0) {
-    double tot[6];
-    for (int f = 0; f < 6; ++f) tot[f] = sh[0][f];
-    for (int w = 1; w < 8; ++w)
-      for (int f = 0; f < 6; ++f) tot[f] = (f == 5) ? fmax(tot[f], sh[w][f]) : tot[f] + sh[w][f];
-    for (int f = 0; f < 5; ++f) out6[f] = sqrt(tot[f] * cc->inv_nint);
-    out6[5] = cc->cfl / tot[5];
-  }
+// the finalise's fixed order (thread-strided, then its tree); a field's square
+// root or division in a thread of its own.
+__global__ void __launch_bounds__(kFinThreads) k_noalloc_reduce(const double *partials, int ntiles, const CavConst *cc,
+                                                                double *out6) {
+  __shared__ double sv[8 * kFinThreads];
+  chain_wait();
+  const int tid = threadIdx.x, f = tid >> 4;
+  double acc[8];
+  load_slice<kFinThreads>(BcArgs{}, partials, 0, ntiles, 0, 0, 0, 0, tid, acc);
+  const double t = tree_slice<kFinThreads>(acc, sv, tid);
+  if ((tid & 15) != 0 || f > 5) return;
+  out6[f] = f < 5 ? sqrt(t * cc->inv_nint) : cc->cfl / t;
+}
+
+// A launch that may start before the one ahead of it in the stream has ended
+// (each waits for that before it reads what it wrote).
+template <class K, class... A>
+cudaError_t launch_after(K kernel, int grid, int block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
@@ -135,12 +148,27 @@ extern "C" CAVITY_API int cavity_step_block_noalloc(const double *q_in, double *
   B.plane = (long long)B.pitch * B.rows;
   B.fstride = B.plane * (nz + 4);
   for (int f = 0; f < 6; ++f) { B.wall[f] = 1; B.nbr[f] = -1; }
-  B.tiles_x = ceil_div((long long)nx * ny, kTX * kTY);
+  // Tiles of consecutive nodes, one CTA each, of a depth that leaves the SMs
+  // equal shares of the tile planes (as the handle's, assign_tiles): with
+  // 16-plane tiles of 256 nodes at all sizes a 40x36x34 block was 18 CTAs and
+  // 137 us a call.  Where tiles of 128 nodes would not fit the scratch, the
+  // 256-node ones do (256 consecutive nodes fill no more tiles than the limit's).
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return CAVITY_ERR_CUDA;
+  int nt = 128;
+  const long long planes = (long long)ceil_div((long long)nx * ny, nt) * nz;
+  int kc = planes <= 8LL * sms ? 1 : planes <= 16LL * sms ? 2 : planes <= 64LL * sms ? 4 : 8;
+  while (kc < kKC && (long long)ceil_div((long long)nx * ny, nt) * ceil_div(nz, kc) > CAVITY_NOALLOC_MAX_TILES) kc *= 2;
+  if ((long long)ceil_div((long long)nx * ny, nt) * ceil_div(nz, kc) > CAVITY_NOALLOC_MAX_TILES) {
+    nt = kTX * kTY;
+    kc = kKC;
+  }
+  B.tiles_x = ceil_div((long long)nx * ny, nt);
   B.tiles_y = 1;
-  B.tiles_z = ceil_div(nz, kKC);
-  B.tiles_zc = B.tiles_z;  // one CTA per tile: KC-plane chunks only
+  B.tiles_z = ceil_div(nz, kc);
+  B.tiles_zc = B.tiles_z;  // kc-plane chunks only
   B.zsplit = nz;
-  B.kc = B.kf = kKC;
+  B.kc = B.kf = kc;
   B.coarse_begin = 0;
   B.fine_begin = 0;
   B.base[0] = (void *)(q_in - (XO<double>::v - 2));
@@ -155,17 +183,19 @@ extern "C" CAVITY_API int cavity_step_block_noalloc(const double *q_in, double *
   S.c = pshift;
 
   cudaStream_t st = (cudaStream_t)stream;
-  k_noalloc_setup<<<1, 32, 0, st>>>(B, C, S, d_block, d_cc, d_cs);
+  k_noalloc_setup<<<1, 128, 0, st>>>(Descriptors{B, C, S}, d_block, d_cc, d_cs);
   if (cudaGetLastError() != cudaSuccess) return CAVITY_ERR_CUDA;
   StepArgs a{};  // tile_counter null: one CTA per tile
   a.blocks = d_block; a.nblocks = 1; a.cc = d_cc; a.cs = d_cs;
-  const int ntiles = B.tiles_x * B.tiles_z;  // at most the limit's count: 256 consecutive nodes fill no fewer tiles
+  const int ntiles = B.tiles_x * B.tiles_z;
   a.partials = d_part; a.parity = 0; a.mode = 0; a.ntiles = ntiles;
   a.ncoarse = ntiles;
   // walls and ghosts read as the caller filled them
-  k_step_f64<kTX * kTY, false><<<ntiles, kTX * kTY, 0, st>>>(a, BcArgs{});
-  if (cudaGetLastError() != cudaSuccess) return CAVITY_ERR_CUDA;
-  k_noalloc_reduce<<<1, 256, 0, st>>>(d_part, ntiles, d_cc, out6);
-  if (cudaGetLastError() != cudaSuccess) return CAVITY_ERR_CUDA;
+  const cudaError_t e = nt == 128 ? launch_after(k_step_f64<128, false>, ntiles, nt, st, a, BcArgs{})
+                                  : launch_after(k_step_f64<kTX * kTY, false>, ntiles, nt, st, a, BcArgs{});
+  if (e != cudaSuccess) return CAVITY_ERR_CUDA;
+  if (launch_after(k_noalloc_reduce, 1, kFinThreads, st, (const double *)d_part, ntiles, (const CavConst *)d_cc, out6) !=
+      cudaSuccess)
+    return CAVITY_ERR_CUDA;
   return CAVITY_OK;
 }
