@@ -365,12 +365,46 @@ __device__ __forceinline__ void rates_vel_f64(const CavConst &C, const NodeF64 &
   x.rw = BDC_TRANSPORT(n.w, nxm, nxp, nym, nyp, nzm, nzp, fma(-C.nu2s, w0, bw));
 }
 
+// The fourth differences p_++ - 4 p_+ + 6 p_0 - 4 p_- + p_-- of the 13-point star
+// along x, y and z, in 64-bit fixed point: the thirteen values as integers in
+// units of 2^-58 of the largest one's power of two (the sum's weights add up to
+// 16: below 2^63), summed exactly and rounded once to FP64.  The error is a few
+// 2^-59 of the largest |p|, where twelve FP64 operations had a few 2^-53; those
+// twelve were 12% of the step kernel's FP64 pipe time, and the 250 integer
+// instructions run in issue slots it leaves empty.  Values below 2^-959 count as
+// zero; NaN or infinity comes out as a finite value (the pressure gradient
+// carries it on).
+__device__ __forceinline__ void fourth_differences(const double p[13], double d4[3]) {
+  unsigned E = 0;
+#pragma unroll
+  for (int q = 0; q < 13; ++q) E = max(E, (unsigned)__double2hiint(p[q]) & 0x7fffffffu);
+  E >>= 20;
+  auto fixed = [&](double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned sh = min(E - ((hi >> 20) & 0x7ffu), 63u);
+    const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+    const unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, 6) << 32) | (lo << 6);
+    const long long sg = (long long)((int)hi >> 31);
+    return ((long long)(m >> sh) ^ sg) - sg;
+  };
+  const long long c6 = 6 * fixed(p[0]);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const long long S = (fixed(p[7 + 2 * d]) + fixed(p[8 + 2 * d])) - 4 * (fixed(p[1 + 2 * d]) + fixed(p[2 + 2 * d])) + c6;
+    const long long sg = S >> 63;
+    const unsigned long long A = (unsigned long long)((S ^ sg) - sg);
+    const int lz = __clzll((long long)A);
+    const unsigned long long N = A << (lz & 63);
+    const unsigned long long r = ((unsigned long long)(E + 4 - lz) << 52) + (N >> 11) + ((N >> 10) & 1);
+    d4[d] = A == 0 || E < 64 ? 0.0 : __longlong_as_double((long long)(r | ((unsigned long long)sg & (1ull << 63))));
+  }
+}
+
 __device__ __forceinline__ void rates_pt_f64(const CavConst &C, const NodeF64 &n, const VelF64 &x, double r[5]) {
-  const double u0 = n.u[0], v0 = n.v[0], w0 = n.w[0], p0 = n.p[0];
-  const double d4x = fma(6.0, p0, fma(-4.0, n.p[2] + n.p[1], n.p[8] + n.p[7]));
-  const double d4y = fma(6.0, p0, fma(-4.0, n.p[4] + n.p[3], n.p[10] + n.p[9]));
-  const double d4z = fma(6.0, p0, fma(-4.0, n.p[6] + n.p[5], n.p[12] + n.p[11]));
-  const double diss = fma(x.ex, d4x, fma(x.ey, d4y, x.ez * d4z));
+  const double u0 = n.u[0], v0 = n.v[0], w0 = n.w[0];
+  double d4[3];
+  fourth_differences(n.p, d4);
+  const double diss = fma(x.ex, d4[0], fma(x.ey, d4[1], x.ez * d4[2]));
   r[0] = fma(-x.b2, x.divV, -diss);
   r[1] = fma(-(n.p[2] - n.p[1]), C.ih2[0], x.ru);
   r[2] = fma(-(n.p[4] - n.p[3]), C.ih2[1], x.rv);
