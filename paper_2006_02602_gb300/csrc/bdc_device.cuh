@@ -264,28 +264,25 @@ __device__ __forceinline__ double warp_max(double v) {
 }
 
 // ---------------------------------------------------------------------------
-// Square root of a positive, normal, finite FP64 value with one operation on
-// the FP64 pipe.  GB300 issues an FP64 warp instruction every 16 cycles an SM
-// (two lanes a clock), FP32 and integer ones up to four a cycle, and the FP64
-// step leaves 90% of the issue slots unused, so everything but the exact
-// residual runs beside it.  With q = 4^k m, m in [1, 4):
+// Square root of a positive, normal, finite FP64 value without the FP64 pipe.
+// GB300 issues an FP64 warp instruction every 16 cycles an SM (two lanes a
+// clock), FP32 and integer ones up to four a cycle.  With q = 4^k m, m in [1, 4):
 //   y ~ 1/sqrt(m) (rsqrt.approx.ftz.f32), s_0 = sh + sl by one Newton step on
 //   the FP32 pair of m's leading 46 bits: relative error below 2^-43;
-//   r = m - s_0^2, exact to its last bit in FP64 (one fused multiply-add);
+//   r = m - s_0^2, exact, as a 64-bit integer (s_0 has 46 fraction bits);
 //   s = s_0 + r y / 2, the correction (below 2^9 units in the last place)
 //   formed in FP32 and added to s_0's significand as an integer.
 // The result is within one unit in the last place of the correctly rounded
 // root (cavity_check_sqrt measures this against CUDA's sqrt; the clamps keep
-// s_0 in [1, 2], where a unit of its last place is 2^-52).  Six FP64
-// operations (an FP64 reciprocal-square-root seed and two Newton steps) gave
-// the same accuracy.  Arguments that are NaN or infinite give a finite value:
+// s_0 in [1, 2], where a unit of its last place is 2^-52; one root in 1300 is
+// not the correctly rounded one, with r from an FP64 fused multiply-add one in
+// 90).  Arguments that are NaN or infinite give a finite value:
 // the rates reach NaN or infinity through beta^2 and the weights.
 __device__ __forceinline__ double sqrt_newton(double q) {
   const int hi = __double2hiint(q);
   const unsigned lo = (unsigned)__double2loint(q);
   const int odd = ~(hi >> 20) & 1;  // the unbiased exponent is odd
   const int mhi = (hi & 0xfffff) | ((1023 + odd) << 20);
-  const double m = __hiloint2double(mhi, (int)lo);
   const float qh = __int_as_float((int)(__funnelshift_l(lo, (unsigned)hi, 3) & 0x7fffffu) | ((127 + odd) << 23));
   // the significand's next 23 bits, as an integer in FP32
   const float ql = __fsub_rn(__uint_as_float(0x4b000000u | ((lo & 0x1fffffffu) >> 6)), 8388608.f);
@@ -297,13 +294,11 @@ __device__ __forceinline__ double sqrt_newton(double q) {
   const int n = __float2int_rn(__fmul_rn(__fmul_rn(res, hy), 0x1p46f));
   long long s0 = ((long long)__float_as_int(sh) << 29) + (896ll << 52) + ((long long)n << 6);
   s0 = max(min(s0, 0x4000000000000000ll), 0x3ff0000000000000ll);
-  const double s0d = __longlong_as_double(s0);
-  const double r = fma(-s0d, s0d, m);
-  const int rhi = __double2hiint(r);
-  // |r| in [2^-104, 2^-20] or 0 (which the maximum maps to 2^-126): FP32 bits, truncated
-  const unsigned ra = max((unsigned)rhi & 0x7fffffffu, 897u << 20) - (896u << 20);
-  const float rf = __uint_as_float(__funnelshift_l((unsigned)__double2loint(r), ra, 3) | ((unsigned)rhi & 0x80000000u));
-  const int n2 = __float2int_rn(__fmul_rn(rf, __fmul_rn(hy, 0x1p52f)));
+  // m - s0^2, below 2^-39, in units of 2^-92 (s0 is a multiple of 2^-46), modulo 2^64
+  const unsigned long long t = (unsigned long long)(s0 - (1022ll << 52)) >> 6;
+  const long long r = (long long)(((1ull << 52 | (unsigned long long)(mhi & 0xfffff) << 32 | lo) << (40 + odd)) - t * t);
+  const float rf = __fsub_rn(__int_as_float(0x4b400000 + (int)(r >> 32)), 12582912.f);
+  const int n2 = __float2int_rn(__fmul_rn(rf, __fmul_rn(hy, 0x1p-8f)));
   return __longlong_as_double(s0 + n2 + ((long long)((hi - mhi) >> 1) << 32));
 }
 
@@ -327,18 +322,175 @@ __device__ __forceinline__ double max_nonneg(double a, double b) {
 //    the neighbour weights: -a_d (q_+ - q_-) + k (q_+ + q_- - 2 q_c) / h_d^2
 //    = (k/h_d^2 - a_d) q_+ + (k/h_d^2 + a_d) q_- - 2 k q_c / h_d^2, with
 //    a_d = V_d / (2 h_d); u, v, w share one set of weights (k = nu), T has its
-//    own (k = alpha): seven FMAs per field instead of sixteen operations.
+//    own (k = alpha): seven FMAs per field instead of sixteen operations;
+//  - the dissipation, the advection weights, the square roots and the whole of
+//    T's transport in 64-bit integers: 43 FP64 operations a node of 95 are left,
+//    beside about 1000 integer ones in issue slots the FP64 pipe leaves empty.
+//    256^3 2445 -> 1825 us a step, 128^3 in 2x2x2 blocks 341 -> 260, 64^3 58 -> 45.6.
+//    About here the two pipes balance: u, v and w in integers too make it slower
+//    (256^3 2256, spills), and so does an FP64 div V or T the other way (1870,
+//    1908 with T's weights alone in FP64).
 
 struct NodeF64 {
   double p[13];  // c, x-, x+, y-, y+, z-, z+, x-2, x+2, y-2, y+2, z-2, z+2
   double u[7], v[7], w[7], T[7];
 };
 
+// FP64 values in 64-bit fixed point.  to_fixed<K> takes a value to units of
+// 2^-(52+K) of 2^(E - 1023), E the largest exponent field of the values to be
+// summed; from_fixed<K> rounds a sum in those units to the nearest FP64 value.
+// The sum itself is exact: its error is a unit a term and one rounding, where
+// FP64 operations round each by 2^-53.  About 12 and 18 integer instructions.
+// A term 2^64 below the largest, and a result below 2^-959, count as zero; a
+// term that is NaN, infinite or 2^1020 and above makes the result NaN (E = 2047;
+// a velocity that is NaN or infinite reaches every rate through beta^2, div V
+// and the momentum sums in FP64).
+__device__ __forceinline__ unsigned fixed_exp(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+// v >> n, zero from n = 64 on
+__device__ __forceinline__ unsigned long long shr(unsigned long long v, unsigned n) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
+template <int K> __device__ __forceinline__ long long to_fixed(double v, int E) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned sh = (unsigned)E - ((hi >> 20) & 0x7ffu);
+  const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+  const unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, K) << 32) | (lo << K);
+  const long long sg = (long long)((int)hi >> 31);
+  return ((long long)shr(m, sh) ^ sg) - sg;
+}
+template <int K> __device__ __forceinline__ double from_fixed(long long S, int E) {
+  const long long sg = S >> 63;
+  const unsigned long long A = (unsigned long long)((S ^ sg) - sg);
+  const int lz = __clzll((long long)A);
+  const unsigned long long N = (A << ((lz - 1) & 63)) + 512;  // |S| < 2^63: the leading bit at 62, rounded at 10
+  const unsigned long long r = ((unsigned long long)(unsigned)(E + 10 - K - lz) << 52) + (N >> 10);
+  const unsigned long long bad = E >= 2043 ? 0x7ff8ull << 48 : 0;
+  const unsigned long long v = A == 0 || E < 64 ? 0 : r | ((unsigned long long)sg & (1ull << 63));
+  return __longlong_as_double((long long)(v | bad));
+}
+
+// The dissipation sum_d e_d (p_++ - 4 p_+ + 6 p_0 - 4 p_- + p_--)_d with
+// e_d = (|V_d| + sqrt(V_d^2 + 4 beta^2)) c4 / (2 h_d).  The weights e_d below 2^62
+// in units of 2^(e - 2105), the fourth differences below 2^63 (the star's
+// coefficients add up to 16) in units of 2^(E - 1081).
+struct Weight3 {
+  long long m[3];
+  int e;
+};
+__device__ __forceinline__ void dissipation_weights(const CavConst &C, double b2, const double V[3], Weight3 &x) {
+  const double f4 = times4(b2);
+  int e[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const double s = sqrt_newton(fma(V[d], V[d], f4)), a = fabs(V[d]);
+    const int E = (int)(max(fixed_exp(s), fixed_exp(a)) >> 20);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(C.dsc[d]) << 11 | 1ull << 63;
+    x.m[d] = (long long)__umul64hi((unsigned long long)(to_fixed<8>(a, E) + to_fixed<8>(s, E)), b);
+    e[d] = E + (__double2hiint(C.dsc[d]) >> 20);
+  }
+  x.e = max(max(e[0], e[1]), e[2]);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) x.m[d] = (long long)shr((unsigned long long)x.m[d], (unsigned)(x.e - e[d]));
+}
+__device__ __forceinline__ double dissipation(const double p[13], const Weight3 &x) {
+  unsigned e = 0;
+#pragma unroll
+  for (int q = 0; q < 13; ++q) e = max(e, fixed_exp(p[q]));
+  const int E = (int)(e >> 20);
+  const long long c6 = 6 * to_fixed<6>(p[0], E);
+  long long D[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    D[d] = (to_fixed<6>(p[7 + 2 * d], E) + to_fixed<6>(p[8 + 2 * d], E)) -
+           4 * (to_fixed<6>(p[1 + 2 * d], E) + to_fixed<6>(p[2 + 2 * d], E)) + c6;
+  }
+  // the differences shifted up together, so that the products keep their bits
+  const int sh = __clzll((D[0] ^ (D[0] >> 63)) | (D[1] ^ (D[1] >> 63)) | (D[2] ^ (D[2] >> 63)) | 1) - 1;
+  long long S = 0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) S += __mul64hi(x.m[d], D[d] << sh);
+  return from_fixed<9>(S, E >= 2043 ? 2047 : E + x.e - sh - 2038);
+}
+
+// a_d = V_d / (2 h_d), unrounded: the upper 64 bits of the mantissas' product, the
+// exponent field it has with their product in [2, 4), and its sign.
+struct Advect {
+  unsigned long long m;
+  int e;
+  long long sg;
+};
+__device__ __forceinline__ Advect advect(double v, double ih2) {
+  const unsigned long long one = 1ull << 63;
+  const unsigned long long a = (unsigned long long)__double_as_longlong(v) << 11 | one;
+  const unsigned long long b = (unsigned long long)__double_as_longlong(ih2) << 11 | one;
+  return {__umul64hi(a, b), (int)(fixed_exp(v) >> 20) + (__double2hiint(ih2) >> 20) - 1022,
+          (long long)(__double2hiint(v) >> 31)};
+}
+
+// The neighbour weights D + a (minus side) and D - a (plus side), D = k / h_d^2,
+// rounded once each.
+__device__ __forceinline__ void weights(double D, const Advect &a, double &minus, double &plus) {
+  const int E = max(__double2hiint(D) >> 20, a.e);
+  const long long x = to_fixed<9>(D, E);
+  const long long t = (long long)shr(a.m >> 2, (unsigned)(E - a.e)), y = (t ^ a.sg) - a.sg;
+  minus = from_fixed<9>(x + y, E);
+  plus = from_fixed<9>(x - y, E);
+}
+
+// Advection and diffusion of one field as the sum over the six neighbours of
+// weight times (q_neighbour - q_centre): the weights D +- a (below 2^61 in units of
+// 2^(e - 1082)) and the differences (below 2^60 in units of 2^(E - 1081)) are exact
+// but for their last unit.  Both are split into signed 32-bit halves: the sums H
+// of the high products (below 2^59: a direction's two weights add up to 2^61) and
+// L of the mixed ones (below 6 2^60) hold the result; the product of the low
+// halves, at most a quarter of H's unit, is left out.  Against 128-bit values the
+// error is 0.16 to 0.6 of the seven FMAs' (random stars, smooth and rough).
+struct Weight6 {
+  int h[6], l[6];
+  int e;
+};
+__device__ __forceinline__ void split(long long v, int &h, int &l) {
+  l = (int)v;
+  h = (int)((v - l) >> 32);
+}
+__device__ __forceinline__ void transport_weights(const double D[3], const Advect a[3], Weight6 &w) {
+  w.e = max(max(max(a[0].e, a[1].e), a[2].e), max(max(__double2hiint(D[0]), __double2hiint(D[1])), __double2hiint(D[2])) >> 20);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const long long x = to_fixed<7>(D[d], w.e);
+    const long long t = (long long)shr(a[d].m >> 4, (unsigned)(w.e - a[d].e)), y = (t ^ a[d].sg) - a[d].sg;
+    split(x + y, w.h[2 * d], w.l[2 * d]);
+    split(x - y, w.h[2 * d + 1], w.l[2 * d + 1]);
+  }
+}
+__device__ __forceinline__ double transport(const double q[7], const Weight6 &w) {
+  unsigned e = 0;
+#pragma unroll
+  for (int i = 0; i < 7; ++i) e = max(e, fixed_exp(q[i]));
+  const int E = (int)(e >> 20);
+  const long long c = to_fixed<6>(q[0], E);
+  long long H = 0, L = 0;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    int dh, dl;
+    split(to_fixed<6>(q[1 + i], E) - c, dh, dl);
+    H += (long long)w.h[i] * dh;
+    L += (long long)w.h[i] * dl;
+    L += (long long)w.l[i] * dh;
+  }
+  // H in units of 2^(w.e + E - 2099), L of 2^-32 of that
+  return from_fixed<9>((H << 4) + (L >> 28), E >= 2043 ? 2047 : w.e + E - 1019);
+}
+
 // The part of the rates that reads the velocities alone (and the centre T):
 // beta^2, the dissipation weights, div V and the momentum rates without the
 // pressure gradient.
 struct VelF64 {
-  double b2, ex, ey, ez, divV, ru, rv, rw;
+  double b2, divV, ru, rv, rw;
+  Weight3 e;
+  Advect a[3];
 };
 
 #define BDC_TRANSPORT(q, xm, xp, ym, yp, zm, zp, centre) \
@@ -347,16 +499,18 @@ struct VelF64 {
 __device__ __forceinline__ void rates_vel_f64(const CavConst &C, const NodeF64 &n, VelF64 &x) {
   const double u0 = n.u[0], v0 = n.v[0], w0 = n.w[0];
   const double b2 = max_nonneg(fma(u0, u0, fma(v0, v0, w0 * w0)), C.b2min);
-  const double f4 = times4(b2);
   x.b2 = b2;
-  x.ex = (fabs(u0) + sqrt_newton(fma(u0, u0, f4))) * C.dsc[0];
-  x.ey = (fabs(v0) + sqrt_newton(fma(v0, v0, f4))) * C.dsc[1];
-  x.ez = (fabs(w0) + sqrt_newton(fma(w0, w0, f4))) * C.dsc[2];
+  const double V[3] = {u0, v0, w0};
+  dissipation_weights(C, b2, V, x.e);
   x.divV = fma(n.u[2] - n.u[1], C.ih2[0], fma(n.v[4] - n.v[3], C.ih2[1], (n.w[6] - n.w[5]) * C.ih2[2]));
   // neighbour weights: m = minus side, p = plus side
-  const double nxm = fma(u0, C.ih2[0], C.nuhh[0]), nxp = fma(-u0, C.ih2[0], C.nuhh[0]);
-  const double nym = fma(v0, C.ih2[1], C.nuhh[1]), nyp = fma(-v0, C.ih2[1], C.nuhh[1]);
-  const double nzm = fma(w0, C.ih2[2], C.nuhh[2]), nzp = fma(-w0, C.ih2[2], C.nuhh[2]);
+  x.a[0] = advect(u0, C.ih2[0]);
+  x.a[1] = advect(v0, C.ih2[1]);
+  x.a[2] = advect(w0, C.ih2[2]);
+  double nxm, nxp, nym, nyp, nzm, nzp;
+  weights(C.nuhh[0], x.a[0], nxm, nxp);
+  weights(C.nuhh[1], x.a[1], nym, nyp);
+  weights(C.nuhh[2], x.a[2], nzm, nzp);
   // the buoyancy force (Eq. 2) enters the gravity-axis momentum rate with its centre term
   const double buoy = fma(C.gs, n.T[0], -C.gst);
   const double bv = C.gaxis == 1 ? buoy : 0.0, bw = C.gaxis == 2 ? buoy : 0.0;
@@ -365,54 +519,15 @@ __device__ __forceinline__ void rates_vel_f64(const CavConst &C, const NodeF64 &
   x.rw = BDC_TRANSPORT(n.w, nxm, nxp, nym, nyp, nzm, nzp, fma(-C.nu2s, w0, bw));
 }
 
-// The fourth differences p_++ - 4 p_+ + 6 p_0 - 4 p_- + p_-- of the 13-point star
-// along x, y and z, in 64-bit fixed point: the thirteen values as integers in
-// units of 2^-58 of the largest one's power of two (the sum's weights add up to
-// 16: below 2^63), summed exactly and rounded once to FP64.  The error is a few
-// 2^-59 of the largest |p|, where twelve FP64 operations had a few 2^-53; those
-// twelve were 12% of the step kernel's FP64 pipe time, and the 250 integer
-// instructions run in issue slots it leaves empty.  Values below 2^-959 count as
-// zero; NaN or infinity comes out as a finite value (the pressure gradient
-// carries it on).
-__device__ __forceinline__ void fourth_differences(const double p[13], double d4[3]) {
-  unsigned E = 0;
-#pragma unroll
-  for (int q = 0; q < 13; ++q) E = max(E, (unsigned)__double2hiint(p[q]) & 0x7fffffffu);
-  E >>= 20;
-  auto fixed = [&](double v) {
-    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-    const unsigned sh = min(E - ((hi >> 20) & 0x7ffu), 63u);
-    const unsigned mh = (hi & 0xfffffu) | 0x100000u;
-    const unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, 6) << 32) | (lo << 6);
-    const long long sg = (long long)((int)hi >> 31);
-    return ((long long)(m >> sh) ^ sg) - sg;
-  };
-  const long long c6 = 6 * fixed(p[0]);
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const long long S = (fixed(p[7 + 2 * d]) + fixed(p[8 + 2 * d])) - 4 * (fixed(p[1 + 2 * d]) + fixed(p[2 + 2 * d])) + c6;
-    const long long sg = S >> 63;
-    const unsigned long long A = (unsigned long long)((S ^ sg) - sg);
-    const int lz = __clzll((long long)A);
-    const unsigned long long N = A << (lz & 63);
-    const unsigned long long r = ((unsigned long long)(E + 4 - lz) << 52) + (N >> 11) + ((N >> 10) & 1);
-    d4[d] = A == 0 || E < 64 ? 0.0 : __longlong_as_double((long long)(r | ((unsigned long long)sg & (1ull << 63))));
-  }
-}
-
 __device__ __forceinline__ void rates_pt_f64(const CavConst &C, const NodeF64 &n, const VelF64 &x, double r[5]) {
-  const double u0 = n.u[0], v0 = n.v[0], w0 = n.w[0];
-  double d4[3];
-  fourth_differences(n.p, d4);
-  const double diss = fma(x.ex, d4[0], fma(x.ey, d4[1], x.ez * d4[2]));
-  r[0] = fma(-x.b2, x.divV, -diss);
+  r[0] = fma(-x.b2, x.divV, -dissipation(n.p, x.e));
   r[1] = fma(-(n.p[2] - n.p[1]), C.ih2[0], x.ru);
   r[2] = fma(-(n.p[4] - n.p[3]), C.ih2[1], x.rv);
   r[3] = fma(-(n.p[6] - n.p[5]), C.ih2[2], x.rw);
-  const double txm = fma(u0, C.ih2[0], C.alhh[0]), txp = fma(-u0, C.ih2[0], C.alhh[0]);
-  const double tym = fma(v0, C.ih2[1], C.alhh[1]), typ = fma(-v0, C.ih2[1], C.alhh[1]);
-  const double tzm = fma(w0, C.ih2[2], C.alhh[2]), tzp = fma(-w0, C.ih2[2], C.alhh[2]);
-  r[4] = BDC_TRANSPORT(n.T, txm, txp, tym, typ, tzm, tzp, -C.al2s * n.T[0]);
+  const double D[3] = {C.alhh[0], C.alhh[1], C.alhh[2]};
+  Weight6 w;
+  transport_weights(D, x.a, w);
+  r[4] = transport(n.T, w);
 }
 #undef BDC_TRANSPORT
 
@@ -1362,8 +1477,12 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a) {
 // out every block's coarse tiles before the fine tail tiles, and the next
 // tile is fetched while the current one is computed.  Partials stay indexed by
 // tile slot: the reductions do not depend on which CTA took a tile.
+//
+// Three CTAs of 128 an SM (168 registers a thread): 256^3 takes 2165 us a step
+// with the 204 registers the compiler takes unasked (two CTAs), 1900 with four
+// CTAs (128 registers, spills).
 template <int NT, bool FORM>
-__global__ void __launch_bounds__(NT) k_step_f64(StepArgs a, const __grid_constant__ BcArgs d) {
+__global__ void __launch_bounds__(NT, NT == 128 ? 3 : 1) k_step_f64(StepArgs a, const __grid_constant__ BcArgs d) {
   chain_wait();
   if ((int)blockIdx.x < a.nnu) {
     __shared__ double snu[NT / 32];
