@@ -7,7 +7,8 @@
 //               interior node of every block, walls (Section 2) formed where
 //               they are read; FP64 residual sums as per-CTA partials, the
 //               spectral-radius maximum of the new state as an atomic maximum;
-//   k_between   what the next step waits for: dt from that maximum, the centre
+//   k_between   what the next step waits for (undivided small FP64 cavities
+//               see to it in the step itself): dt from that maximum, the centre
 //               shift, and with cut faces the ghost layers of the new state
 //               from the neighbours' layers (Section 4.5, Listings 1-2, V3: p
 //               at depth 2, u, v, w, T at depth 1);
@@ -154,20 +155,26 @@ inline void set_cav_physics(CavConst &C, const int gn[3], const cavity_params &p
   C.gaxis = p.gravity_axis;
 }
 
+// Steps of an undivided FP64 cavity follow one another without a kernel between
+// them: step s takes dt from the maximum step s - 1 left in its slot, writes its
+// own, and clears the one after, which step s - 2 wrote and step s - 1 read.
+// Other steps use slot 0.
+constexpr int kStepSlots = 3;
+
 struct CavState {
   double dt;         // dt of the next step
-  double c;          // pending centre-pressure shift of the stored p
+  double c;          // pending centre-pressure shift of the stored p (after dt: step_tile_f64 reads the pair)
   double t;          // simulated time
   long long step;    // steps taken
   double res[5];     // RMS dq/dt of the last step
   double nu_hot, nu_cold;
   int flags;         // bit 0: non-finite residual or spectral radius
   int pad;
-  // for the step in flight (zero before it): the largest spectral bound of its
-  // new state, and the FP64 step's largest published dt-filter floor
-  // (float_key ^ 0x80000000, 0 = none)
-  double smax;
-  unsigned int sfl, pad2;
+  // for the step in flight (zero before it), in the step's slot (kStepSlots):
+  // the largest spectral bound of its new state, and the FP64 step's largest
+  // published dt-filter floor (float_key ^ 0x80000000, 0 = none)
+  double smax[kStepSlots];
+  unsigned int sfl[kStepSlots], pad2;
   double dt0;        // dt as the last finalise left it (dt itself moves on within a graph)
   double nu_sum;     // sum of nu_hot over the steps (the adjoint's forward run zeroes it)
 };
@@ -653,6 +660,9 @@ struct StepArgs {
   int skip_shell;              // 1: leave the nodes within two layers of a cut face to k_shell_f64
   int ncoarse;                 // coarse tiles of all blocks (scheduling indices below it)
   int nnu;                     // the first CTAs: the x walls' Nusselt sums of the state read here
+  int slot;                    // of this step's maximum, dt-filter floor and tile counter
+  int chained;                 // 1: dt and the centre shift from the step before (no kernel in between)
+  double *dt_out;              // chained: dt goes here, too (null: nowhere)
 };
 
 // p of one stored node through L2
@@ -675,9 +685,9 @@ __device__ __forceinline__ double centre_mean(int n, const double *v) {
   return csum * (n == 8 ? 0.125 : n == 4 ? 0.25 : n == 2 ? 0.5 : 1.0);
 }
 
-__device__ __forceinline__ void step_max(CavState &st, double smax) {
+__device__ __forceinline__ void step_max(double *slot, double smax) {
   // positive values order like their bit patterns
-  atomicMax((unsigned long long *)&st.smax, (unsigned long long)__double_as_longlong(smax));
+  atomicMax((unsigned long long *)slot, (unsigned long long)__double_as_longlong(smax));
 }
 
 // A programmatic dependent: every earlier kernel of the chain has finished
@@ -770,11 +780,10 @@ __device__ __forceinline__ double adiabatic_T(double T1, double T2) { return div
 // FP64 operations in the warps that hold a node next to an x wall, a few in the
 // first and last planes.  u = v = w = 0 and the isothermal T never change and
 // stay stored.  Large cavities read stored walls, which k_between writes: the
-// line is at 64 tile planes an SM, where forming them takes 3.5% of the step
-// (128^3: 390 us a step, 381 stored) and storing them 5 us; at 64^3 the step is
-// 62 us with walls formed, 59 without any.
+// line is at 64 tile planes an SM: 128^3 263 us a step with walls formed, 257
+// stored, 256^3 1890 and 1843; 64^3 45 either way, 32^3 11.6 and 13.1.
 template <int NT, bool FORM>
-__device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float &wfloor, int &fcav) {
+__device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, const double *dc, float &wfloor, int &fcav) {
   const TileRef tile = tile_ref(a.blocks, a.nblocks, a.ncoarse, cta);
   const BlockDev &B = a.blocks[tile.b];
   const CavConst &C = a.cc[B.cav];
@@ -787,7 +796,7 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
   // at or below an exact spectral value some warp recorded): warps far from
   // the maximum start near it too
   if (a.mode == 0) {
-    const unsigned u = *(volatile const unsigned *)&st.sfl;
+    const unsigned u = *(volatile const unsigned *)&st.sfl[a.slot];
     if (u != 0u) wfloor = fmaxf(wfloor, key_float((int)(u ^ 0x80000000u)));
   }
   float published = wfloor;
@@ -796,8 +805,8 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
   const int k0 = tile.k0;
   const int k1 = tile.k1;
   const bool active = j <= B.ny;
-  const double dt = st.dt;
-  const double cshift = st.c;
+  if (!FORM || !dc) dc = &st.dt;
+  const double dt = dc[0], cshift = dc[1];
 
   const double *__restrict__ src = (const double *)B.base[a.parity];
   double *__restrict__ dst = (double *)B.base[a.parity ^ 1];
@@ -915,7 +924,7 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
         wfloor = fmaxf(wfloor, key_float(__reduce_max_sync(am, float_key(best))));
         if (wfloor > published) {  // publish a rise for the other warps
           if ((int)(threadIdx.x & 31) == __ffs(am) - 1)
-            atomicMax(&st.sfl, (unsigned)float_key(wfloor) ^ 0x80000000u);
+            atomicMax(&st.sfl[a.slot], (unsigned)float_key(wfloor) ^ 0x80000000u);
           published = wfloor;
         }
       } else {
@@ -955,7 +964,7 @@ __device__ __forceinline__ void step_tile_f64(const StepArgs &a, int cta, float 
       unsigned long long m = redm[0];
       for (int q = 1; q < NT / 32; ++q) m = redm[q] > m ? redm[q] : m;
       v = __longlong_as_double((long long)m);
-      if (s == 0 && a.mode == 0) step_max(st, v);
+      if (s == 0 && a.mode == 0) step_max(&st.smax[a.slot], v);
     }
     if (s == 0) a.partials[(long long)tile.slot * kPartStride + f] = v;
   }
@@ -1078,7 +1087,7 @@ struct BcArgs {
   double *bc_partials;        // [k_bc cta][2]
   unsigned int *counter;      // [nsteps][ncav] CTAs done, then [ncav] steps done (zero between launches)
   const double *t_wall;       // hot walls then cold walls, per cavity at wall_off
-  unsigned int *tile_counter; // the FP64 step's tile counter: reset here
+  unsigned int *tile_counter; // the FP64 step's tile counters (kStepSlots): reset here
   long long shell_begin, shell_end;  // k_shell_f64 partial slots of this step (single cavity; empty if equal)
   int parity;                 // buffer set holding the new state
   int nslices;                // finalise CTAs per cavity (1 .. kFinSlices)
@@ -1091,6 +1100,7 @@ struct BcArgs {
   double *mid;                // [nsteps][ncav][kFinSlices][8] slice totals
   StepResult *rec;            // [nsteps][ncav]
   double *dt_out;             // k_between: the next step's dt goes here, too (null: nowhere)
+  int slot;                   // k_between: the slot of the step before it
   StepRecord *log;            // after a step: the step log (host memory), or null
   long long log_cap;          // its records per cavity
   int mode;                   // 0 after a step, 1 after init / set_fields,
@@ -1385,9 +1395,11 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a) {
     if (f == 5) {
       out.dt = C.cfl / t;
       if (last_step) {  // the next step starts from this state
-        st.smax = 0.0;
-        st.sfl = 0u;
-        if (cav == 0) *a.tile_counter = 0u;
+        for (int q = 0; q < kStepSlots; ++q) {
+          st.smax[q] = 0.0;
+          st.sfl[q] = 0u;
+          if (cav == 0) a.tile_counter[q] = 0u;
+        }
       }
     }
     if (f >= 6) {
@@ -1492,15 +1504,42 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 3 : 1) k_step_f64(StepArgs a, 
   float wfloor = -INFINITY;
   int fcav = -1;
   if (!a.tile_counter) {
-    step_tile_f64<NT, FORM>(a, blockIdx.x, wfloor, fcav);
+    step_tile_f64<NT, FORM>(a, blockIdx.x, nullptr, wfloor, fcav);
     return;
+  }
+  const double *dc = nullptr;
+  if (FORM && a.chained) {
+    // what k_between does for the others, in every CTA (one cavity, one block);
+    // starting the first tile's loads before it changes nothing (32^3 11.7 us)
+    __shared__ double s_dc[2];
+    dc = s_dc;
+    CavState &st = a.cs[0];
+    if (threadIdx.x == 0) {
+      const CavConst &C = a.cc[0];
+      const double *p = (const double *)a.blocks[0].base[a.parity];
+      double c[kMaxCentre];
+#pragma unroll
+      for (int q = 0; q < kMaxCentre; ++q) c[q] = q < C.ncentre ? __ldcg(p + C.centre_off[q]) : 0.0;
+      s_dc[1] = centre_mean(C.ncentre, c);
+    } else if (threadIdx.x == 32) {
+      const double dt = a.cc[0].cfl / __ldcg(&st.smax[(a.slot + kStepSlots - 1) % kStepSlots]);
+      s_dc[0] = dt;
+      if ((int)blockIdx.x == a.nnu) {
+        const int next = (a.slot + 1) % kStepSlots;
+        st.smax[next] = 0.0;
+        st.sfl[next] = 0u;
+        a.tile_counter[next - a.slot] = 0u;
+        if (a.dt_out) *a.dt_out = dt;
+      }
+    }
+    __syncthreads();
   }
   // the first tile of each CTA is its own index; the counter goes on from the grid's size
   __shared__ int s_tile[2];
   int tile = blockIdx.x - a.nnu;
   for (int n = 0; tile < a.ntiles; n ^= 1) {
     if (threadIdx.x == 0) s_tile[n] = (int)(gridDim.x - a.nnu + atomicAdd(a.tile_counter, 1u));
-    step_tile_f64<NT, FORM>(a, tile, wfloor, fcav);
+    step_tile_f64<NT, FORM>(a, tile, dc, wfloor, fcav);
     __syncthreads();
     tile = s_tile[n];
   }
@@ -1739,13 +1778,15 @@ __global__ void __launch_bounds__(kBetweenThreads) k_between(ExchArgs a, BcArgs 
     if (tid == 0) st.c = centre_mean(C.ncentre, shc);
   }
   if (tid == 32) {
-    const double t = __ldcg(&st.smax);
+    const double t = __ldcg(&st.smax[b.slot]);
     const double dt = C.cfl / t;
     st.dt = dt;
     if (b.dt_out) *b.dt_out = dt;
-    st.smax = 0.0;
-    st.sfl = 0u;
-    if (blockIdx.x == 0) *b.tile_counter = 0u;
+    for (int q = 0; q < kStepSlots; ++q) {
+      st.smax[q] = 0.0;
+      st.sfl[q] = 0u;
+      if (blockIdx.x == 0) b.tile_counter[q] = 0u;
+    }
   }
 }
 

@@ -468,7 +468,7 @@ __device__ __forceinline__ void f32_partials(double *partials, CavState &st, int
     double acc = red[0][tid];
     for (int q = 1; q < NT / 32; ++q) acc = (tid == 5) ? fmax(acc, red[q][tid]) : acc + red[q][tid];
     partials[(long long)cta * kPartStride + tid] = acc;
-    if (tid == 5) step_max(st, acc);
+    if (tid == 5) step_max(st.smax, acc);
   }
 }
 

@@ -167,7 +167,7 @@ struct cavity {
   StepResult *d_rec = nullptr;  // [kGraphMax][ncav]
   StepRecord *d_log = nullptr;  // the step log (device address of caller-owned host memory), or null
   long long log_cap = 0;
-  unsigned int *d_counter = nullptr;  // the FP64 step's tile counter, then BcArgs::counter
+  unsigned int *d_counter = nullptr;  // the FP64 step's tile counters (kStepSlots), then BcArgs::counter
   int nsm = 0;                        // SMs of the device
   int persist_ctas = 0;               // CTAs of the persistent FP64 step kernel that fit on the GPU
   void *d_fields = nullptr, *d_xbuf = nullptr;
@@ -249,15 +249,13 @@ int check_desc(const cavity_desc &d) {
 // planes above it in fine chunks scheduled after every block's coarse tiles.
 //
 // FP64: what counts is the number of tile planes (128 nodes x 1 plane) an SM
-// gets.  A tile plane takes its SM's FP64 pipe about 3.3 us whatever else the
-// SM runs; a tile's own cost (queue loads, tile look-up, reduction) is about a
-// third of one.  So large cavities take 8-plane tiles with 2-plane ones in the
+// gets.  A tile plane takes an SM about 2.1 us whatever else it runs (256^3); a
+// tile's own cost (queue loads, tile look-up, reduction) is about a third of one.  So large cavities take 8-plane tiles with 2-plane ones in the
 // end, small ones 4-plane and 1-plane tiles, and the fine tiles hold 8 planes
 // an SM (all of a cavity of up to 38^3), enough to level what the coarse ones
-// leave.  Measured per step, chunks of 8 and 8-plane tails before: 32^3
-// 59.4 -> 20.6 us, 64^3 137 -> 66.5, 128^3 410 (8 planes, fine tiles in the
-// last 8 of 128 only) -> 384; the other side of the line: 4 planes at 256^3
-// 2835 against 2798 us, 8 planes at 64^3 80 against 66.5.
+// leave.  Measured per step with either, 4-plane tiles first: 32^3 11.6 and
+// 14.9 us, 64^3 45 and 65, 97x65x50 51 and 64, 128^3 265 and 257, 256^3 1951 and
+// 1843.
 //
 // FP32: tail chunks of at most kFineKC32 planes, only in blocks deeper than one
 // chunk (a shallower block is one chunk: the ring's fill is paid per tile).
@@ -586,7 +584,7 @@ int alloc_device(cavity *h) {
   CK(cudaMalloc(&h->d_bc_part, sizeof(double) * 2 * std::max(std::max(1, h->n_bc), h->f32 ? 0 : kGraphMax * h->n_nu)));
   CK(cudaMalloc(&h->d_fin, sizeof(double) * kGraphMax * 8 * kFinSlices * h->ncav));
   CK(cudaMalloc(&h->d_rec, sizeof(StepResult) * kGraphMax * h->ncav));
-  const size_t counter_bytes = sizeof(unsigned int) * (1 + (size_t)(kGraphMax + 1) * h->ncav);
+  const size_t counter_bytes = sizeof(unsigned int) * (kStepSlots + (size_t)(kGraphMax + 1) * h->ncav);
   CK(cudaMalloc(&h->d_counter, counter_bytes));
   CK(cudaMemsetAsync(h->d_counter, 0, counter_bytes, h->stream));
   {
@@ -640,6 +638,9 @@ StepArgs step_args(cavity *h, int parity, int mode, int s) {
   a.ncoarse = h->n_coarse;
   a.skip_shell = 0;
   a.nnu = 0;
+  a.slot = 0;
+  a.chained = 0;
+  a.dt_out = nullptr;
   return a;
 }
 
@@ -660,7 +661,7 @@ BcArgs bc_args(cavity *h, int parity, int mode) {
   a.faces = h->d_wall;
   a.nfaces = (int)h->hwall.size();
   a.cc = h->d_cc; a.cs = h->d_cs; a.ncav = h->ncav;
-  a.step_partials = h->d_step_part; a.bc_partials = h->d_bc_part; a.counter = h->d_counter + 1;
+  a.step_partials = h->d_step_part; a.bc_partials = h->d_bc_part; a.counter = h->d_counter + kStepSlots;
   a.tile_counter = h->d_counter;
   a.t_wall = h->d_twall; a.parity = parity; a.mode = mode;
   a.shell_begin = a.shell_end = 0;
@@ -673,6 +674,7 @@ BcArgs bc_args(cavity *h, int parity, int mode) {
   a.part_stride = (long long)h->part_cap * kPartStride;
   a.bc_stride = 2LL * h->n_nu;
   a.dt_out = nullptr;
+  a.slot = 0;
   a.mid = h->d_fin;
   a.rec = h->d_rec;
   return a;
@@ -738,12 +740,26 @@ cudaError_t launch_step_f32(cavity *h, const StepF32Args &a, bool pdl) {
   return cudaErrorInvalidValue;
 }
 
+// Whether a step takes dt and the centre shift from the one before it by itself
+// (an undivided FP64 cavity whose walls the step forms) instead of from a
+// k_between: 32^3 11.6 us a step (12.2 with it), 16^3 9.6 (10.9).  The FP32-mixed
+// step has no register left for it (126 of 128 a thread; the code costs it 7%),
+// and an exchange or stored walls need the kernel in between anyway.
+bool self_chained(const cavity *h) { return !h->f32 && h->ncav == 1 && h->n_cut == 0 && h->form_walls; }
+
+void chain_step(StepArgs &a, int s) {  // step s of a sequence
+  a.slot = s % kStepSlots;
+  a.chained = s > 0;
+  a.tile_counter += a.slot;
+}
+
 // The kernel of step `s` of a graph, reading buffer set `parity`.  From the
-// second step on it is a programmatic dependent of the k_between before it; the
-// first gets a plain launch.
+// second step on it is a programmatic dependent of the step or the k_between
+// before it; the first gets a plain launch.
 cudaError_t launch_step_kernel(cavity *h, int parity, int s) {
   if (!h->f32) {
     StepArgs a = step_args(h, parity, 0, s);
+    if (self_chained(h)) chain_step(a, s);
     int ctas = 0;
     BcArgs d = fin_args(h, parity, 1, &ctas);
     if (s > 0) {
@@ -876,7 +892,8 @@ int launch_steps(cavity *h, int parity, int nsteps) {
     }
     CK(launch_step_kernel(h, parity, s));
     // (the state a graph leaves has its ghost layers and stored walls, too)
-    if (s < nsteps - 1 || h->n_cut > 0 || (!h->f32 && !h->form_walls)) CK(launch_between(h, parity ^ 1, true));
+    if ((s < nsteps - 1 && !self_chained(h)) || h->n_cut > 0 || (!h->f32 && !h->form_walls))
+      CK(launch_between(h, parity ^ 1, true));
     if (s == nsteps - 1) CK(launch_finalize(h, parity ^ 1, nsteps, true));
   }
   return CAVITY_OK;
@@ -1126,6 +1143,8 @@ cudaError_t launch_recompute(cavity *h, int s, bool pdl) {
   const AdjointStore &A = h->adj;
   if (!h->f32) {
     StepArgs a = step_args(h, 0, 0, 0);
+    if (self_chained(h)) chain_step(a, s);
+    a.dt_out = A.dts + s;
     a.blocks = A.seg_blocks + s;
     return launch_step_f64(h, a, BcArgs{}, pdl);
   }
@@ -1135,13 +1154,15 @@ cudaError_t launch_recompute(cavity *h, int s, bool pdl) {
   return launch_step_f32(h, a, pdl);
 }
 
-// dt, the centre shift (and stored walls) of slot s for the recomputed step after it
+// dt, the centre shift (and stored walls) of slot s for the recomputed step after it,
+// or for the reverse step from the segment's last state
 cudaError_t launch_recompute_between(cavity *h, int s) {
   const AdjointStore &A = h->adj;
   ExchArgs x = exch_args(h, 0);
   BcArgs b = bc_args(h, 0, 3);
   x.blocks = b.blocks = A.seg_blocks + s;
   b.dt_out = A.dts + s;
+  b.slot = self_chained(h) ? (s - 1) % kStepSlots : 0;
   const int grid = 1 + (h->f32 || h->form_walls ? 0 : h->n_bc);
   if (h->f32) return launch_chained(h, true, k_between<float>, grid, dim3(kBetweenThreads), 0, x, b, 0);
   return launch_chained(h, true, k_between<double>, grid, dim3(kBetweenThreads), 0, x, b, 0);
@@ -1775,7 +1796,7 @@ int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *gr
     CK(cudaMemcpyAsync(A.dts, &h->d_cs->dt, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
     for (int s = 0; s + 1 < len; ++s) {
       CK(launch_recompute(h, s, s > 0));
-      CK(launch_recompute_between(h, s + 1));
+      if (!self_chained(h) || s + 2 == len) CK(launch_recompute_between(h, s + 1));
     }
     // the walls (formed by the step where it reads them) of every stored state
     BcArgs ba = bc_args(h, 0, 3);
