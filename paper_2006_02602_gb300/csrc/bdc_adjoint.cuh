@@ -148,8 +148,12 @@ struct AdjCoef {
   R r[5], a[3], D[3], b, b2, lam[3], isq[3];
   bool floored;
 };
-// (D0: the first axis wanted; 2 for a plane that only passes z terms)
-template <int D0, class R>
+// lambda_d without 1 / sqrt: the square root is no FP64-pipe operation (sqrt_newton)
+__device__ __forceinline__ double lambda_r(double V, double q) { return 0.5 * (fabs(V) + sqrt_newton(q)); }
+__device__ __forceinline__ float lambda_r(float V, float q) { return 0.5f * (fabsf(V) + q * rsqrt_r(q)); }
+// (D0: the first axis wanted; 2 for a plane that only passes z terms.  OWN: isq
+// is wanted)
+template <int D0, bool OWN, class R>
 __device__ __forceinline__ void adj_coef(const AdjK<R> &K, const R V[3], const R y[5], R dt, AdjCoef<R> &c) {
   R b2 = V[0] * V[0] + V[1] * V[1] + V[2] * V[2];
   c.floored = b2 < K.b2min;
@@ -161,11 +165,26 @@ __device__ __forceinline__ void adj_coef(const AdjK<R> &K, const R V[3], const R
 #pragma unroll
   for (int d = D0; d < 3; ++d) {
     const R q = V[d] * V[d] + (R)4 * b2;
-    c.isq[d] = rsqrt_r(q);
-    c.lam[d] = (R)0.5 * (abs_r(V[d]) + q * c.isq[d]);
+    if (OWN) {
+      c.isq[d] = rsqrt_r(q);
+      c.lam[d] = (R)0.5 * (abs_r(V[d]) + q * c.isq[d]);
+    } else {
+      c.lam[d] = lambda_r(V[d], q);
+    }
     c.a[d] = V[d] * K.ih2[d];
     c.D[d] = c.r[0] * K.c4ih[d] * c.lam[d];
   }
+}
+
+// D_z alone: all that the outermost plane at either end of a chunk passes on.  FP64
+// only, where its 12 FP64 operations instead of 70 count (32^3 51 -> 46 us a reverse
+// step with the halo's square roots, 48^3 131 -> 124); the branch costs the FP32
+// sweep its schedule (128^3 110 -> 127).
+template <class R>
+__device__ __forceinline__ R adj_dz(const AdjK<R> &K, const R V[3], R y0, R dt) {
+  R b2 = V[0] * V[0] + V[1] * V[1] + V[2] * V[2];
+  if (b2 < K.b2min) b2 = K.b2min;
+  return dt * y0 * K.c4ih[2] * lambda_r(V[2], V[2] * V[2] + (R)4 * b2);
 }
 
 // ---------------------------------------------------------------------------
@@ -282,6 +301,7 @@ __global__ void __launch_bounds__(32 * TY, sizeof(R) == 4 ? 2 : 1) k_adj_sweep(c
       for (int d = 0; d < 3; ++d) vz[d][2] = at(qk + pl + (U + d) * fs, o);
     }
     const bool full = k >= k0 && k <= k1;  // uniform
+    const bool outer = sizeof(R) == 8 && (k == k0 - 2 || k == k1 + 2);
     const R V[3] = {vz[0][1], vz[1][1], vz[2][1]};
     R y[5];
 #pragma unroll
@@ -290,10 +310,14 @@ __global__ void __launch_bounds__(32 * TY, sizeof(R) == 4 ? 2 : 1) k_adj_sweep(c
       yn[f] = act && k <= k1 + 1 ? at(Yk + pl + f * fs, o) : (R)0;  // (zero off the interior)
     }
     AdjCoef<R> c;
-    if (full) adj_coef<0>(K, V, y, dt, c);
-    else adj_coef<2>(K, V, y, dt, c);
+    if (full) adj_coef<0, true>(K, V, y, dt, c);
+    else if (!outer) adj_coef<2, false>(K, V, y, dt, c);
     // z: to the planes below (s = 1) and above (s = -1)
-    {
+    if (outer) {  // two planes off the chunk: the fourth difference's outer weight alone
+      const R D = adj_dz(K, V, y[0], dt);
+      if (k < k0) P[4] -= D;
+      else P[0] -= D;
+    } else {
       const R wm = K.nh[2] + c.a[2], wp = K.nh[2] - c.a[2], tm = K.ah[2] + c.a[2], tp = K.ah[2] - c.a[2];
 #pragma unroll
       for (int f = 0; f < 3; ++f) {
@@ -341,7 +365,7 @@ __global__ void __launch_bounds__(32 * TY, sizeof(R) == 4 ? 2 : 1) k_adj_sweep(c
       s[AX][pos] = c.a[0]; s[AY][pos] = c.a[1]; s[DX][pos] = c.D[0]; s[DY][pos] = c.D[1]; s[BB][pos] = c.b;
       if (hpos >= 0) {
         AdjCoef<R> h;
-        adj_coef<0>(K, hV, hy, dt, h);
+        adj_coef<0, false>(K, hV, hy, dt, h);
         s[R1][hpos] = h.r[1]; s[R2][hpos] = h.r[2]; s[R3][hpos] = h.r[3]; s[R4][hpos] = h.r[4];
         s[AX][hpos] = h.a[0]; s[AY][hpos] = h.a[1]; s[DX][hpos] = h.D[0]; s[DY][hpos] = h.D[1]; s[BB][hpos] = h.b;
         if (hin && k < k1) {
