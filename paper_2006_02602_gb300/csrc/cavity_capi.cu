@@ -15,6 +15,7 @@
 #include <cfloat>
 #include <cstdlib>
 #include <cstddef>
+#include <climits>
 #include <cstring>
 #include <new>
 #include <string>
@@ -792,6 +793,12 @@ void launch_walls(cavity *h, int parity) {
   else k_bc<double><<<h->n_bc, kBcThreads, 0, h->stream>>>(b);
 }
 
+FinTail no_tail() {
+  FinTail t{};
+  t.begin = INT_MAX;
+  return t;
+}
+
 // A state refresh (no step): walls with the Nusselt partials, then the
 // reductions, dt among them.
 void launch_refresh(cavity *h, int parity) {
@@ -799,18 +806,22 @@ void launch_refresh(cavity *h, int parity) {
   const int nfin = h->ncav * h->nslices;
   if (h->f32) {
     k_bc<float><<<h->n_bc, kBcThreads, 0, h->stream>>>(b);
-    k_finalize<float><<<nfin, kFinThreads, 0, h->stream>>>(b);
+    k_finalize<float><<<nfin, kFinThreads, 0, h->stream>>>(b, no_tail());
   } else {
     k_bc<double><<<h->n_bc, kBcThreads, 0, h->stream>>>(b);
-    k_finalize<double><<<nfin, kFinThreads, 0, h->stream>>>(b);
+    k_finalize<double><<<nfin, kFinThreads, 0, h->stream>>>(b, no_tail());
   }
 }
 
+// The finalise of `nsteps` steps; the state in buffer set `parity` gets its
+// ghost layers and stored walls in the same launch.
 cudaError_t launch_finalize(cavity *h, int parity, int nsteps, bool pdl) {
   int ctas = 0;
   const BcArgs b = fin_args(h, parity, nsteps, &ctas);
-  if (h->f32) return launch_chained(h, pdl, k_finalize<float>, ctas, dim3(kFinThreads), 0, b);
-  return launch_chained(h, pdl, k_finalize<double>, ctas, dim3(kFinThreads), 0, b);
+  const FinTail t{ctas, h->n_cut, exch_args(h, parity), bc_args(h, parity, 3)};
+  ctas += h->n_cut + (h->f32 || h->form_walls ? 0 : h->n_bc);
+  if (h->f32) return launch_chained(h, pdl, k_finalize<float>, ctas, dim3(kFinThreads), 0, b, t);
+  return launch_chained(h, pdl, k_finalize<double>, ctas, dim3(kFinThreads), 0, b, t);
 }
 
 // What the step after the one that left its state in buffer set `parity` waits
@@ -876,7 +887,7 @@ int launch_step_overlapped(cavity *h, int parity) {
   ba.wall_ctas = h->n_bc;
   ba.shell_begin = h->n_step;
   ba.shell_end = (long long)h->n_step + h->n_shell;
-  k_finalize<double><<<h->ncav * h->nslices + h->n_bc, kFinThreads, 0, h->stream>>>(ba);
+  k_finalize<double><<<h->ncav * h->nslices + h->n_bc, kFinThreads, 0, h->stream>>>(ba, no_tail());
   CK(cudaGetLastError());
   return CAVITY_OK;
 }
@@ -891,10 +902,8 @@ int launch_steps(cavity *h, int parity, int nsteps) {
       continue;
     }
     CK(launch_step_kernel(h, parity, s));
-    // (the state a graph leaves has its ghost layers and stored walls, too)
-    if ((s < nsteps - 1 && !self_chained(h)) || h->n_cut > 0 || (!h->f32 && !h->form_walls))
-      CK(launch_between(h, parity ^ 1, true));
     if (s == nsteps - 1) CK(launch_finalize(h, parity ^ 1, nsteps, true));
+    else if (!self_chained(h)) CK(launch_between(h, parity ^ 1, true));
   }
   return CAVITY_OK;
 }
@@ -1910,7 +1919,6 @@ int cavity_time_kernels(cavity_t *h, int nsteps, double ms[4]) {
     cudaEventRecord(ev[0], h->stream);
     cudaError_t e = launch_step_kernel(h, par, 0);
     cudaEventRecord(ev[1], h->stream);
-    if (e == cudaSuccess && (h->n_cut > 0 || (!h->f32 && !h->form_walls))) e = launch_between(h, par ^ 1, false);
     if (e == cudaSuccess) e = launch_finalize(h, par ^ 1, 1, false);
     cudaEventRecord(ev[2], h->stream);
     cudaEventRecord(ev[3], h->stream);
