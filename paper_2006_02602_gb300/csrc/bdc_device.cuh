@@ -1,7 +1,7 @@
 // Device-side data structures and kernels of the buoyancy-driven-cavity step
 // (Xue & Roy, arXiv 2006.02602).  Shared by the C-ABI translation unit only.
 //
-// Per step, on the handle's stream (CUDA graphs of 1, 4 and 16 steps per
+// Per step, on the handle's stream (CUDA graphs of 1, 2, 4 and 16 steps per
 // buffer parity, each kernel a programmatic dependent of the one before):
 //   k_step      fused residual (Eqs. 1-3) + explicit Euler update of every
 //               interior node of every block, walls (Section 2) formed where

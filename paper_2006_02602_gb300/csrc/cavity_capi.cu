@@ -107,9 +107,10 @@ struct AdjointStore {
 constexpr int kAdjParts = 2 * 152;  // argmax partials of a state
 
 // Steps of one graph: a graph ends with one finalise launch for all of its
-// steps, so a long run is mostly 16-step graphs.
-constexpr int kGraphs = 3;
-constexpr int kGraphSteps[kGraphs] = {1, 4, kGraphMax};
+// steps, so a long run is mostly 16-step graphs (2 for calls of two or three steps:
+// FP64 32^3 in calls of two 17.4 us a step, 24.6 as two graphs of one).
+constexpr int kGraphs = 4;
+constexpr int kGraphSteps[kGraphs] = {1, 2, 4, kGraphMax};
 
 struct cavity {
   int dev = 0;

@@ -1,6 +1,6 @@
 """Steps chained in graphs against the same steps one call at a time.
 
-A call's steps run in graphs of 16, 4 and 1 steps; inside a graph dt comes from
+A call's steps run in graphs of 16, 4, 2 and 1 steps; inside a graph dt comes from
 an atomic maximum, the centre shift from the state, and one finalise at the end
 reduces every step's partials.  A call of one step finalises after it.  Fields,
 dt, time and the records of the step log must not depend on the split: the
@@ -42,7 +42,7 @@ def test_split_of_a_run_changes_nothing(m, prec, n, blocks, local):
     precision = m.CAVITY_FP64 if prec == "fp64" else m.CAVITY_FP32_MIXED
     kw = dict(blocks=blocks, precision=precision, seed=3, noise_amp=1e-3, Ra=3e4)
     q = workloads.smooth_state(n, seed=5)
-    steps = 39  # 16 + 16 + 4 + 1 + 1 + 1
+    steps = 39  # 16 + 16 + 4 + 2 + 1
     got = []
     for calls in ([steps], [1] * steps, [3, 17, 5, 14]):
         with m.Cavity(*n, **kw) as c:
