@@ -266,15 +266,16 @@ CAVITY_API int cavity_batch_get_fields(cavity_t *h, int cav, int field_mask, dou
  * steps on this handle's own cavities, times the four fastest once more
  * (each keeps its better time) and keeps the fastest.  The state is
  * saved before the trials and restored after them (the step counter and the
- * fields are as before the call).  out (optional) receives the chosen tile
+ * fields are as before the call).  Without it the chunk depth follows the
+ * cavity's size.  out (optional) receives the chosen tile
  * height (8 or 16 rows of 32 nodes), z-chunk, ring depth, kernel form (3:
  * two nodes per thread, the z neighbours below the plane in registers, the
  * one form) and microseconds per step.  Every shape gives the same fields.
  * With the environment variable BDC_F32_TILE
  * ("TY,KC,R,form", a compiled shape, read at creation) the shape is pinned and
- * no trials run (out[4] = 0).  FP64 handles have a single shape (32 x 4
- * threads, 8-plane chunks; BDC_F64_TY=8, read at creation, selects 32 x 8):
- * CAVITY_ERR_UNSUPPORTED. */
+ * no trials run (out[4] = 0).  FP64 handles have a single shape (tiles of 128
+ * nodes, their depth by the cavity's size; BDC_F64_TY=8, read at creation,
+ * selects 256 nodes): CAVITY_ERR_UNSUPPORTED. */
 CAVITY_API int cavity_autotune(cavity_t *h, int steps, double out[5]);
 
 /* Discrete adjoint, part 1: from the current state run nsteps steps and
@@ -330,14 +331,15 @@ CAVITY_API int cavity_set_time_stepping(cavity_t *h, int mode);
 
 /* Measurement: run nsteps steps as plain launches (no graph replay) with CUDA
  * events around every kernel on the handle's stream.  ms[0..3] receive the
- * mean duration per launch of the fused step kernel, the wall/finalise
- * kernel, the pack kernel and the unpack kernel (0 where a kernel does not
- * run).  The steps are real steps of the state. */
+ * mean duration per step of the fused step kernel, of what follows it
+ * (exchange or stored walls where the cavity has them, the finalise; one step a
+ * graph, so a finalise every step), and twice 0 (the exchange has no
+ * kernels of its own).  The steps are real steps of the state. */
 CAVITY_API int cavity_time_kernels(cavity_t *h, int nsteps, double ms[4]);
 
 /* Self-check of the FP64 square root the fused FP64 step uses for the wave
- * speeds lambda_d = (|V_d| + sqrt(V_d^2 + 4 beta^2)) / 2 (Section 2): a
- * Newton iteration seeded by the approximate reciprocal square root.  On the
+ * speeds lambda_d = (|V_d| + sqrt(V_d^2 + 4 beta^2)) / 2 (Section 2): FP32 and
+ * integer operations around the approximate reciprocal square root.  On the
  * current CUDA device, evaluates it and CUDA's correctly rounded sqrt for the
  * n host values x (positive, normal, finite; copied in and out by the call,
  * which synchronises) and returns the largest relative difference in
