@@ -1385,6 +1385,8 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, const __grid
     if (tid == 0) *cnt = 0u;
     // the slice totals loaded in parallel
     if (tid < nsl * 8) shm[tid] = mid[tid];
+  } else if (nwall) {
+    __syncthreads();  // warp 3 is done with rows 6 and 7 of sv (its part of the slice's tree)
   }
   if (tid < 8) shc[tid] = cp;
   if (nwall) {
