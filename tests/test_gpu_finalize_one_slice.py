@@ -28,7 +28,7 @@ def m():
 @pytest.mark.parametrize("n", [(16, 16, 16), (24, 24, 24), (20, 17, 13), (2, 3, 2)])
 def test_every_record_equals_that_of_single_steps(m, n):
     steps = 320
-    kw = dict(seed=3, noise_amp=1e-3, Ra=2e3)
+    kw = dict(seed=3, noise_amp=1e-3, Ra=5e2)  # (stable at two nodes an axis)
     logs = [m.StepLog(steps) for _ in range(2)]
     with m.Cavity(*n, **kw) as a, m.Cavity(*n, **kw) as b:
         m.cavity_set_step_log(a.h, logs[0])
