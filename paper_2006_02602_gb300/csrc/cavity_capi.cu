@@ -815,13 +815,17 @@ void launch_refresh(cavity *h, int parity) {
   }
 }
 
+// Whether a step leaves its state's walls stored: where the next one reads them, be it
+// the step kernel of a large FP64 cavity or the overlapped schedule's shell kernel.
+bool stores_walls(const cavity *h) { return !h->f32 && (!h->form_walls || h->overlap); }
+
 // The finalise of `nsteps` steps; the state in buffer set `parity` gets its
 // ghost layers and stored walls in the same launch.
 cudaError_t launch_finalize(cavity *h, int parity, int nsteps, bool pdl) {
   int ctas = 0;
   const BcArgs b = fin_args(h, parity, nsteps, &ctas);
   const FinTail t{ctas, h->n_cut, exch_args(h, parity), bc_args(h, parity, 3)};
-  ctas += h->n_cut + (h->f32 || h->form_walls ? 0 : h->n_bc);
+  ctas += h->n_cut + (stores_walls(h) ? h->n_bc : 0);
   if (h->f32) return launch_chained(h, pdl, k_finalize<float>, ctas, dim3(kFinThreads), 0, b, t);
   return launch_chained(h, pdl, k_finalize<double>, ctas, dim3(kFinThreads), 0, b, t);
 }
@@ -831,7 +835,7 @@ cudaError_t launch_finalize(cavity *h, int parity, int nsteps, bool pdl) {
 cudaError_t launch_between(cavity *h, int parity, bool pdl) {
   const ExchArgs x = exch_args(h, parity);
   const BcArgs b = bc_args(h, parity, 3);
-  const int grid = h->ncav + h->n_cut + (h->f32 || h->form_walls ? 0 : h->n_bc);
+  const int grid = h->ncav + h->n_cut + (stores_walls(h) ? h->n_bc : 0);
   if (h->f32) return launch_chained(h, pdl, k_between<float>, grid, dim3(kBetweenThreads), 0, x, b, h->n_cut);
   return launch_chained(h, pdl, k_between<double>, grid, dim3(kBetweenThreads), 0, x, b, h->n_cut);
 }
@@ -1174,7 +1178,7 @@ cudaError_t launch_recompute_between(cavity *h, int s) {
   x.blocks = b.blocks = A.seg_blocks + s;
   b.dt_out = A.dts + s;
   b.slot = self_chained(h) ? (s - 1) % kStepSlots : 0;
-  const int grid = 1 + (h->f32 || h->form_walls ? 0 : h->n_bc);
+  const int grid = 1 + (stores_walls(h) ? h->n_bc : 0);
   if (h->f32) return launch_chained(h, true, k_between<float>, grid, dim3(kBetweenThreads), 0, x, b, 0);
   return launch_chained(h, true, k_between<double>, grid, dim3(kBetweenThreads), 0, x, b, 0);
 }
