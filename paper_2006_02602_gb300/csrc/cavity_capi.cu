@@ -929,17 +929,27 @@ void drop_graphs(cavity *h) {
       if (g) { cudaGraphExecDestroy(g); g = nullptr; }
 }
 
+// While it lives, this thread may make calls that allocate although one of its
+// (or, in global mode, anyone's) streams is being captured.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // The graphs of kGraphSteps[q] steps, built when a call first needs them (every
 // setter that changes a launch drops them), captured on a stream of the
-// handle's own.
+// handle's own.  A caller may be capturing another stream meanwhile: instantiating
+// would be refused then, and would end that capture.
 int ensure_graph(cavity *h, int q) {
   if (h->graph[q][1]) return CAVITY_OK;
+  RelaxedCapture relaxed;
   if (h->overlap) CK(ensure_side(h));
   if (!h->capture) CK(cudaStreamCreateWithFlags(&h->capture, cudaStreamNonBlocking));
   for (int par = 0; par < 2; ++par) {
     if (h->graph[q][par]) continue;
     cudaGraph_t g = nullptr;
-    CK(cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal));
+    CK(cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeRelaxed));
     std::swap(h->stream, h->capture);
     const int rc = launch_steps(h, par, kGraphSteps[q]);
     std::swap(h->stream, h->capture);
