@@ -191,12 +191,15 @@ int fail(cavity *h, int code, const std::string &msg) {
   return code;
 }
 
+// (the error goes to the caller, not to the next call that asks for the last one)
 #define CK(call)                                                                   \
   do {                                                                             \
     cudaError_t e_ = (call);                                                       \
-    if (e_ != cudaSuccess)                                                         \
+    if (e_ != cudaSuccess) {                                                       \
+      cudaGetLastError();                                                          \
       return fail(h, e_ == cudaErrorMemoryAllocation ? CAVITY_ERR_OOM : CAVITY_ERR_CUDA, \
                   std::string(#call) + ": " + cudaGetErrorString(e_));             \
+    }                                                                              \
   } while (0)
 
 struct DeviceGuard {

@@ -42,3 +42,29 @@ def test_steps_while_another_stream_is_captured(m, prec):
         ref.step(63)
         assert np.array_equal(c.fields(), ref.fields())
         assert c.time == ref.time
+
+
+@pytest.mark.filterwarnings("ignore:The CUDA Graph is empty")
+def test_a_capture_of_the_handles_own_stream_is_refused_and_leaves_nothing_behind(m):
+    import torch
+    s = torch.cuda.Stream()
+    with m.Cavity(20, 17, 15, seed=1, noise_amp=1e-3, stream=s.cuda_stream) as c:
+        c.sync()
+        g = torch.cuda.CUDAGraph()
+        refused = False
+        try:
+            with torch.cuda.graph(g, stream=s):
+                try:
+                    c.step(3)
+                except m.CavityError:
+                    refused = True
+        except RuntimeError:  # the refused launch may have ended the capture
+            pass
+        assert refused
+        torch.cuda.synchronize()
+        # the refusal is not the next call's error
+        with m.Cavity(20, 17, 15, seed=1, noise_amp=1e-3) as a, m.Cavity(20, 17, 15, seed=1, noise_amp=1e-3) as b:
+            a.step(5)
+            for _ in range(5):
+                b.step(1)
+            assert np.array_equal(a.fields(), b.fields())
