@@ -990,6 +990,18 @@ int run_piece(cavity *h, int q, int par) {
   return CAVITY_OK;
 }
 
+// The graphs a call of nsteps steps from the present buffer set replays, before it is timed.
+int build_graphs(cavity *h, int nsteps) {
+  int par = h->parity;
+  for (int q = kGraphs - 1; q >= 0; --q)
+    for (; nsteps >= kGraphSteps[q]; nsteps -= kGraphSteps[q]) {
+      const int rc = ensure_graph(h, q, par);
+      if (rc != CAVITY_OK) return rc;
+      par ^= kGraphSteps[q] & 1;
+    }
+  return CAVITY_OK;
+}
+
 int run_steps(cavity *h, int nsteps) {
   for (int q = kGraphs - 1; q >= 0; --q)
     for (; nsteps >= kGraphSteps[q]; nsteps -= kGraphSteps[q]) {
@@ -1680,9 +1692,11 @@ int cavity_autotune(cavity_t *h, int steps, double out[5]) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (rc == CAVITY_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess))
     rc = fail(h, CAVITY_ERR_CUDA, "event creation failed");
-  // one trial of a shape: `steps` graph-replayed steps after a warm-up, from the saved state
+  // one trial of a shape: `steps` graph-replayed steps after a warm-up, from the saved
+  // state (their graphs built before: that takes longer than a small cavity's steps)
   auto trial = [&](const F32Shape &s, double &us) -> int {
     int r = retile(h, s.p, s.ty, s.kc, s.r);
+    if (r == CAVITY_OK) r = build_graphs(h, steps);
     if (r == CAVITY_OK) r = cavity_step(h, 2);  // warm-up
     if (r != CAVITY_OK) return r;
     cudaEventRecord(e0, h->stream);
