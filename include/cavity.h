@@ -264,10 +264,13 @@ CAVITY_API int cavity_batch_get_fields(cavity_t *h, int cav, int field_mask, dou
 /* Autotuner of the FP32-mixed step kernel: times every compiled tile shape
  * (x-y tile extent, z-chunk length, ring depth) for `steps` graph-replayed
  * steps on this handle's own cavities, times the four fastest once more
- * (each keeps its better time) and keeps the fastest.  The state is
+ * (each keeps its better time) and keeps the fastest.  The shapes' z-chunks are
+ * 16 planes and more; the shape held on entry is timed as well and stays where
+ * none of them is faster (without this call the chunk depth follows the
+ * cavity's size, down to one plane).  The state is
  * saved before the trials and restored after them (the step counter and the
- * fields are as before the call).  Without it the chunk depth follows the
- * cavity's size.  out (optional) receives the chosen tile
+ * fields are as before the call).  out (optional) receives the fastest compiled
+ * shape, also where the held one stays: its tile
  * height (8 or 16 rows of 32 nodes), z-chunk, ring depth, kernel form (3:
  * two nodes per thread, the z neighbours below the plane in registers, the
  * one form) and microseconds per step.  Every shape gives the same fields.

@@ -1,8 +1,11 @@
-"""What the autotuner times.
+"""What the autotuner times and what it leaves behind.
 
 The time it reports, and ranks the shapes by, is that of steps, not of building
-their graphs.
+their graphs.  The depths it tries start at 16 planes, below which the depth that
+follows the size goes; so the shape held on entry is timed as well, and a handle is
+not slower after the call than before it.
 """
+import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -46,3 +49,20 @@ def test_reported_time_is_that_of_the_steps(m, monkeypatch):
         us = _us_per_step(torch, s, c, steps, 12)
     # (23 us a step; what of building the two graphs the warm-up does not cover, 3.5 us a step)
     assert 0.9 * us <= t["us_per_step"] <= 1.09 * us, (t, us)
+
+
+@pytest.mark.parametrize("n", [(32, 32, 32), (61, 47, 83), (20, 16, 12)])
+def test_not_slower_after_than_before(m, n):
+    import torch
+    s = torch.cuda.Stream()
+    kw = dict(precision=m.CAVITY_FP32_MIXED, seed=4, noise_amp=1e-3, Ra=1e4)
+    with m.Cavity(*n, stream=s.cuda_stream, **kw) as c, m.Cavity(*n, **kw) as ref:
+        c.step(40)
+        before = _us_per_step(torch, s, c, 80, 8)
+        m.cavity_autotune(c.h, 10)
+        c.step(40)
+        after = _us_per_step(torch, s, c, 80, 8)
+        assert after <= 1.2 * before  # (16 planes against 1 to 8: 1.5 to 2.8 times)
+        ref.step(2 * 40 + 2 * 8 * 80)
+        assert np.array_equal(c.fields(), ref.fields())
+        assert c.time == ref.time
