@@ -151,14 +151,15 @@ typedef struct {
 
 /* Step log in host memory: after each step the device writes that step's
  * record of cavity c (0 for a single cavity) to host[((step - 1) % capacity)
- * * ncav + c], in the launch that finishes the step, so a caller that wants
+ * * ncav + c], in the steps' order and beside the steps that follow (two steps
+ * later at most; the last steps' of a call at its end), so a caller that wants
  * every step's diagnostics reads them from host memory when it next
  * synchronises, without a synchronising getter per step.  host must be
  * page-locked host memory (cudaHostAlloc, cudaHostRegister, a pinned torch
  * tensor) of capacity * ncav records, kept alive while attached; NULL
- * detaches.  Records of steps the adjoint's reverse sweep recomputes are
- * written again.  CAVITY_ERR_INVALID_ARG for capacity < 1 or memory the device
- * cannot address. */
+ * detaches.  Steps that the adjoint's reverse sweep recomputes have been logged
+ * and are not logged again.  CAVITY_ERR_INVALID_ARG for capacity < 1 or memory
+ * the device cannot address. */
 CAVITY_API int cavity_set_step_log(cavity_t *h, cavity_step_record *host, long long capacity);
 
 /* Page-locked, zeroed host memory for `records` step records (records >= 1),

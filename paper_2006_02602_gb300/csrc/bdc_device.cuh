@@ -178,6 +178,9 @@ struct CavState {
   unsigned int sfl[kStepSlots], pad2;
   double dt0;        // dt as the last finalise left it (dt itself moves on within a graph)
   double nu_sum;     // sum of nu_hot over the steps (the adjoint's forward run zeroes it)
+  // the step log's running values between two finalises (k_step_record's own)
+  double log_t, log_dt;
+  long long log_bad;
 };
 
 struct StepRecord {   // one step's record in the host-memory step log (the C ABI's cavity_step_record)
@@ -1293,6 +1296,78 @@ __device__ __forceinline__ int nu_cta(const BcArgs &a, int cta, double *sh) {
   return F.cav;
 }
 
+// The totals of a step, field f's in thread 16 f: the slices' totals (shm, [slice][field])
+// combined by the field's 16 threads (slice s in thread 16 f + s, a butterfly over the
+// first nsl), then in fields 6 and 7 the tree of the wall CTAs' Nusselt partials w0 ..
+// w1 - 1, thread-strided (rows 6 and 7 of sv, which nobody may be reading any more).
+template <int NT>
+__device__ __forceinline__ double step_totals(const double *bc_partials, int w0, int w1, int nsl, const double *shm,
+                                              double *sv, int tid) {
+  const int f = tid >> 4, s = tid & 15;
+  if (w1 > w0) {
+    double h = 0.0, c = 0.0;
+    for (int q = w0 + tid; q < w1; q += NT) {
+      h += bc_partials[2LL * q];
+      c += bc_partials[2LL * q + 1];
+    }
+    sv[6 * NT + tid] = h;
+    sv[7 * NT + tid] = c;
+  }
+  __syncthreads();
+  double t = s < nsl ? shm[s * 8 + f] : 0.0;
+  for (int o = 1; o < nsl; o <<= 1) t = fin_comb(f, t, __shfl_xor_sync(0xffffffffu, t, o));
+  if (w1 > w0 && f >= 6) t += fin_tree<NT>(sv, f, s);
+  return t;
+}
+
+// The step log's record of step s of a sequence of steps that one finalise ends, one CTA a
+// cavity, on a stream beside the steps': it waits for step s + 1 (whose launch leaves
+// the x walls' Nusselt partials of step s) and runs beside step s + 2, by the finalise's
+// sums in the finalise's order.  The finalise writes the last two records.  So every
+// record is in host memory two steps later at most; with the finalise's alone they came
+// once a sequence, up to 16 steps late, those that a shorter ring has no room for never.
+// A logged step takes 1-3% more than an unlogged one (FP64 32^3 11.7 us, 11.4; 64^3 46.4, 44.9;
+// 128^3 in 2x2x2 blocks 268, 264; FP32-mixed 256^3 211.1, 210.8): the finalise has to
+// wait for the records and is no programmatic dependent of the last step then.
+static __global__ void __launch_bounds__(kFinThreads) k_step_record(BcArgs a, int s) {
+  constexpr int NT = kFinThreads;
+  __shared__ double sv[8 * NT];
+  __shared__ double shm[kFinSlices * 8];
+  __shared__ double val[8];
+  const int cav = blockIdx.x, tid = threadIdx.x, f = tid >> 4;
+  const CavConst &C = a.cc[cav];
+  for (int g = 0; g < a.nslices; ++g) {
+    double acc[8];
+    load_slice<NT>(a, a.step_partials, C.slice_q[g], C.slice_q[g + 1], 0, 0, 0, 0, tid, acc);
+    const double t = tree_slice<NT>(acc, sv, tid);
+    if ((tid & 15) == 0) shm[g * 8 + f] = t;
+    __syncthreads();  // (before the next slice, or the wall partials, overwrite sv)
+  }
+  double t = step_totals<NT>(a.bc_partials, a.wall_ctas ? C.nu_begin : 0, a.wall_ctas ? C.nu_end : 0, a.nslices, shm, sv,
+                             tid);
+  const bool bad = (tid & 15) == 0 && f < 6 && !isfinite(t);
+  if ((tid & 15) == 0) {
+    if (f >= 6 && a.mode == 4) t *= C.wscale[f - 6];
+    val[f] = f < 5 ? sqrt(t * C.inv_nint) : f == 5 ? C.cfl / t : t * C.inv_nwall;
+  }
+  const int any = __syncthreads_or(bad);
+  if (tid != 0) return;
+  CavState &st = a.cs[cav];
+  const double tt = s == 0 ? st.t + st.dt0 : st.log_t + st.log_dt;
+  const long long step = st.step + s + 1, nonfin = (s == 0 ? 0 : st.log_bad) | (any ? 1 : 0);
+  st.log_t = tt;
+  st.log_dt = val[5];
+  st.log_bad = nonfin;
+  StepRecord &o = a.log[((step - 1) % a.log_cap) * a.ncav + cav];
+  o.step = step;
+  o.t = tt;
+  o.dt = val[5];
+  for (int q = 0; q < 5; ++q) o.res[q] = val[q];
+  o.nu_hot = val[6];
+  o.nu_cold = val[7];
+  o.flags = *(volatile int *)&st.flags | nonfin;
+}
+
 // What a graph's last step leaves beside its sums, in CTAs from `begin` on of the
 // same launch: the exchange of the new state's cut faces, then its stored walls.
 // (They write ghosts and walls, the finalise reads partials and interior nodes.)
@@ -1389,25 +1464,10 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, const __grid
     __syncthreads();  // warp 3 is done with rows 6 and 7 of sv (its part of the slice's tree)
   }
   if (tid < 8) shc[tid] = cp;
-  if (nwall) {
-    // the wall CTAs' Nusselt partials, thread-strided, into fields 6 and 7 of
-    // the tree (the graph's earlier steps' were left by the next step's launch)
-    double h = 0.0, c = 0.0;
-    const double *bp = a.bc_partials + m * a.bc_stride;
-    const int q0 = a.nu_only ? C.nu_begin : C.bc_begin, q1 = a.nu_only ? C.nu_end : C.bc_xend;
-    for (int q = q0 + tid; q < q1; q += NT) {  // the other walls' partials are zeros
-      h += bp[2LL * q];
-      c += bp[2LL * q + 1];
-    }
-    sv[6 * NT + tid] = h;
-    sv[7 * NT + tid] = c;
-  }
-  __syncthreads();
-  // the slice totals of field f combined by its 16 threads (slice s in thread
-  // 16 f + s, a butterfly over the first nsl), then the wall partials' tree
-  double t = s < nsl ? shm[s * 8 + f] : 0.0;
-  for (int o = 1; o < nsl; o <<= 1) t = fin_comb(f, t, __shfl_xor_sync(0xffffffffu, t, o));
-  if (nwall && f >= 6) t += fin_tree<NT>(sv, f, s);
+  // (the graph's earlier steps' wall partials were left by the next step's launch)
+  const int w0 = !nwall ? 0 : a.nu_only ? C.nu_begin : C.bc_begin;
+  const int w1 = !nwall ? 0 : a.nu_only ? C.nu_end : C.bc_xend;  // (the other walls' are zeros)
+  double t = step_totals<NT>(a.bc_partials + m * a.bc_stride, w0, w1, nsl, shm, sv, tid);
   // one thread of each field group finishes its field (the FP64 chains run
   // side by side): residual norms, dt, Nusselt numbers; thread 1 the centre
   StepResult &out = a.rec[(long long)m * a.ncav + cav];
@@ -1487,7 +1547,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, const __grid
       st.nu_hot = nh;
       st.nu_cold = nc;
     }
-    if (a.log && M - tid <= a.log_cap) {  // each step's record, written to host memory
+    if (a.log && M - tid <= min(a.log_cap, 2ll)) {  // the last records, written to host memory (k_step_record's before)
       const long long step = step0 + tid + 1;
       StepRecord &o = a.log[((step - 1) % a.log_cap) * a.ncav + cav];
       o.step = step;

@@ -902,9 +902,25 @@ int launch_step_overlapped(cavity *h, int parity) {
   return CAVITY_OK;
 }
 
+// The step log's record of step `s` of a sequence, on the side stream, after the step launched last.
+int launch_record(cavity *h, int parity, int s) {
+  int ctas = 0;
+  BcArgs b = fin_args(h, parity, 1, &ctas);
+  b.step_partials = step_partials(h, s);
+  b.bc_partials += s * b.bc_stride;
+  CK(cudaEventRecord(h->ev_shell, h->stream));
+  CK(cudaStreamWaitEvent(h->side, h->ev_shell, 0));
+  k_step_record<<<h->ncav, kFinThreads, 0, h->side>>>(b, s);
+  CK(cudaGetLastError());
+  return CAVITY_OK;
+}
+
 // nsteps explicit steps from buffer set `parity` (launched, or captured into a
 // graph): the steps one after another, then one finalise launch for all of them.
+// With a step log the records of all but the last two (the finalise's) are written
+// beside the steps.
 int launch_steps(cavity *h, int parity, int nsteps) {
+  const bool records = h->d_log && nsteps > 2;
   for (int s = 0; s < nsteps; ++s, parity ^= 1) {
     if (h->overlap) {
       const int rc = launch_step_overlapped(h, parity);
@@ -912,8 +928,19 @@ int launch_steps(cavity *h, int parity, int nsteps) {
       continue;
     }
     CK(launch_step_kernel(h, parity, s));
-    if (s == nsteps - 1) CK(launch_finalize(h, parity ^ 1, nsteps, true));
-    else if (!self_chained(h)) CK(launch_between(h, parity ^ 1, true));
+    if (records && s >= 1 && s <= nsteps - 2) {
+      const int rc = launch_record(h, parity, s - 1);
+      if (rc != CAVITY_OK) return rc;
+    }
+    if (s == nsteps - 1) {
+      if (records) {  // the finalise moves on the time, which the records start from
+        CK(cudaEventRecord(h->ev_exch, h->side));
+        CK(cudaStreamWaitEvent(h->stream, h->ev_exch, 0));
+      }
+      CK(launch_finalize(h, parity ^ 1, nsteps, !records));
+    } else if (!self_chained(h)) {
+      CK(launch_between(h, parity ^ 1, true));
+    }
   }
   return CAVITY_OK;
 }
@@ -1475,6 +1502,7 @@ int cavity_set_step_log(cavity_t *h, cavity_step_record *host, long long capacit
     dev = (StepRecord *)pa.devicePointer;
   }
   CK(cudaStreamSynchronize(h->stream));
+  if (host) CK(ensure_side(h));  // the records' stream
   h->d_log = dev;
   h->log_cap = host ? capacity : 0;
   drop_graphs(h);  // the finalise launches in the graphs carry the log
