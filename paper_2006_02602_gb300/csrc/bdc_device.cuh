@@ -74,10 +74,10 @@ struct CavConst {
   // FP32 copies (rounded to nearest, as a device conversion would) of the
   // constants the FP32 kernels and estimates use, so that no kernel spends
   // FP64-pipe conversions on them: 1/h, 1/(2h), nu/h^2, alpha/h^2, c4/2, gs,
-  // T_inf, beta_min^2, the diffusive spectral term, cfl; 1/h^2, c4, nu, alpha
+  // T_inf, beta_min^2, the diffusive spectral term, cfl, c4
   float fih[3], fh2[3], fnh[3], fah[3];
   float fc4h, fgs, ftinf, fb2min, fdiffsr, fcfl;
-  float fihh[3], fc4, fnu, falpha;
+  float fc4;
   // the spectral bound at rest, S0 = beta_min (1/h_x + 1/h_y + 1/h_z) + the
   // diffusive term (FP64), and 2 beta_min (FP32): the FP64 step's dt filter
   // works on S - S0
@@ -137,11 +137,8 @@ inline void set_cav_physics(CavConst &C, const int gn[3], const cavity_params &p
     C.fh2[d] = (float)C.ih2[d];
     C.fnh[d] = (float)(C.nu * C.ihh[d]);
     C.fah[d] = (float)(C.alpha * C.ihh[d]);
-    C.fihh[d] = (float)C.ihh[d];
   }
   C.fc4 = (float)C.c4;
-  C.fnu = (float)C.nu;
-  C.falpha = (float)C.alpha;
   {
     const double b0 = std::sqrt(C.b2min);
     C.s0 = b0 * (C.ih[0] + C.ih[1] + C.ih[2]) + C.diffsr;
