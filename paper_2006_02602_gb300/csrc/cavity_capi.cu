@@ -1913,15 +1913,17 @@ int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *gr
     ba.blocks = A.seg_blocks;
     ba.faces = A.seg_faces;
     ba.nfaces = (int)h->hwall.size() * len;
-    const dim3 parts(kAdjParts, len);
-    if (h->f32) {
-      k_bc<float><<<h->n_bc * len, kBcThreads, 0, h->stream>>>(ba);
-      k_adj_argmax_seg<float><<<parts, 256, 0, h->stream>>>(A.seg_blocks, h->hcc[0], A.argpart);
-    } else {
-      k_bc<double><<<h->n_bc * len, kBcThreads, 0, h->stream>>>(ba);
-      k_adj_argmax_seg<double><<<parts, 256, 0, h->stream>>>(A.seg_blocks, h->hcc[0], A.argpart);
-    }
+    if (h->f32) k_bc<float><<<h->n_bc * len, kBcThreads, 0, h->stream>>>(ba);
+    else k_bc<double><<<h->n_bc * len, kBcThreads, 0, h->stream>>>(ba);
     CK(cudaGetLastError());
+    constexpr int kGridY = 65535;  // a longer segment's states take more than one launch
+    for (int s = 0; s < len; s += kGridY) {
+      const dim3 parts(kAdjParts, std::min(kGridY, len - s));
+      double *out = A.argpart + 2 * (size_t)kAdjParts * s;
+      if (h->f32) k_adj_argmax_seg<float><<<parts, 256, 0, h->stream>>>(A.seg_blocks + s, h->hcc[0], out);
+      else k_adj_argmax_seg<double><<<parts, 256, 0, h->stream>>>(A.seg_blocks + s, h->hcc[0], out);
+      CK(cudaGetLastError());
+    }
     // reverse sweep over the segment
     CK(cudaEventRecord(h->adj_ev[2 * c], h->stream));
     for (int s = len - 1; s >= 0; --s) {
