@@ -1896,53 +1896,57 @@ int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *gr
     h->adj_ev.push_back(e);
   }
   auto slot = [&](int s) { return (void *)(A.seg_mem + (size_t)s * A.set_bytes); };
-  for (int c = nseg - 1; c >= 0; --c) {
-    const int s0 = c * ck, len = std::min(ck, A.nsteps - s0);
-    // recompute the segment from its checkpoint (copied to slot 0), each step
-    // reading slot s and writing slot s + 1
-    CK(cudaMemcpyAsync(slot(0), A.ckpt_mem + (size_t)c * A.set_bytes, A.set_bytes, cudaMemcpyDeviceToDevice,
-                       h->stream));
-    CK(cudaMemcpyAsync(h->d_cs, A.ckpt_cs + c, sizeof(CavState), cudaMemcpyDeviceToDevice, h->stream));
-    CK(cudaMemcpyAsync(A.dts, &h->d_cs->dt, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
-    for (int s = 0; s + 1 < len; ++s) {
-      CK(launch_recompute(h, s, s > 0));
-      if (!self_chained(h) || s + 2 == len) CK(launch_recompute_between(h, s + 1));
-    }
-    // the walls (formed by the step where it reads them) of every stored state
-    BcArgs ba = bc_args(h, 0, 3);
-    ba.blocks = A.seg_blocks;
-    ba.faces = A.seg_faces;
-    ba.nfaces = (int)h->hwall.size() * len;
-    if (h->f32) k_bc<float><<<h->n_bc * len, kBcThreads, 0, h->stream>>>(ba);
-    else k_bc<double><<<h->n_bc * len, kBcThreads, 0, h->stream>>>(ba);
-    CK(cudaGetLastError());
-    constexpr int kGridY = 65535;  // a longer segment's states take more than one launch
-    for (int s = 0; s < len; s += kGridY) {
-      const dim3 parts(kAdjParts, std::min(kGridY, len - s));
-      double *out = A.argpart + 2 * (size_t)kAdjParts * s;
-      if (h->f32) k_adj_argmax_seg<float><<<parts, 256, 0, h->stream>>>(A.seg_blocks + s, h->hcc[0], out);
-      else k_adj_argmax_seg<double><<<parts, 256, 0, h->stream>>>(A.seg_blocks + s, h->hcc[0], out);
+  auto sweep = [&]() -> int {
+    for (int c = nseg - 1; c >= 0; --c) {
+      const int s0 = c * ck, len = std::min(ck, A.nsteps - s0);
+      // recompute the segment from its checkpoint (copied to slot 0), each step
+      // reading slot s and writing slot s + 1
+      CK(cudaMemcpyAsync(slot(0), A.ckpt_mem + (size_t)c * A.set_bytes, A.set_bytes, cudaMemcpyDeviceToDevice,
+                         h->stream));
+      CK(cudaMemcpyAsync(h->d_cs, A.ckpt_cs + c, sizeof(CavState), cudaMemcpyDeviceToDevice, h->stream));
+      CK(cudaMemcpyAsync(A.dts, &h->d_cs->dt, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
+      for (int s = 0; s + 1 < len; ++s) {
+        CK(launch_recompute(h, s, s > 0));
+        if (!self_chained(h) || s + 2 == len) CK(launch_recompute_between(h, s + 1));
+      }
+      // the walls (formed by the step where it reads them) of every stored state
+      BcArgs ba = bc_args(h, 0, 3);
+      ba.blocks = A.seg_blocks;
+      ba.faces = A.seg_faces;
+      ba.nfaces = (int)h->hwall.size() * len;
+      if (h->f32) k_bc<float><<<h->n_bc * len, kBcThreads, 0, h->stream>>>(ba);
+      else k_bc<double><<<h->n_bc * len, kBcThreads, 0, h->stream>>>(ba);
       CK(cudaGetLastError());
+      constexpr int kGridY = 65535;  // a longer segment's states take more than one launch
+      for (int s = 0; s < len; s += kGridY) {
+        const dim3 parts(kAdjParts, std::min(kGridY, len - s));
+        double *out = A.argpart + 2 * (size_t)kAdjParts * s;
+        if (h->f32) k_adj_argmax_seg<float><<<parts, 256, 0, h->stream>>>(A.seg_blocks + s, h->hcc[0], out);
+        else k_adj_argmax_seg<double><<<parts, 256, 0, h->stream>>>(A.seg_blocks + s, h->hcc[0], out);
+        CK(cudaGetLastError());
+      }
+      // reverse sweep over the segment
+      CK(cudaEventRecord(h->adj_ev[2 * c], h->stream));
+      for (int s = len - 1; s >= 0; --s) {
+        a.B.base[0] = slot(s);
+        a.dt = A.dts + s;
+        a.argpart = A.argpart + 2 * (size_t)kAdjParts * s;
+        a.objective = s0 + s > 0;
+        a.X = X;
+        a.Q = Q;
+        const bool pdl = s < len - 1;
+        if (h->f32)
+          CK(launch_chained(h, pdl, k_adj_sweep<float, kAdjTY>, A.ctas, dim3(32 * kAdjTY), adj_smem_bytes<float, kAdjTY>(), a));
+        else
+          CK(launch_chained(h, pdl, k_adj_sweep<double, kAdjTY>, A.ctas, dim3(32 * kAdjTY), adj_smem_bytes<double, kAdjTY>(), a));
+        std::swap(X, Q);
+      }
+      CK(cudaEventRecord(h->adj_ev[2 * c + 1], h->stream));
     }
-    // reverse sweep over the segment
-    CK(cudaEventRecord(h->adj_ev[2 * c], h->stream));
-    for (int s = len - 1; s >= 0; --s) {
-      a.B.base[0] = slot(s);
-      a.dt = A.dts + s;
-      a.argpart = A.argpart + 2 * (size_t)kAdjParts * s;
-      a.objective = s0 + s > 0;
-      a.X = X;
-      a.Q = Q;
-      const bool pdl = s < len - 1;
-      if (h->f32)
-        CK(launch_chained(h, pdl, k_adj_sweep<float, kAdjTY>, A.ctas, dim3(32 * kAdjTY), adj_smem_bytes<float, kAdjTY>(), a));
-      else
-        CK(launch_chained(h, pdl, k_adj_sweep<double, kAdjTY>, A.ctas, dim3(32 * kAdjTY), adj_smem_bytes<double, kAdjTY>(), a));
-      std::swap(X, Q);
-    }
-    CK(cudaEventRecord(h->adj_ev[2 * c + 1], h->stream));
-  }
-  // the state after the forward run
+    return CAVITY_OK;
+  };
+  rc = sweep();
+  // the state after the forward run, also where the sweep failed on the way
   CK(cudaMemcpyAsync(h->hb[0].base[A.final_parity], A.final_mem, A.set_bytes, cudaMemcpyDeviceToDevice, h->stream));
   CK(cudaMemcpyAsync(h->d_cs, &A.final_cs, sizeof(CavState), cudaMemcpyHostToDevice, h->stream));
   h->parity = A.final_parity;
@@ -1952,6 +1956,7 @@ int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *gr
   if (grad_wall)
     CK(cudaMemcpyAsync(grad_wall, A.thetabar, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
+  if (rc != CAVITY_OK) return rc;
   if (grad_ra) *grad_ra = ra;
   double tot = 0.0;
   for (int c = 0; c < nseg; ++c) {
