@@ -44,6 +44,12 @@ UNIT = "point-updates/s"
 # T 13, buoyancy 2), update 11, residual sums 10, spectral radius of the new
 # state 25
 FP64_FLOP_PER_POINT = 190
+# FP64-pipe instructions the step kernel executes per interior point (ncu,
+# sm__inst_executed_pipe_fp64 of one launch at 128^3 in 2x2x2 blocks, times 32 lanes
+# over the points): 41 in the rates, 11 in the update and the residual sums, the rest
+# candidates for the next dt and the reduction.  What the formulation above holds
+# beside them runs as 64-bit integer sums
+FP64_INST_PER_POINT = 58
 # algorithmic HBM bytes per interior point-update of one fused pass: every
 # stored array read once and written once (FP64: 5 x 8 B; FP32-mixed: 7 x 4 B,
 # u, v, w and the hi/lo pairs of p and T)
@@ -59,11 +65,11 @@ ADJ_BYTES_PER_POINT = 68
 # (precision, workload, blocks, shape); the FP32 shape is the autotuner's
 # "TY,KC,R,form"
 FP64_SHAPE = "128x8"  # tiles of 128 nodes x 8 planes (then x 2)
-TRAFFIC = {("fp64", "cfg2", (2, 2, 2), FP64_SHAPE): 114.949632e6 + 56.212736e6,
-           ("fp32", "cfg3", (1, 1, 1), "8,96,4,3"): 613.445632e6 + 434.552064e6,
-           ("fp32", "cfg3", (1, 1, 1), "8,64,4,3"): 575.716096e6 + 435.488256e6,
-           ("fp32", "cfg3", (1, 1, 1), "8,32,4,3"): 585.227776e6 + 434.474240e6,
-           ("fp32", "cfg4", None, "8,64,4,3"): 612.079360e6 + 324.579072e6}
+TRAFFIC = {("fp64", "cfg2", (2, 2, 2), FP64_SHAPE): 115.047680e6 + 57.321728e6,
+           ("fp32", "cfg3", (1, 1, 1), "8,96,4,3"): 609.722880e6 + 435.107328e6,
+           ("fp32", "cfg3", (1, 1, 1), "8,64,4,3"): 573.457408e6 + 435.460352e6,
+           ("fp32", "cfg3", (1, 1, 1), "8,32,4,3"): 584.207360e6 + 434.930432e6,
+           ("fp32", "cfg4", None, "8,64,4,3"): 610.918400e6 + 325.046528e6}
 F32_FORMS = {3: "k_step_f32q (two nodes per thread, f32x2; z neighbours below the plane in registers)"}
 # FP64 peak derived from the unit counts: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
@@ -293,8 +299,12 @@ def roofline_for(precision, pts, step_ms, hbm, traffic=None, form=3, fp64_measur
                     ": TMA-staged fused residual + update + partials", traffic=traffic, kernel_ms=step_ms, **hbm_obj)
     tf = FP64_FLOP_PER_POINT * pts / step_s / 1e12
     peak = fp64_measured or FP64_PEAK_TFLOPS
+    inst = FP64_INST_PER_POINT * pts / step_s / 1e12
     return {"kernel": "k_step_f64 (fused residual + update + reductions)", "bound": "alu", "achieved": tf,
             "peak": peak, "unit": "TFLOP/s", "frac": tf / peak, "traffic": traffic,
+            # the roofline proper: an FMA, the peak's instruction, is two flops
+            "fp64_pipe": {"achieved": inst, "peak": peak / 2, "unit": "T FP64 instructions/s", "frac": 2 * inst / peak,
+                          "instructions_per_point": FP64_INST_PER_POINT},
             "peak_source": ("measured FP64 FMA throughput (cavity_measure_fp64_peak: independent DFMA chains on "
                             "every SM, of measured)" if fp64_measured else
                             "derived FP64 peak: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz"),
@@ -303,7 +313,8 @@ def roofline_for(precision, pts, step_ms, hbm, traffic=None, form=3, fp64_measur
             "flop_per_point_note": "counted on the formulation in floating point; the oracle's plain formulation of "
                                    "Eqs. 1-3 counts about 212.  The kernel does about half of them (dissipation, "
                                    "neighbour weights, T's transport, square roots) as 64-bit integer sums beside "
-                                   "the FP64 pipe, so frac can exceed 1", "hbm_view": hbm_obj}
+                                   "the FP64 pipe, so frac, a rate of the formulation, can exceed 1; fp64_pipe has "
+                                   "the fraction of what the kernel executes", "hbm_view": hbm_obj}
 
 
 def measure(m, torch, precision, workload, blocks, steps, warmup, rank, world, local, stream, e2e=True,
@@ -379,8 +390,8 @@ def measure(m, torch, precision, workload, blocks, steps, warmup, rank, world, l
     if e2e:
         # end to end through the public API with host buffers: initial state
         # from host; every step's residual + Nusselt record written by the
-        # device into page-locked host memory (the step log) as the step
-        # finishes, read on the host after the final synchronisation; final
+        # device into page-locked host memory (the step log) beside the steps
+        # after it, read on the host after the final synchronisation; final
         # fields back to host
         # the initial state and the final fields in page-locked host memory
         host0 = torch.empty(tuple(c.fields().shape), dtype=torch.float64, pin_memory=True).numpy()
@@ -512,6 +523,7 @@ def summary(line) -> dict:
     out = {}
     for name, v in [("headline", line)] + list(line.get("variants", {}).items()):
         r = v.get("roofline") or {}
+        r = dict(r, **r.get("fp64_pipe", {}))  # (FP64: what the pipe executes, not the formulation's flops)
         out[name] = {"value": v.get("value"), "ms_per_step": v.get("ms_per_step", v.get("backward_ms_per_step")),
                      "bound": r.get("bound"), "frac": r.get("frac"), "kernel_ms": r.get("kernel_ms")}
     return out
