@@ -1156,8 +1156,11 @@ int get_fields_cav(cavity *h, int cav, int mask, double *host, size_t count) {
 // The reverse sweep's chunk depth and CTAs: 32 x kAdjTY columns; the depth that
 // makes (waves + 0.25) x (depth + 2.5) least, waves the mean of the exact and the
 // rounded-up number, at least 1.5 in all: a chunk sweeps four planes of z terms
-// beside its own (2.5 planes' work), and the last CTAs run half alone.  128^3 FP32, us a launch: 161 at 4 planes, 146 at 8, 144 at 11,
-// 145 at 16, 154 at 19, 160 at 32 (one wave of 256 CTAs on 304 places).
+// beside its own (2.5 planes' work), and the last CTAs run half alone.  What it picks
+// against a sweep over the depths, us a reverse step: 128^3 FP32 110.0 at 15 planes (110.5 at 10,
+// 108.5 at 14, 117.7 at 8, 123 at 19, 126 at 32), 64^3 FP32 32.8 at 2 (28.3 at 4), 97x65x50 FP32 42.2 at
+// 4 (37.8 at 7), FP64 390 (359 at 3); FP64 32^3 46.0 at 1 (71.7 at 2), 48^3 124.8 at 4 (136 at 2):
+// the best but for up to 16% at sizes whose last wave is nearly empty.
 int adj_tiling(cavity *h, int *kc, int *ctas) {
   const cavity_desc &d = h->descs[0];
   int per_sm = 1;
