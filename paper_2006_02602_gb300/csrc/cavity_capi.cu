@@ -157,7 +157,8 @@ struct cavity {
   int nslices = kFinSlices;  // k_finalize CTAs per cavity: about 128 step partials a slice
   int form_walls = 1;  // FP64: walls formed where the step reads them (0: stored between the steps)
   int n_coarse = 0;  // FP64 step tiles of KC planes (scheduled before the fine ones)
-  int part_cap = 0;  // step partials allocated (CTAs)
+  int part_cap = 0;  // step partials allocated (CTAs) a set
+  int part_sets = kGraphMax;  // sets: steps of the longest graph (16, 4 or 1)
 
   BlockDev *d_blocks = nullptr;
   CavConst *d_cc = nullptr;
@@ -562,8 +563,15 @@ int ensure_partials(cavity *h) {
   CK(cudaStreamSynchronize(h->stream));
   if (h->d_step_part) cudaFree(h->d_step_part);
   h->d_step_part = nullptr;
-  // one set per step of a graph: all are reduced at its end
-  CK(cudaMalloc(&h->d_step_part, kGraphMax * sizeof(double) * kPartStride * std::max(1, need)));
+  h->part_cap = 0;
+  // one set per step of a graph: all are reduced at its end.  Sixteen are 1.2% of a large
+  // FP64 state; where they are what no longer fits, graphs are shorter.
+  for (h->part_sets = kGraphMax;; h->part_sets /= 4) {
+    const cudaError_t e = cudaMalloc(&h->d_step_part, h->part_sets * sizeof(double) * kPartStride * std::max(1, need));
+    if (e == cudaSuccess) break;
+    if (e != cudaErrorMemoryAllocation || h->part_sets == 1) CK(e);
+    cudaGetLastError();
+  }
   h->part_cap = std::max(1, need);
   return CAVITY_OK;
 }
@@ -1021,7 +1029,7 @@ int run_piece(cavity *h, int q, int par) {
 int build_graphs(cavity *h, int nsteps) {
   int par = h->parity;
   for (int q = kGraphs - 1; q >= 0; --q)
-    for (; nsteps >= kGraphSteps[q]; nsteps -= kGraphSteps[q]) {
+    for (; kGraphSteps[q] <= h->part_sets && nsteps >= kGraphSteps[q]; nsteps -= kGraphSteps[q]) {
       const int rc = ensure_graph(h, q, par);
       if (rc != CAVITY_OK) return rc;
       par ^= kGraphSteps[q] & 1;
@@ -1031,7 +1039,7 @@ int build_graphs(cavity *h, int nsteps) {
 
 int run_steps(cavity *h, int nsteps) {
   for (int q = kGraphs - 1; q >= 0; --q)
-    for (; nsteps >= kGraphSteps[q]; nsteps -= kGraphSteps[q]) {
+    for (; kGraphSteps[q] <= h->part_sets && nsteps >= kGraphSteps[q]; nsteps -= kGraphSteps[q]) {
       const int rc = run_piece(h, q, h->parity);
       if (rc != CAVITY_OK) return rc;
       h->parity ^= kGraphSteps[q] & 1;
