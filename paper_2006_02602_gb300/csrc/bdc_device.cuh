@@ -1384,6 +1384,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, const __grid
   __shared__ double shc[8];
   __shared__ double snu[NT / 32];
   __shared__ double st_t[kGraphMax];
+  __shared__ double one[8];
   __shared__ bool am_last;
   static_assert(kFinSlices * 8 <= NT && kFinSlices == 16, "one slice total per thread, 16 threads a field");
   static_assert(kBcThreads == NT, "a wall position per thread");
@@ -1433,6 +1434,17 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, const __grid
     const BlockDev &B = a.blocks[C.centre_blk[tid]];
     cp = load_p<S>((const S *)B.base[a.parity], B.fstride, C.centre_off[tid]);
   }
+  // (and, where there is one step alone, the state it advances, which only that CTA writes)
+  double t0 = 0.0, dt0 = 0.0, nu_sum0 = 0.0;
+  long long step0 = 0;
+  int flags0 = 0;
+  if (M == 1 && tid == 0) {
+    t0 = st.t;
+    dt0 = st.dt0;
+    nu_sum0 = st.nu_sum;
+    step0 = st.step;
+    flags0 = st.flags;
+  }
   double *mid = a.mid + ((long long)m * a.ncav + cav) * kFinSlices * 8;
   // the step's wall CTAs in this launch
   const int nwall = !a.wall_ctas ? 0 : a.nu_only ? C.nu_end - C.nu_begin : C.bc_end - C.bc_begin;
@@ -1470,28 +1482,53 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, const __grid
   StepResult &out = a.rec[(long long)m * a.ncav + cav];
   const bool nonfin = s == 0 && f < 6 && (f == 5 || a.mode != 1) && !isfinite(t);
   if (s == 0) {
-    if (f < 5) out.res[f] = sqrt(t * C.inv_nint);
-    if (f == 5) {
-      out.dt = C.cfl / t;
-      if (last_step) {  // the next step starts from this state
-        for (int q = 0; q < kStepSlots; ++q) {
-          st.smax[q] = 0.0;
-          st.sfl[q] = 0u;
-          if (cav == 0) a.tile_counter[q] = 0u;
-        }
+    if (f >= 6 && a.mode == 4) t *= C.wscale[f - 6];  // sums of 3 T_w - 4 T_1 + T_2 -> wall fluxes
+    const double v = f < 5 ? sqrt(t * C.inv_nint) : f == 5 ? C.cfl / t : t * C.inv_nwall;
+    if (M == 1) one[f] = v;
+    else if (f < 5) out.res[f] = v;
+    else if (f == 5) out.dt = v;
+    else out.nu[f - 6] = v;
+    if (f == 5 && last_step) {  // the next step starts from this state
+      for (int q = 0; q < kStepSlots; ++q) {
+        st.smax[q] = 0.0;
+        st.sfl[q] = 0u;
+        if (cav == 0) a.tile_counter[q] = 0u;
       }
-    }
-    if (f >= 6) {
-      if (a.mode == 4) t *= C.wscale[f - 6];  // sums of 3 T_w - 4 T_1 + T_2 -> wall fluxes
-      out.nu[f - 6] = t * C.inv_nwall;
     }
   }
   if (tid == 1 && last_step && a.mode != 1) {  // the pending shift of the final state
     st.c = centre_mean(C.ncentre, shc);
   }
   const int bad = __syncthreads_or(nonfin);
+  if (M == 1) {
+    // one step: nothing to go through, and no round trips through a.rec.  Calls of one
+    // step took 1-2 us more by the way below: FP32-mixed 128^3 65.5 us (63.9 now), in 2x2x2
+    // blocks 65.2 (64.0), FP64 275.5 (274.2)
+    const bool step = a.mode != 1;  // (mode 1: no step was taken)
+    if (tid < 5 && step) st.res[tid] = one[tid];
+    if (tid == 5) st.dt = st.dt0 = one[5];
+    if (tid == 6) st.nu_hot = one[6];
+    if (tid == 7) st.nu_cold = one[7];
+    if (tid != 0) return;
+    if (bad) atomicOr(&st.flags, 1);
+    if (!step) return;
+    st.t = t0 + dt0;
+    st.step = step0 + 1;
+    st.nu_sum = nu_sum0 + one[6];
+    if (a.log) {
+      StepRecord &o = a.log[(step0 % a.log_cap) * a.ncav + cav];
+      o.step = step0 + 1;
+      o.t = t0 + dt0;
+      o.dt = one[5];
+      for (int q = 0; q < 5; ++q) o.res[q] = one[q];
+      o.nu_hot = one[6];
+      o.nu_cold = one[7];
+      o.flags = flags0 | (bad ? 1 : 0);
+    }
+    return;
+  }
   if (tid == 0) out.bad = bad;
-  if (M > 1) {
+  {
     // the cavity's last step to get here goes through all of them
     __threadfence();
     __syncthreads();
@@ -1503,24 +1540,13 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, const __grid
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-  } else {
-    __syncthreads();
-  }
-  if (a.mode == 1) {  // no step was taken
-    if (tid == 0) {
-      st.dt = st.dt0 = out.dt;
-      st.nu_hot = out.nu[0];
-      st.nu_cold = out.nu[1];
-      if (out.bad) atomicOr(&st.flags, 1);
-    }
-    return;
   }
   const StepResult *r = a.rec + cav;  // step q at r[q * ncav]
   // the time after each step: the dt of a step is the one before it left
   if (tid < M) sv[tid] = tid == 0 ? st.dt0 : __ldcg(&r[(long long)(tid - 1) * a.ncav].dt);
   const unsigned badm = __ballot_sync(0xffffffffu, tid < M && __ldcg(&r[(long long)tid * a.ncav].bad));
-  const long long step0 = st.step;
-  const int flags0 = st.flags;
+  step0 = st.step;
+  flags0 = st.flags;
   __syncthreads();
   if (tid == 0) {
     double tt = st.t;
