@@ -1,8 +1,9 @@
 // Device-side data structures and kernels of the buoyancy-driven-cavity step
 // (Xue & Roy, arXiv 2006.02602).  Shared by the C-ABI translation unit only.
 //
-// Per step, on the handle's stream (CUDA graphs of 1, 2, 4 and 16 steps per
-// buffer parity, each kernel a programmatic dependent of the one before):
+// Per step, on the handle's stream (sequences of 1, 2, 4 and 16 steps per
+// buffer parity, launched or as CUDA graphs, each kernel a programmatic dependent
+// of the one before):
 //   k_step      fused residual (Eqs. 1-3) + explicit Euler update of every
 //               interior node of every block, walls (Section 2) formed where
 //               they are read; FP64 residual sums as per-CTA partials, the
@@ -12,10 +13,11 @@
 //               shift, and with cut faces the ghost layers of the new state
 //               from the neighbours' layers (Section 4.5, Listings 1-2, V3: p
 //               at depth 2, u, v, w, T at depth 1);
-//   k_finalize  once a graph, for all of its steps (the last one's exchange and
+//   k_finalize  once a sequence, for all of its steps (the last one's exchange and
 //               stored walls in the same launch): the partials reduced in a
-//               fixed order: residual norms, Nusselt numbers, time, step log,
-//               non-finite flag.
+//               fixed order: residual norms, Nusselt numbers, time, non-finite
+//               flag, the step log's last two records;
+//   k_step_record  with a step log, beside the steps after it: a step's record.
 // On a state refresh: k_bc (walls stored), k_pack / k_unpack.
 //
 // Storage: each block holds two buffer sets (ping-pong); a set is NF
@@ -332,8 +334,10 @@ __device__ __forceinline__ double max_nonneg(double a, double b) {
 //    a_d = V_d / (2 h_d); u, v, w share one set of weights (k = nu), T has its
 //    own (k = alpha): seven FMAs per field instead of sixteen operations;
 //  - the dissipation, the advection weights, the square roots and the whole of
-//    T's transport in 64-bit integers: 43 FP64 operations a node of 95 are left,
-//    beside about 1000 integer ones in issue slots the FP64 pipe leaves empty.
+//    T's transport in 64-bit integers: 41 FP64 operations a node are left here and
+//    11 in the update and the residual sums; the kernel executes 58 (95 before) of
+//    its 1911 instructions a node on the FP64 pipe, the others in issue slots that
+//    it leaves empty (ncu, 128^3 in 2x2x2 blocks).
 //    256^3 2445 -> 1825 us a step, 128^3 in 2x2x2 blocks 341 -> 260, 64^3 58 -> 45.6.
 //    About here the two pipes balance: u, v and w in integers too make it slower
 //    (256^3 2256, spills), and so does an FP64 div V or T the other way (1870,
@@ -1595,9 +1599,9 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(BcArgs a, const __grid
 // tile is fetched while the current one is computed.  Partials stay indexed by
 // tile slot: the reductions do not depend on which CTA took a tile.
 //
-// Three CTAs of 128 an SM (168 registers a thread): 256^3 takes 2165 us a step
-// with the 204 registers the compiler takes unasked (two CTAs), 1900 with four
-// CTAs (128 registers, spills).
+// Three CTAs of 128 an SM (168 registers a thread; the form that reads stored walls
+// spills 8 bytes): 256^3 takes 2165 us a step with the 204 registers the compiler
+// takes unasked (two CTAs), 1900 with four CTAs (128 registers, spills).
 template <int NT, bool FORM>
 __global__ void __launch_bounds__(NT, NT == 128 ? 3 : 1) k_step_f64(StepArgs a, const __grid_constant__ BcArgs d) {
   chain_wait();

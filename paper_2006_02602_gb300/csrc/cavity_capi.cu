@@ -1,7 +1,7 @@
 // C ABI of the buoyancy-driven-cavity step (include/cavity.h): host runtime
 // that lays out the blocks of one or many cavities in HBM, builds the work
-// lists of the kernels in bdc_device.cuh / bdc_step_f32.cuh, captures one CUDA
-// graph per buffer parity and replays it.  Two arithmetic forms share the
+// lists of the kernels in bdc_device.cuh / bdc_step_f32.cuh, launches them and
+// captures CUDA graphs of them to replay.  Two arithmetic forms share the
 // runtime: FP64 (five FP64 arrays per buffer set) and FP32-mixed (p_hi, p_lo,
 // u, v, w, T in FP32, read by the step kernel through TMA tensor maps).  A
 // handle holds either one cavity split into blocks (Section 3.2
@@ -107,9 +107,9 @@ struct AdjointStore {
 };
 constexpr int kAdjParts = 2 * 152;  // argmax partials of a state
 
-// Steps of one graph: a graph ends with one finalise launch for all of its
-// steps, so a long run is mostly 16-step graphs (2 for calls of two or three steps:
-// FP64 32^3 in calls of two 17.4 us a step, 24.6 as two graphs of one).
+// Steps of one graph (or sequence of launches): it ends with one finalise launch for
+// all of its steps, so a long run is mostly 16-step graphs (2 for calls of two or three
+// steps: FP64 32^3 in calls of two 17.4 us a step, 24.6 as two graphs of one).
 constexpr int kGraphs = 4;
 constexpr int kGraphSteps[kGraphs] = {1, 2, 4, kGraphMax};
 
@@ -873,10 +873,8 @@ int launch_exchange(cavity *h, int parity) {
   return CAVITY_OK;
 }
 
-// The overlapped step (FP64, cut faces): shell nodes first, then the
-// exchange of the new ghost layers on the side stream while the persistent
-// kernel steps the remaining nodes; walls and the finalise after both.
-// second stream and the fork/join events of the step graphs (created once)
+// second stream and the fork/join events (created once): of the overlapped step, of the
+// step log's records
 cudaError_t ensure_side(cavity *h) {
   cudaError_t e = cudaSuccess;
   if (!h->side) e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
@@ -885,6 +883,9 @@ cudaError_t ensure_side(cavity *h) {
   return e;
 }
 
+// The overlapped step (FP64, cut faces): shell nodes first, then the
+// exchange of the new ghost layers on the side stream while the persistent
+// kernel steps the remaining nodes; walls and the finalise after both.
 int launch_step_overlapped(cavity *h, int parity) {
   const ShellArgs sa{h->d_blocks, h->d_shell, (int)h->hshell.size(), h->d_cc, h->d_cs, h->d_step_part,
                      (long long)h->n_step, parity, h->local_dt};
