@@ -1199,8 +1199,7 @@ int adj_tiling(cavity *h, int *kc, int *ctas) {
 
 // Per segment slot: its block descriptor (slot s read, slot s + 1 written), its
 // wall faces (one walls launch covers the segment) and, in the FP32 form, its
-// tensor maps; made again when the tiling has changed.  The constant walls
-// (u = v = w = 0, the isothermal T) go into every slot.
+// tensor maps; made again when the tiling has changed.
 int adj_tables(cavity *h) {
   AdjointStore &A = h->adj;
   const int ckpt = A.ckpt;
@@ -1230,6 +1229,14 @@ int adj_tables(cavity *h) {
     CK(cudaStreamSynchronize(h->stream));  // the host vectors end here
     A.layout = h->layout;
   }
+  return CAVITY_OK;
+}
+
+// The constant walls (u = v = w = 0, the isothermal T) in every slot: the forward run's,
+// which the reverse sweep recomputes with whatever the handle has been given since.
+int adj_walls(cavity *h) {
+  AdjointStore &A = h->adj;
+  const int ckpt = A.ckpt;
   BcArgs ba = bc_args(h, 0, 5);
   ba.blocks = A.seg_blocks;
   ba.faces = A.seg_faces;
@@ -1846,6 +1853,7 @@ int cavity_adjoint_forward(cavity_t *h, int nsteps, int ckpt, double *J) {
   }
   A.have_forward = false;
   int rc = adj_tables(h);
+  if (rc == CAVITY_OK) rc = adj_walls(h);
   if (rc != CAVITY_OK) return rc;
   A.nsteps = nsteps;
   A.run_ckpt = ckpt;
