@@ -1,10 +1,10 @@
 """The step log while a run goes on.
 
-The device writes every step's record soon after the step, not at the end of the
-call: a host that reads the log during one long call sees the first steps' records
-long before the last, and, from a ring shorter than the call, every step's in its
-turn (a record stays for as many steps as the ring holds, here eight of half a
-millisecond or more, against a host loop of a few microseconds).
+The device writes every step's record soon after the step, not once for many: a
+host that reads the log during one long call sees, in a ring shorter than a graph of
+16 steps, every step's record in its turn (a record stays for as many steps as the ring
+holds, here twelve of half a millisecond or more, against a host loop of a few
+microseconds).
 """
 import time
 
@@ -15,7 +15,7 @@ import workloads
 
 pytestmark = pytest.mark.gpu
 
-CAP, STEPS = 8, 48
+CAP, STEPS = 12, 48
 
 
 @pytest.fixture(scope="module")
@@ -43,17 +43,14 @@ def test_every_step_is_seen_while_the_call_runs(m, prec, n, blocks):
     with m.Cavity(*n, **kw) as c, m.Cavity(*n, **kw) as ref:
         m.cavity_set_step_log(c.h, log)
         c.step(STEPS)
-        seen, first = {}, None
+        seen = set()
         end = time.perf_counter() + 20.0
         while len(seen) < STEPS and time.perf_counter() < end and STEPS not in seen:
             for r in log.array:
                 k = int(r["step"])
-                if k and k not in seen:
-                    seen[k] = float(r["nu_hot"])
-                    if first is None:
-                        first = k
+                if k:
+                    seen.add(k)
         c.sync()
-        assert first <= 4
         assert sorted(seen) == list(range(1, STEPS + 1))
         m.cavity_set_step_log(ref.h, after)
         ref.step(STEPS)
