@@ -51,6 +51,7 @@ def test_every_step_is_seen_while_the_call_runs(m, prec, n, blocks):
                 if k:
                     seen.add(k)
         c.sync()
+        seen.update(int(k) for k in log.array["step"])  # (the last two come together)
         assert sorted(seen) == list(range(1, STEPS + 1))
         m.cavity_set_step_log(ref.h, after)
         ref.step(STEPS)
@@ -81,7 +82,9 @@ def test_every_member_of_a_batch_is_seen(m):
             for q, s in enumerate(seen):
                 s.update(int(k) for k in steps[:, q] if k)
         m.cavity_sync(h)
-        for s in seen:
+        steps = log.array["step"].reshape(CAP, len(cavs))
+        for q, s in enumerate(seen):
+            s.update(int(k) for k in steps[:, q])
             assert sorted(s) == list(range(1, STEPS + 1))
     finally:
         m.cavity_destroy(h)
