@@ -84,6 +84,7 @@ struct AdjointStore {
   int nsteps = 0, run_ckpt = 0;  // of the last forward run
   int ckpt = 0, ncp = 0;         // as allocated
   int layout = -1;             // the tiling the segment's tables were made for
+  int setup = 0;               // the parameters and wall temperatures of the last forward run
   size_t set_bytes = 0;        // one buffer set of the block
   void *mem = nullptr;         // the one allocation behind the pointers below
   char *ckpt_mem = nullptr;    // ncp buffer sets: the state at steps 0, ckpt, 2 ckpt, ...
@@ -120,6 +121,7 @@ struct cavity {
   std::vector<cudaEvent_t> adj_ev;  // two per segment: around its reverse steps' launches
   double adj_rates_ms = 0.0;        // mean duration of one in the last reverse sweep
   int layout = 0;                   // counts assign_tiles calls
+  int setup = 0;                    // counts the parameters and wall temperatures set
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   int ncav = 1;
@@ -1457,6 +1459,7 @@ int cavity_set_params(cavity_t *h, const cavity_params *p) {
   CK(cudaStreamSynchronize(h->stream));
   h->u_ref_auto = auto_uref;
   for (auto &pc : h->prms) pc = q;
+  h->setup += 1;
   int rc = upload_consts(h);
   if (rc != CAVITY_OK) return rc;
   if (h->steps_taken == 0) return init_state(h);
@@ -1473,6 +1476,7 @@ int cavity_set_wall_temperature(cavity_t *h, int wall, const double *host, size_
   CK(cudaStreamSynchronize(h->stream));
   std::copy(host, host + n, h->twall.begin() + h->hcc[0].wall_off + (wall ? nw : 0));
   h->wall_custom[wall] = 1;
+  h->setup += 1;
   int rc = upload_consts(h);
   if (rc != CAVITY_OK) return rc;
   return refresh_state(h);
@@ -1857,6 +1861,7 @@ int cavity_adjoint_forward(cavity_t *h, int nsteps, int ckpt, double *J) {
   if (rc != CAVITY_OK) return rc;
   A.nsteps = nsteps;
   A.run_ckpt = ckpt;
+  A.setup = h->setup;
   CK(cudaMemsetAsync(&h->d_cs[0].nu_sum, 0, sizeof(double), h->stream));
   for (int n = 0; n < nsteps; n += ckpt) {
     const int c = n / ckpt;
@@ -1976,6 +1981,11 @@ int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *gr
   if (grad_wall)
     CK(cudaMemcpyAsync(grad_wall, A.thetabar, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
+  // (set since: its walls and its dt by what holds now, as after the setter)
+  if (A.setup != h->setup) {
+    const int r2 = refresh_state(h);
+    if (rc == CAVITY_OK) rc = r2;
+  }
   if (rc != CAVITY_OK) return rc;
   if (grad_ra) *grad_ra = ra;
   double tot = 0.0;
