@@ -157,9 +157,9 @@ typedef struct {
  * synchronises, without a synchronising getter per step.  host must be
  * page-locked host memory (cudaHostAlloc, cudaHostRegister, a pinned torch
  * tensor) of capacity * ncav records, kept alive while attached; NULL
- * detaches.  Steps that the adjoint's reverse sweep recomputes have been logged
- * and are not logged again.  CAVITY_ERR_INVALID_ARG for capacity < 1 or memory
- * the device cannot address. */
+ * detaches.  Records of steps the adjoint's reverse sweep recomputes are
+ * written again.  CAVITY_ERR_INVALID_ARG for capacity < 1 or memory the device
+ * cannot address. */
 CAVITY_API int cavity_set_step_log(cavity_t *h, cavity_step_record *host, long long capacity);
 
 /* Page-locked, zeroed host memory for `records` step records (records >= 1),

@@ -834,11 +834,13 @@ void launch_refresh(cavity *h, int parity) {
 bool stores_walls(const cavity *h) { return !h->f32 && (!h->form_walls || h->overlap); }
 
 // The finalise of `nsteps` steps; the state in buffer set `parity` gets its
-// ghost layers and stored walls in the same launch.
-cudaError_t launch_finalize(cavity *h, int parity, int nsteps, bool pdl) {
+// ghost layers and stored walls in the same launch.  (blocks: other descriptors than
+// the handle's, of an undivided cavity.)
+cudaError_t launch_finalize(cavity *h, int parity, int nsteps, bool pdl, const BlockDev *blocks = nullptr) {
   int ctas = 0;
-  const BcArgs b = fin_args(h, parity, nsteps, &ctas);
-  const FinTail t{ctas, h->n_cut, exch_args(h, parity), bc_args(h, parity, 3)};
+  BcArgs b = fin_args(h, parity, nsteps, &ctas);
+  FinTail t{ctas, h->n_cut, exch_args(h, parity), bc_args(h, parity, 3)};
+  if (blocks) b.blocks = t.walls.blocks = blocks;
   ctas += h->n_cut + (stores_walls(h) ? h->n_bc : 0);
   if (h->f32) return launch_chained(h, pdl, k_finalize<float>, ctas, dim3(kFinThreads), 0, b, t);
   return launch_chained(h, pdl, k_finalize<double>, ctas, dim3(kFinThreads), 0, b, t);
@@ -1249,12 +1251,12 @@ int adj_walls(cavity *h) {
   return CAVITY_OK;
 }
 
-// A recomputed step: slot s to slot s + 1 (nothing is finalised)
+// A recomputed step: slot s to slot s + 1 (nothing is finalised, but for a step log)
 cudaError_t launch_recompute(cavity *h, int s, bool pdl) {
   const AdjointStore &A = h->adj;
   if (!h->f32) {
     StepArgs a = step_args(h, 0, 0, 0);
-    if (self_chained(h)) chain_step(a, s);
+    if (self_chained(h) && !h->d_log) chain_step(a, s);
     a.dt_out = A.dts + s;
     a.blocks = A.seg_blocks + s;
     return launch_step_f64(h, a, BcArgs{}, pdl);
@@ -1931,8 +1933,13 @@ int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *gr
       CK(cudaMemcpyAsync(h->d_cs, A.ckpt_cs + c, sizeof(CavState), cudaMemcpyDeviceToDevice, h->stream));
       CK(cudaMemcpyAsync(A.dts, &h->d_cs->dt, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
       for (int s = 0; s + 1 < len; ++s) {
-        CK(launch_recompute(h, s, s > 0));
-        if (!self_chained(h) || s + 2 == len) CK(launch_recompute_between(h, s + 1));
+        CK(launch_recompute(h, s, s > 0 && !h->d_log));
+        if (h->d_log) {  // its record is written again: a finalise after every step
+          CK(launch_finalize(h, 0, 1, true, A.seg_blocks + s + 1));
+          CK(cudaMemcpyAsync(A.dts + s + 1, &h->d_cs->dt, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
+        } else if (!self_chained(h) || s + 2 == len) {
+          CK(launch_recompute_between(h, s + 1));
+        }
       }
       // the walls (formed by the step where it reads them) of every stored state
       BcArgs ba = bc_args(h, 0, 3);
