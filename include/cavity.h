@@ -302,7 +302,7 @@ CAVITY_API int cavity_adjoint_forward(cavity_t *h, int nsteps, int ckpt, double 
  * forward (linearised about its FP32 trajectory); the returned gradients
  * are FP64 either way.  When u_ref was left to its default it follows Ra
  * (u_ref^2 = Ra Pr) in the derivative.  The state is restored to the one
- * after the forward run. */
+ * after the forward run (its walls and dt by what has been set since). */
 CAVITY_API int cavity_adjoint_backward(cavity_t *h, double *grad_wall, size_t n, double *grad_ra);
 
 /* Measurement: mean duration in ms, from CUDA events on the handle's stream
